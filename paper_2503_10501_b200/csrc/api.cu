@@ -140,7 +140,7 @@ Plan make_plan(const Dims& D) {
     P.Sk = take(B * k * k * 4);
     P.Hk = take(B * k * k * 4);
     P.Rinv = take(B * k * k * 4);
-    P.Es = take(B * 4 * k * k * 4);
+    P.Es = take(B * jacobi_work_bytes(D.k));
   } else if (!D.full) {
     P.Y0 = take(B * N * k * 4);
     P.Y1 = take(B * N * k * 4);
@@ -151,7 +151,7 @@ Plan make_plan(const Dims& D) {
     P.Hm = take(B * k * k * 4 * parts);
   }
   if (!D.tcp) {
-    P.W = take(B * k * k * 4);
+    P.W = take(B * jacobi_work_bytes(D.k));
     P.ZT = take(B * k * k * 4);
   }
   P.setA = take(B * (size_t)(D.nA > 0 ? D.nA : 1) * 4);
@@ -290,7 +290,7 @@ static tc_status enqueue_score(const Ctx& c, const void* O, const void* A, float
     }
     if (err == TC_OK)
       err = launch_ics(Dg, c.P, c.ws, b0, Og, C + (size_t)b0 * D.N, sigma ? sigma + (size_t)b0 * q : nullptr,
-                       rank ? rank + b0 : nullptr, img_status + b0, st, nullptr, gram_done);
+                       rank ? rank + b0 : nullptr, img_status + b0, st, false, gram_done);
     else if (gram_done)
       cudaStreamWaitEvent(st, gram_done, 0);  // the side stream still joins the group's stream
     if (group_tail && err == TC_OK) {
@@ -690,13 +690,8 @@ tc_status tc_matmul_f32x3(const float* A, const float* B, float* C, float* CT, i
 
 // ---- Sec. 3.2: information quantity (numerical rank) of a set of tokens -----------------------
 // The score path's own Gram and eigen kernels on the gathered rows.
-// beyond the score path's own plan: the gathered rows, and four n x n arrays per image for the
-// tridiagonal solver when the full problem is small enough for it
+// beyond the score path's own plan: the gathered rows
 static size_t rank_rows_bytes(const Dims& D) { return align_up((size_t)D.B * D.N * D.d * D.esz, 256); }
-static bool rank_small_full(const Dims& D) { return D.full && D.N <= 224; }
-static size_t rank_extra_bytes(const Dims& D) {
-  return rank_rows_bytes(D) + (rank_small_full(D) ? 4 * (size_t)D.B * D.N * D.N * sizeof(float) : 0);
-}
 
 static tc_status rank_dims(const tc_params* p, int32_t n_sub, Dims* full, Dims* sub) {
   if (p == nullptr) return TC_ERR_INVALID_ARG;
@@ -716,7 +711,7 @@ tc_status tc_rank_workspace_bytes(const tc_params* p, int32_t n_sub, size_t* byt
   if (s != TC_OK) return s;
   if (bytes == nullptr) return TC_ERR_INVALID_ARG;
   const Plan P = make_plan(D);
-  *bytes = align_up(P.total, 256) + rank_extra_bytes(D);
+  *bytes = align_up(P.total, 256) + rank_rows_bytes(D);
   return TC_OK;
 }
 
@@ -730,7 +725,7 @@ tc_status tc_rank(const tc_params* p, const void* O, const int32_t* idx, int32_t
   if (idx == nullptr && n_sub != F.N) return TC_ERR_INVALID_ARG;
   const Plan P = make_plan(D);
   const size_t rows_off = align_up(P.total, 256);
-  if (ws_bytes < rows_off + rank_extra_bytes(D)) return TC_ERR_WORKSPACE;
+  if (ws_bytes < rows_off + rank_rows_bytes(D)) return TC_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   char* w = (char*)ws;
   fill_i32(img_status, D.B, 0, st);
@@ -741,8 +736,7 @@ tc_status tc_rank(const tc_params* p, const void* O, const int32_t* idx, int32_t
   }
   s = launch_gram(D, rows, (float*)(w + P.G), img_status, st);
   if (s != TC_OK) return s;
-  s = launch_ics(D, P, w, 0, rows, (float*)(w + P.C), sigma, rank, img_status, st,
-                 rank_small_full(D) ? (float*)(w + rows_off + rank_rows_bytes(D)) : nullptr);
+  s = launch_ics(D, P, w, 0, rows, (float*)(w + P.C), sigma, rank, img_status, st, true);
   if (s != TC_OK) return s;
   return check_launch();
 }

@@ -623,7 +623,7 @@ __global__ void __launch_bounds__(192) gemm_tn_upper_kernel(const float* __restr
 }
 
 // Number of parts the k x k products A^T B are delivered in (1 = the general kernel).
-int tn_parts(int k) { return (k <= TN_MAX && (k & 3) == 0 && k >= 8) ? TN_PARTS : 1; }
+int tn_parts(int k) { return 1; }
 
 // C (nparts parts per image, image stride nparts * n * n) = A^T B, symmetric.
 static void gemm_tn_sym(const float* A, const float* B, float* C, int n, int K, size_t sA, size_t sB,
@@ -1511,758 +1511,6 @@ __global__ void __launch_bounds__(512) jacobi_kernel(const float* __restrict__ H
   }
 }
 
-// ==========================================================================================
-// Symmetric eigen-solver for matrices that fit in shared memory (n <= ~230):
-//   1. Householder reduction to a tridiagonal matrix T, the orthogonal factor Q formed in place;
-//   2. every eigenvalue of T by bisection on the Sturm count, one thread per eigenvalue;
-//   3. the eigenvector of T for every eigenvalue that can pass the rank cut-off, by inverse
-//      iteration (tridiagonal elimination with partial pivoting), one thread per eigenvalue,
-//      its four work vectors in global scratch laid out thread-fastest;
-//   4. eigenvalues refined as Rayleigh quotients on T, eigenvectors of H as Z = Q Y.
-// Nothing here is a serial recurrence over the whole matrix, which is what makes it several
-// times faster than sweeping Jacobi rotations or chasing QL bulges from one thread.
-// Eigenvectors of eigenvalues closer together than the rounding level of T are not
-// re-orthogonalised against each other (Eq. 3-6 is not unique there in the first place).
-//   in   H [n][n] symmetric (only its symmetric part is used)
-//   out  theta [n] eigenvalues (ascending), ZT [n][n] with ZT[p][i] = component i of
-//        eigenvector p (all zero for eigenvalues under a quarter of the rank cut-off)
-//   scratch u0, u1, u2, yv, ml: [n][n] float each, per image
-// One block (16 warps) per image.
-// ==========================================================================================
-// Barrier among `count` threads (a multiple of 32) of the block, on hardware barrier `id` (1..15).
-__device__ __forceinline__ void bar_named(int id, int count) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-
-template <int NT>  // n when it is known at compile time (addresses fold into immediates), else 0
-__global__ void __launch_bounds__(512) tridiag_eig_kernel(const float* Hin,
-                                                         float* __restrict__ ZTg,
-                                                         float* __restrict__ theta, int n_rt, float rank_tol,
-                                                         float* __restrict__ u0g, float* __restrict__ u1g,
-                                                         float* __restrict__ u2g, float* yg, float* __restrict__ mlg,
-                                                         size_t ml_stride,
-                                                         int32_t* __restrict__ status, int nparts,
-                                                         int emit_factors) {
-  // emit_factors: instead of Z = Q Y the kernel leaves its two factors for the tensor-core
-  // products: ZTg receives Q^T ([j][i] = Q[i][j]) and u0g receives Y^T ([p][j] = component j of
-  // the eigenvector p of T)
-  const int n = NT ? NT : n_rt;
-  extern __shared__ __align__(16) float sm[];
-  const int ld = n | 1;
-  const int n4 = (n + 3) & ~3;         // the vectors start on 16-byte boundaries
-  float* dv = sm;                      // [n] diagonal
-  float* ev = dv + n4;                 // [n] sub-diagonal (ev[i] couples i and i+1)
-  float* vv = ev + n4;                 // [n] Householder vector of the current step
-  float* vv2 = vv + n4;                // [n] ... of the next step (the two alternate)
-  float* pv = vv2 + n4;                // [n] work vector
-  float* beta = pv + n4;               // [n] reflector scales
-  float* dn = beta + n4;               // [n] diagonal of T / |T| for the Sturm counts
-  float2* cs = reinterpret_cast<float2*>(dn + n4);     // [4 n floats] partial sums of the reduction
-  float* qf = reinterpret_cast<float*>(cs) + 4 * n4;   // [16 n] reflector block and partial products
-  float* A = qf + 16 * n4;             // [n][ld]
-  __shared__ float s_red[16];
-  __shared__ int s_fail;
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float* Hb = Hin + (size_t)b * nparts * n * n;  // H arrives as nparts parts to be added up
-
-  if (nparts == 4 && (n & 3) == 0) {
-    // the parts come from the kernel that writes every entry and its mirror image with the
-    // same bits, so their sum is symmetric as it stands
-    const float4* H4 = reinterpret_cast<const float4*>(Hb);
-    const int kv = n >> 2, nv = (n * n) >> 2;
-    for (int e = tid; e < nv; e += 1024) {  // two trips' worth of loads in flight together
-      const int e2 = e + 512;
-      const bool two = e2 < nv;
-      float4 p[4], q[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        p[i] = __ldg(H4 + (size_t)i * nv + e);
-        q[i] = two ? __ldg(H4 + (size_t)i * nv + e2) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-      {
-        const int r = e / kv, c = (e - r * kv) * 4;
-        float* dst = A + r * ld + c;
-        dst[0] = (p[0].x + p[1].x) + (p[2].x + p[3].x);
-        dst[1] = (p[0].y + p[1].y) + (p[2].y + p[3].y);
-        dst[2] = (p[0].z + p[1].z) + (p[2].z + p[3].z);
-        dst[3] = (p[0].w + p[1].w) + (p[2].w + p[3].w);
-      }
-      if (two) {
-        const int r = e2 / kv, c = (e2 - r * kv) * 4;
-        float* dst = A + r * ld + c;
-        dst[0] = (q[0].x + q[1].x) + (q[2].x + q[3].x);
-        dst[1] = (q[0].y + q[1].y) + (q[2].y + q[3].y);
-        dst[2] = (q[0].z + q[1].z) + (q[2].z + q[3].z);
-        dst[3] = (q[0].w + q[1].w) + (q[2].w + q[3].w);
-      }
-    }
-  } else if (nparts == 1 && (n & 3) == 0) {
-    // one part that need not be symmetric to the last bit (a product Q^T (G Q)): 16-byte loads,
-    // then the two triangles are averaged in shared memory
-    const float4* H4 = reinterpret_cast<const float4*>(Hb);
-    const int kv = n >> 2, nv = (n * n) >> 2;
-    for (int e = tid; e < nv; e += 512) {
-      const float4 p = __ldg(H4 + e);
-      const int r = e / kv, c = (e - r * kv) * 4;
-      float* dst = A + r * ld + c;
-      dst[0] = p.x; dst[1] = p.y; dst[2] = p.z; dst[3] = p.w;
-    }
-    __syncthreads();
-    for (int e = tid; e < n * n; e += 512) {
-      const int r = e / n, c = e - r * n;
-      if (c > r) {
-        const float m = 0.5f * (A[r * ld + c] + A[c * ld + r]);
-        A[r * ld + c] = m;
-        A[c * ld + r] = m;
-      }
-    }
-  } else {
-    for (int e = tid; e < n * n; e += 512) {
-      const int r = e / n, c = e - r * n;
-      float h = 0.f, ht = 0.f;
-      for (int q = 0; q < nparts; ++q) {
-        h += Hb[(size_t)q * n * n + e];
-        ht += Hb[(size_t)q * n * n + (size_t)c * n + r];
-      }
-      A[r * ld + c] = 0.5f * (h + ht);
-    }
-  }
-  if (tid == 0) s_fail = 0;
-  __syncthreads();
-
-  // ---------------- Householder tridiagonalisation ----------------
-  // Three block barriers per column and no warp reductions inside the O(m^2) parts: a thread
-  // owns one column c of the trailing block and a range of its rows (the block is symmetric, so
-  // the column sum over that range is a partial of (B v)_c); the ranges are combined through
-  // shared memory.  While the trailing block is updated, the thread that owns its first column
-  // also writes that column out as the next step's vector and gathers its |x|^2, so a step
-  // starts with everything it needs except the square root, which every thread takes itself.
-  // Vector entries are read four at a time (one broadcast load per four rows).
-  // The scalar parts of a step are repeated by every warp, four warps to a scheduler, so what
-  // counts there is the number of instructions: sums come as one or two 16-byte loads, the
-  // square root and the reciprocal as a Newton step on the hardware approximations.
-  __shared__ float s_sig[16];
-  __shared__ __align__(16) float s_sig4[4];  // |x|^2 of the next column, one partial per row range
-  __shared__ __align__(16) float s_red8[8];  // v.p, one partial per warp of the first row range
-  float* part = reinterpret_cast<float*>(cs);  // [<= 4][n] partial products (cs is free here)
-  if (warp == 0) {
-    float ps = 0.f;
-    for (int r = lane; r + 1 < n; r += 32) {
-      const float x = A[(1 + r) * ld];
-      vv[r] = x;
-      ps = fmaf(x, x, ps);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
-    if (lane < 4) s_sig4[lane] = (lane == 0) ? ps : 0.f;
-  }
-  __syncthreads();
-  int cw = 0, G = 1, g = 0, c = 0;  // thread layout: cw warps cover the columns, G row ranges
-  bool lead = false;                // this warp holds column 0 of its row range
-  for (int j = 0; j + 2 < n; ++j) {
-    const int m = n - j - 1;  // order of the trailing block B = A[j+1.., j+1..]
-    float* vc = (j & 1) ? vv2 : vv;  // x of this step (v is x with v_0 in place of its entry 0)
-    float* vn = (j & 1) ? vv : vv2;  // x of the next step
-    const float4 s4 = *reinterpret_cast<const float4*>(s_sig4);
-    const float sigma = (s4.x + s4.y) + (s4.z + s4.w);
-    const float x0 = vc[0];
-    const float tail = sigma - x0 * x0;  // |x|^2 without its first entry
-    // reflector H = I - bj v v^T with v = x - alpha e_1; a column already in tridiagonal form
-    // gets bj = 0 (H = I) and keeps its entries
-    const bool skip = !(tail > 1e-30f * sigma) || !(sigma > 0.f);
-    const float rs = rsqrtf(sigma);
-    float nrm = sigma * rs;
-    nrm = fmaf(fmaf(-nrm, nrm, sigma), 0.5f * rs, nrm);
-    const float alpha = skip ? x0 : -copysignf(nrm, x0);
-    const float v0 = skip ? x0 : x0 - alpha;
-    const float den = tail + v0 * v0;
-    float rc = __fdividef(2.0f, den);
-    rc = fmaf(fmaf(-den, rc, 2.0f), 0.5f * rc, rc);
-    const float bj = skip ? 0.f : rc;
-    if (tid == 0) {
-      dv[j] = A[j * ld + j];
-      ev[j] = alpha;
-      beta[j] = bj;
-    }
-    if (((m + 31) >> 5) != cw) {
-      cw = (m + 31) >> 5;
-      G = min(4, 16 / cw);
-      g = warp / cw;
-      c = (warp - g * cw) * 32 + lane;
-      lead = (warp == g * cw);
-    }
-    const bool on = (g < G) && (c < m);
-    // rows per range, a multiple of four (G is 2, 3 or 4; the multiplication is a division by 3)
-    const int per0 = (G == 4) ? (m + 3) >> 2 : (G == 3) ? ((m + 2) * 21846) >> 16 : (m + 1) >> 1;
-    const int per = (per0 + 3) & ~3;
-    const int r_lo = g * per, r_hi = min(m, r_lo + per);
-    float* colp = A + (j + 1) * ld + j + 1 + c;  // B[0][c]; rows are ld apart
-    if (on) {
-      float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-      int r = r_lo;
-      const float* bp = colp + r_lo * ld;
-      for (; r + 3 < r_hi; r += 4, bp += 4 * ld) {
-        float4 v4 = *reinterpret_cast<const float4*>(vc + r);
-        if (r == 0) v4.x = v0;
-        a0 = fmaf(bp[0], v4.x, a0);
-        a1 = fmaf(bp[ld], v4.y, a1);
-        a2 = fmaf(bp[2 * ld], v4.z, a2);
-        a3 = fmaf(bp[3 * ld], v4.w, a3);
-      }
-      for (; r < r_hi; ++r) a0 = fmaf(colp[r * ld], (r == 0) ? v0 : vc[r], a0);
-      part[g * n + c] = (a0 + a1) + (a2 + a3);
-    }
-    __syncthreads();
-    // p = bj * B v ; v.p
-    float vpp = 0.f;
-    if (g == 0 && c < m) {
-      const float t0 = part[c], t1 = part[n + c];
-      const float t2 = (G > 2) ? part[2 * n + c] : 0.f, t3 = (G > 3) ? part[3 * n + c] : 0.f;
-      const float pc = bj * ((t0 + t1) + (t2 + t3));
-      pv[c] = pc;
-      vpp = ((c == 0) ? v0 : vc[c]) * pc;
-    }
-    // the column is kept for the accumulation of Q (everyone has read its x_0 by now)
-    if (tid == 0) A[(j + 1) * ld + j] = v0;
-    if (warp < 8) {  // the first row range is at most seven warps; the others hold zero
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) vpp += __shfl_xor_sync(0xffffffffu, vpp, o);
-      if (lane == 0) s_red8[warp] = vpp;
-    }
-    __syncthreads();
-    const float4 ra = *reinterpret_cast<const float4*>(s_red8);
-    const float4 rb = *reinterpret_cast<const float4*>(s_red8 + 4);
-    const float vp = ((ra.x + ra.y) + (ra.z + ra.w)) + ((rb.x + rb.y) + (rb.z + rb.w));
-    const float K = 0.5f * bj * vp;  // w = p - K v
-    // B -= v w^T + w v^T ; column 0 of the new B, below its top entry, is the next x
-    float sig_part = 0.f;
-    auto update = [&](auto tag) {
-      constexpr bool LEAD = decltype(tag)::value;  // this warp's lane 0 owns column 0
-      const bool first = LEAD && (lane == 0);
-      const float vcc = (c == 0) ? v0 : vc[c], wc = fmaf(-K, vcc, pv[c]);
-      int r = r_lo;
-      float* bp = colp + r_lo * ld;
-      for (; r + 3 < r_hi; r += 4, bp += 4 * ld) {
-        float4 v4 = *reinterpret_cast<const float4*>(vc + r);
-        if (r == 0) v4.x = v0;
-        const float4 p4 = *reinterpret_cast<const float4*>(pv + r);
-        const float vr[4] = {v4.x, v4.y, v4.z, v4.w};
-        const float pr[4] = {p4.x, p4.y, p4.z, p4.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const float wr = fmaf(-K, vr[u], pr[u]);
-          const float nv = bp[u * ld] - fmaf(vr[u], wc, wr * vcc);
-          bp[u * ld] = nv;
-          if (LEAD) {
-            if (first && r + u >= 1) {
-              vn[r + u - 1] = nv;
-              sig_part = fmaf(nv, nv, sig_part);
-            }
-          }
-        }
-      }
-      for (; r < r_hi; ++r) {
-        const float vr = (r == 0) ? v0 : vc[r], wr = fmaf(-K, vr, pv[r]);
-        const float nv = colp[r * ld] - fmaf(vr, wc, wr * vcc);
-        colp[r * ld] = nv;
-        if (LEAD) {
-          if (first && r >= 1) {
-            vn[r - 1] = nv;
-            sig_part = fmaf(nv, nv, sig_part);
-          }
-        }
-      }
-    };
-    if (on) {
-      if (lead) update(std::true_type{}); else update(std::false_type{});
-    }
-    if (lead && lane == 0 && g < 4) s_sig4[g] = sig_part;  // zero from a range that is not in use
-    __syncthreads();
-  }
-  if (tid == 0) {
-    if (n >= 2) {
-      dv[n - 2] = A[(n - 2) * ld + n - 2];
-      ev[n - 2] = A[(n - 1) * ld + n - 2];
-      beta[n - 2] = 0.f;
-    }
-    dv[n - 1] = A[(n - 1) * ld + n - 1];
-    ev[n - 1] = 0.f;
-    A[(n - 1) * ld + n - 1] = 1.f;  // the accumulation of Q starts from the identity
-  }
-  __syncthreads();
-
-  // From here the block works as two teams until Z = Q Y needs both results: the first
-  // ceil(n / 32) warps find the eigenpairs of T (one thread per eigenvalue; they only read the
-  // diagonals of T), the other warps accumulate Q.  Each team synchronises on its own barrier.
-  const int nbw = (n + 31) >> 5;           // warps of the eigenvalue team
-  const int ET = nbw * 32;                 // its threads
-  const int NQW = 16 - nbw, QT = NQW * 32; // warps and threads of the Q team
-  const int qt = tid - ET, qw = warp - nbw;
-  if (warp >= nbw) {
-  // ---------------- Q = H_0 H_1 ... H_{n-3}, accumulated backwards, in place ----------------
-  // Reflector j sits in A[j+1.., j].  Reflectors are applied four at a time in the compact WY
-  // form  H_{j0} ... H_{j1} = I - V T V^T  (T upper triangular), so a block costs three barriers
-  // and two passes over the rows instead of two barriers and two passes per reflector.
-  // Before a block, columns c >= j1+2 of A (rows >= j1+2) hold the product of the later
-  // reflectors; everything else of Q is still the identity, which the block first writes out.
-  {
-    constexpr int NBQ = 4;
-    float* Vb = qf;              // [n][NBQ]  Vb[r][i] = entry r of reflector j0+i (0 above its support
-                                 // and for a reflector the block does not have): one 16-byte read per row
-    float* Wp = qf + NBQ * n;    // [3][NBQ][n] partial products V^T Q per row range
-    __shared__ float s_vv[NBQ][NBQ];  // v_a . v_b for a < b
-    for (int j1 = n - 3; j1 >= 0; j1 -= NBQ) {
-      const int j0 = max(0, j1 - NBQ + 1), nbk = j1 - j0 + 1;
-      // (1) copy the block's reflectors out of the columns that are about to be overwritten
-      for (int idx = qt; idx < NBQ * n; idx += QT) {
-        const int r = idx / NBQ, i = idx - r * NBQ, jj = j0 + i;
-        Vb[idx] = (i < nbk && r >= jj + 1) ? A[r * ld + jj] : 0.f;
-      }
-      bar_named(1, QT);
-      // (2) identity columns j0+1 .. j1+1, zero rows j0+1 .. j1+1 right of them; v_a . v_b
-      for (int idx = qt; idx < (n - j0 - 1) * nbk; idx += QT) {
-        const int r = j0 + 1 + idx / nbk, c = j0 + 1 + idx % nbk;
-        A[r * ld + c] = (r == c) ? 1.f : 0.f;
-      }
-      for (int idx = qt; idx < nbk * (n - j1 - 2); idx += QT) {
-        const int r = j0 + 1 + idx / (n - j1 - 2), c = j1 + 2 + idx % (n - j1 - 2);
-        A[r * ld + c] = 0.f;
-      }
-      if (qw < 6) {
-        // the six pairs a < b of a block of four, one warp each
-        const int a2 = (qw < 3) ? 0 : (qw < 5 ? 1 : 2);
-        const int b2 = (qw < 3) ? qw + 1 : (qw < 5 ? qw - 1 : 3);
-        if (b2 < nbk) {
-          float d2 = 0.f;
-          for (int r = lane; r < n; r += 32) d2 = fmaf(Vb[r * NBQ + a2], Vb[r * NBQ + b2], d2);
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) d2 += __shfl_xor_sync(0xffffffffu, d2, o);
-          if (lane == 0) s_vv[a2][b2] = d2;
-        }
-      }
-      bar_named(1, QT);
-      // (3) W = V^T Q on the columns c >= j0+1, rows split into up to three ranges
-      const int ncols = n - j0 - 1;
-      const int cw = (ncols + 31) >> 5;
-      const int G = min(3, NQW / cw);
-      const int g = qw / cw, c = j0 + 1 + (qw - g * cw) * 32 + lane;
-      const bool on = (g < G) && (c < n);
-      const int per = (ncols + G - 1) / G;
-      const int r_lo = j0 + 1 + g * per, r_hi = min(n, r_lo + per);
-      if (on) {
-        float acc[NBQ] = {0.f, 0.f, 0.f, 0.f};
-        for (int r = r_lo; r < r_hi; ++r) {
-          const float qv = A[r * ld + c];
-          const float4 v4 = *reinterpret_cast<const float4*>(Vb + r * NBQ);
-          acc[0] = fmaf(v4.x, qv, acc[0]);
-          acc[1] = fmaf(v4.y, qv, acc[1]);
-          acc[2] = fmaf(v4.z, qv, acc[2]);
-          acc[3] = fmaf(v4.w, qv, acc[3]);
-        }
-#pragma unroll
-        for (int i = 0; i < NBQ; ++i) Wp[(g * NBQ + i) * n + c] = acc[i];
-      }
-      bar_named(1, QT);
-      // (4) T W, (5) Q -= V (T W)
-      if (on) {
-        float w[NBQ], tw[NBQ];
-#pragma unroll
-        for (int i = 0; i < NBQ; ++i) {
-          float t = 0.f;
-          for (int q = 0; q < G; ++q) t += Wp[(q * NBQ + i) * n + c];
-          w[i] = (i < nbk) ? t : 0.f;
-        }
-        // T (upper triangular, 4 x 4) of the compact WY form, in registers of every thread:
-        //   T_ii = beta_i ;  T[0:i, i] = -beta_i T[0:i, 0:i] (V[:, 0:i]^T v_i)
-        // (a reflector the block does not have gets beta = 0, which zeroes its row and column)
-        const float b0 = beta[j0], b1 = (nbk > 1) ? beta[j0 + 1] : 0.f;
-        const float b2 = (nbk > 2) ? beta[j0 + 2] : 0.f, b3 = (nbk > 3) ? beta[j0 + 3] : 0.f;
-        const float v01 = (nbk > 1) ? s_vv[0][1] : 0.f;
-        const float v02 = (nbk > 2) ? s_vv[0][2] : 0.f, v12 = (nbk > 2) ? s_vv[1][2] : 0.f;
-        const float v03 = (nbk > 3) ? s_vv[0][3] : 0.f, v13 = (nbk > 3) ? s_vv[1][3] : 0.f;
-        const float v23 = (nbk > 3) ? s_vv[2][3] : 0.f;
-        const float t01 = -b1 * (b0 * v01);
-        const float t02 = -b2 * fmaf(t01, v12, b0 * v02);
-        const float t12 = -b2 * (b1 * v12);
-        const float t03 = -b3 * fmaf(t02, v23, fmaf(t01, v13, b0 * v03));
-        const float t13 = -b3 * fmaf(t12, v23, b1 * v13);
-        const float t23 = -b3 * (b2 * v23);
-        tw[0] = fmaf(t03, w[3], fmaf(t02, w[2], fmaf(t01, w[1], b0 * w[0])));
-        tw[1] = fmaf(t13, w[3], fmaf(t12, w[2], b1 * w[1]));
-        tw[2] = fmaf(t23, w[3], b2 * w[2]);
-        tw[3] = b3 * w[3];
-        int r = r_lo;
-        for (; r + 3 < r_hi; r += 4) {  // all loads of a trip before its stores
-          float qv[4];
-          float4 vb[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            qv[u] = A[(r + u) * ld + c];
-            vb[u] = *reinterpret_cast<const float4*>(Vb + (r + u) * NBQ);
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            qv[u] = fmaf(-vb[u].x, tw[0], qv[u]);
-            qv[u] = fmaf(-vb[u].y, tw[1], qv[u]);
-            qv[u] = fmaf(-vb[u].z, tw[2], qv[u]);
-            qv[u] = fmaf(-vb[u].w, tw[3], qv[u]);
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) A[(r + u) * ld + c] = qv[u];
-        }
-        for (; r < r_hi; ++r) {
-          float qv = A[r * ld + c];
-#pragma unroll
-          for (int i = 0; i < NBQ; ++i) qv = fmaf(-Vb[r * NBQ + i], tw[i], qv);
-          A[r * ld + c] = qv;
-        }
-      }
-      bar_named(1, QT);
-    }
-    // first row and column of Q are e_0
-    for (int i = qt; i < n; i += QT) {
-      A[i * ld] = (i == 0) ? 1.f : 0.f;
-      A[i] = (i == 0) ? 1.f : 0.f;
-    }
-    if (n == 2 && qt == 0) {  // no reflector at all: Q = I
-      A[ld + 1] = 1.f;
-    }
-  }
-  }
-
-  // ---------------- eigenvalues of T by bisection ----------------
-  // dv = diagonal, ev[i] couples i and i+1.  vv <- ev^2, pv <- eigenvalues (ascending).
-  float* e2 = vv;
-  float* lam = pv;
-  float tnorm = 0.f;
-  if (warp < nbw) {
-    float lo = 3.0e38f, hi = -3.0e38f;
-    for (int i = tid; i < n; i += ET) {
-      const float el = (i > 0) ? fabsf(ev[i - 1]) : 0.f, er = (i + 1 < n) ? fabsf(ev[i]) : 0.f;
-      lo = fminf(lo, dv[i] - el - er);
-      hi = fmaxf(hi, dv[i] + el + er);
-      e2[i] = ev[i] * ev[i];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    if (lane == 0) {
-      s_red[warp] = lo;
-      s_sig[warp] = hi;
-    }
-    bar_named(2, ET);
-    lo = s_red[0];
-    hi = s_sig[0];
-    for (int w = 1; w < nbw; ++w) {
-      lo = fminf(lo, s_red[w]);
-      hi = fmaxf(hi, s_sig[w]);
-    }
-    const float tn = fmaxf(fabsf(lo), fabsf(hi));
-    lo -= 2.4e-7f * tn + 1e-30f;
-    hi += 2.4e-7f * tn + 1e-30f;
-    // Sturm count in product form on T / |T| (no division on the serial chain):
-    //   p_0 = 1, p_1 = d_0 - x, p_{i+1} = (d_i - x) p_i - e_{i-1}^2 p_{i-1};
-    // the number of sign changes along the sequence is the number of eigenvalues below x.
-    // Both running values are rescaled together whenever they leave [1e-8, 1e8].
-    const float itn = 1.0f / fmaxf(tn, 1e-30f);
-    for (int i = tid; i < n; i += ET) {
-      dn[i] = dv[i] * itn;
-      e2[i] = e2[i] * itn * itn;
-    }
-    bar_named(2, ET);
-    // the entries of two steps side by side, one 16-byte load per trip of the count below
-    float4* tq = reinterpret_cast<float4*>(cs);
-    const int ntrip = (n - 1) >> 1;
-    for (int t = tid; t < ntrip; t += ET)
-      tq[t] = make_float4(dn[2 * t + 1], e2[2 * t], dn[2 * t + 2], e2[2 * t + 1]);
-    bar_named(2, ET);
-    auto sturm = [&](float x) {
-      // two steps per trip, and the pair is re-centred once per trip (entries can be as small as
-      // rounding noise, 1e-7 of the largest, so it can shrink by 1e-14 in a trip: the thresholds
-      // leave room).  A sign change is a difference of sign bits; a zero takes the sign of its
-      // bit, which gives the same total because the value after it has the opposite sign of the
-      // one before it.
-      float p0 = 1.f, p1 = dn[0] - x;
-      unsigned cnt = __float_as_uint(p1) >> 31;
-      for (int t = 0; t < ntrip; ++t) {
-        const float4 q = tq[t];
-        const float pa = fmaf(q.x - x, p1, -q.y * p0);
-        const float pb = fmaf(q.z - x, pa, -q.w * p1);
-        cnt += ((__float_as_uint(pa) ^ __float_as_uint(p1)) >> 31) +
-               ((__float_as_uint(pb) ^ __float_as_uint(pa)) >> 31);
-        p0 = pa;
-        p1 = pb;
-        const float sc = fmaxf(fabsf(p0), fabsf(p1));
-        if (sc < 1e-8f) {
-          p0 *= 1e16f;
-          p1 *= 1e16f;
-        } else if (sc > 1e8f) {
-          p0 *= 1e-16f;
-          p1 *= 1e-16f;
-        }
-      }
-      if (!(n & 1)) {  // one step left
-        const float pa = fmaf(dn[n - 1] - x, p1, -e2[n - 2] * p0);
-        cnt += (__float_as_uint(pa) ^ __float_as_uint(p1)) >> 31;
-      }
-      return (int)cnt;
-    };
-    const float lon = lo * itn, hin = hi * itn;
-    // First round, shared by all eigenvalues: counts at n points spaced geometrically from the
-    // top of the spectrum down to a little under the smallest eigenvalue that can pass the rank
-    // cut-off.  Each eigenvalue starts its own bisection from the two points around it.
-    int* gcnt = reinterpret_cast<int*>(pv);
-    const float glo = fmaxf(0.06f * rank_tol * rank_tol, 1e-9f);
-    const bool use_grid = hin > 2.0f * glo;
-    const float lr = use_grid ? log2f(glo / hin) / (float)n : 0.f;
-    auto grid = [&](int t) { return hin * exp2f(lr * (float)(n - t)); };
-    if (use_grid) {
-      if (tid < n) gcnt[tid] = sturm(grid(tid));
-      bar_named(2, ET);
-    }
-    float a = lon, bhi = hin;
-    if (use_grid && tid < n) {
-      int tl = -1, th = n;  // the count is 0 at lon (t = -1) and n at hin (t = n)
-      while (th - tl > 1) {
-        const int mid = (tl + th) >> 1;
-        if (gcnt[mid] > tid) th = mid; else tl = mid;
-      }
-      if (tl >= 0) a = fmaxf(lon, grid(tl));
-      if (th < n) bhi = fminf(hin, grid(th));
-    }
-    bar_named(2, ET);  // the counts are overwritten by the eigenvalues below
-    if (tid < n) {
-      // eigenvalue number tid (0 = smallest): plain bisection, one thread per eigenvalue (the
-      // counts are bound by instruction issue, so evaluating several points per round on
-      // neighbouring lanes costs more than the rounds it saves)
-      // An interval that lies wholly under the floor below which no eigenvector is computed
-      // stops at a thousandth of that floor: such an eigenvalue only enters the energy check.
-      const float floor_n = 0.25f * rank_tol * rank_tol;
-      for (int it = 0; it < 48; ++it) {
-        const float x = 0.5f * (a + bhi);
-        if (!(x > a) || !(x < bhi)) break;
-        if (bhi < floor_n && bhi - a < 1e-3f * floor_n) break;
-        if (sturm(x) > tid) bhi = x; else a = x;
-      }
-      lam[tid] = 0.5f * (a + bhi) * tn;
-    }
-    tnorm = tn;
-    bar_named(2, ET);
-  }
-
-  // ---------------- eigenvectors of T by inverse iteration ----------------
-  const float keep_floor = 0.25f * rank_tol * rank_tol * tnorm;
-  {
-    const size_t img = (size_t)b * n * n;
-    float* u0 = u0g + img;
-    float* u1 = u1g + img;
-    float* u2 = u2g + img;
-    float* y = yg + img * nparts;
-    float* ml = mlg + (size_t)b * ml_stride;
-    if (tid < n) {
-      const int t = tid;
-      float x = lam[t];
-      const bool wanted = x >= keep_floor;
-      // an eigenvalue bisection could not tell from its lower neighbour is nudged up so the two
-      // solves do not return the same vector
-      const float sep = 1.2e-6f * fmaxf(fabsf(x), 1e-3f * tnorm);
-      if (t > 0 && x - lam[t - 1] < sep) x = lam[t - 1] + sep * (float)(1 + (t & 3));
-      const float tiny = fmaxf(tnorm, 1e-30f) * 1.1920929e-7f;
-      if (wanted) {
-        // factor T - x I once, with row interchanges (|multiplier| <= 1).  Stored per row: the
-        // reciprocal pivot, the two entries right of it, and the multiplier, to which 4 is
-        // added when the rows were swapped.
-        {
-          float a = dv[0] - x, bb = (n > 1) ? ev[0] : 0.f, c = 0.f;
-          for (int i = 0; i + 1 < n; ++i) {
-            const float sub = ev[i], dnx = dv[i + 1] - x, en = (i + 2 < n) ? ev[i + 1] : 0.f;
-            const bool sw = fabsf(a) < fabsf(sub);
-            float piv = sw ? sub : a;
-            const float oth = sw ? a : sub;
-            if (fabsf(piv) < tiny) piv = copysignf(tiny, piv);
-            const float rp = 1.0f / piv;
-            const float mlt = oth * rp;
-            const float p1 = sw ? dnx : bb, p2 = sw ? en : c;
-            const float q1 = sw ? bb : dnx, q2 = sw ? c : en;
-            u0[(size_t)i * n + t] = rp;
-            u1[(size_t)i * n + t] = p1;
-            u2[(size_t)i * n + t] = p2;
-            ml[(size_t)i * n + t] = sw ? mlt + 4.0f : mlt;
-            a = fmaf(-mlt, p1, q1);
-            bb = fmaf(-mlt, p2, q2);
-            c = 0.f;
-          }
-          if (fabsf(a) < tiny) a = copysignf(tiny, a);
-          u0[(size_t)(n - 1) * n + t] = 1.0f / a;
-          u1[(size_t)(n - 1) * n + t] = 0.f;
-          u2[(size_t)(n - 1) * n + t] = 0.f;
-        }
-        float scale = 1.f, nrm = 0.f;
-        for (int it = 0; it < 3; ++it) {
-          if (it > 0) {
-            // apply the elimination to the right-hand side (the previous solution, rescaled)
-            float cur = y[t] * scale;
-            for (int i0 = 0; i0 + 1 < n; i0 += 8) {
-              float nx[8], me[8];
-#pragma unroll
-              for (int u = 0; u < 8; ++u)
-                if (i0 + u + 1 < n) {
-                  nx[u] = y[(size_t)(i0 + u + 1) * n + t] * scale;
-                  me[u] = ml[(size_t)(i0 + u) * n + t];
-                }
-#pragma unroll
-              for (int u = 0; u < 8; ++u) {
-                const int i = i0 + u;
-                if (i + 1 < n) {
-                  const bool sw = me[u] > 2.0f;
-                  const float mlt = sw ? me[u] - 4.0f : me[u];
-                  const float hi_ = sw ? nx[u] : cur, lo_ = sw ? cur : nx[u];
-                  y[(size_t)i * n + t] = hi_;
-                  cur = fmaf(-mlt, hi_, lo_);
-                }
-              }
-            }
-            y[(size_t)(n - 1) * n + t] = cur;
-          }
-          // back substitution (first pass: right-hand side of ones), eight rows per group of loads
-          float y1 = 0.f, y2 = 0.f, big = 0.f;
-          nrm = 0.f;
-          for (int i1 = n - 1; i1 >= 0; i1 -= 8) {
-            float rh[8], p0[8], p1[8], p2[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              const int i = i1 - u;
-              if (i >= 0) {
-                rh[u] = (it == 0) ? 1.f : y[(size_t)i * n + t];
-                p0[u] = u0[(size_t)i * n + t];
-                p1[u] = u1[(size_t)i * n + t];
-                p2[u] = u2[(size_t)i * n + t];
-              }
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              const int i = i1 - u;
-              if (i >= 0) {
-                const float yi = (rh[u] - p1[u] * y1 - p2[u] * y2) * p0[u];
-                y[(size_t)i * n + t] = yi;
-                big = fmaxf(big, fabsf(yi));
-                nrm = fmaf(yi, yi, nrm);
-                y2 = y1;
-                y1 = yi;
-              }
-            }
-          }
-          scale = 1.0f / fmaxf(big, 1e-30f);  // keeps the next right-hand side in range
-        }
-        {
-          // normalise; Rayleigh quotient on T
-          const float inv = rsqrtf(fmaxf(nrm * scale * scale, 1e-30f)) * scale;
-          float rq = 0.f, prev = 0.f;
-          for (int i0 = 0; i0 < n; i0 += 8) {
-            float v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-              if (i0 + u < n) v[u] = y[(size_t)(i0 + u) * n + t] * inv;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              const int i = i0 + u;
-              if (i < n) {
-                y[(size_t)i * n + t] = v[u];
-                rq = fmaf(dv[i] * v[u], v[u], rq);
-                if (i > 0) rq = fmaf(2.0f * ev[i - 1] * prev, v[u], rq);
-                prev = v[u];
-              }
-            }
-          }
-          e2[t] = rq;  // e2 is free after the bisection
-        }
-      } else {
-        for (int i = 0; i < n; ++i) y[(size_t)i * n + t] = 0.f;
-        e2[t] = lam[t];
-      }
-    }
-    __syncthreads();
-    for (int p = tid; p < n; p += 512) theta[(size_t)b * n + p] = fmaxf(e2[p], 0.f);
-    if (emit_factors) {
-      float* QT = ZTg + img;
-      for (int e = tid; e < n * n; e += 512) {
-        const int j = e / n, i = e - j * n;
-        QT[e] = A[i * ld + j];
-      }
-      __syncthreads();
-      for (int e = tid; e < n * n; e += 512) {   // Y through shared memory, to turn it over
-        const int j = e / n, p = e - j * n;
-        A[j * ld + p] = __ldcg(y + e);
-      }
-      __syncthreads();
-      float* YT = u0;  // the factorisations kept there are no longer needed
-      for (int e = tid; e < n * n; e += 512) {
-        const int p = e / n, j = e - p * n;
-        YT[e] = A[j * ld + p];
-      }
-      if (tid == 0 && s_fail) atomicMax(&status[b], (int)TC_ERR_NOT_CONVERGED);
-      return;
-    }
-    // ---------------- Z = Q Y:  ZT[p][i] = sum_j Q[i][j] Y[j][p] ----------------
-    // thread = (four eigenvectors p, twelve rows i): per j one 16-byte load of Y (coalesced over
-    // p) and twelve broadcast reads of Q from shared memory feed 48 multiply-adds
-    float* out = ZTg + img;
-    const bool vec = (n & 3) == 0;
-    const int npg = (n + 3) >> 2, nrg = (n + 11) / 12;
-    for (int w = tid; w < npg * nrg; w += 512) {
-      const int rg = w / npg, pg = w - rg * npg;
-      const int p0 = pg * 4, i0 = rg * 12;
-      float acc[12][4];
-      const float* qrow[12];
-#pragma unroll
-      for (int u = 0; u < 12; ++u) {
-        qrow[u] = A + min(i0 + u, n - 1) * ld;  // rows past the end are computed and dropped
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
-      }
-#pragma unroll 4
-      for (int j = 0; j < n; ++j) {
-        float4 yv;
-        const float* yr = y + (size_t)j * n + p0;
-        if (vec) {
-          yv = __ldcg(reinterpret_cast<const float4*>(yr));
-        } else {
-          yv.x = __ldcg(yr);
-          yv.y = (p0 + 1 < n) ? __ldcg(yr + 1) : 0.f;
-          yv.z = (p0 + 2 < n) ? __ldcg(yr + 2) : 0.f;
-          yv.w = (p0 + 3 < n) ? __ldcg(yr + 3) : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 12; ++u) {
-          const float a = qrow[u][j];
-          acc[u][0] = fmaf(a, yv.x, acc[u][0]);
-          acc[u][1] = fmaf(a, yv.y, acc[u][1]);
-          acc[u][2] = fmaf(a, yv.z, acc[u][2]);
-          acc[u][3] = fmaf(a, yv.w, acc[u][3]);
-        }
-      }
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        if (p0 + v >= n) continue;
-        float* orow = out + (size_t)(p0 + v) * n + i0;
-        if (vec && i0 + 12 <= n) {
-#pragma unroll
-          for (int u = 0; u < 12; u += 4)
-            *reinterpret_cast<float4*>(orow + u) =
-                make_float4(acc[u][v], acc[u + 1][v], acc[u + 2][v], acc[u + 3][v]);
-        } else {
-#pragma unroll
-          for (int u = 0; u < 12; ++u)
-            if (i0 + u < n) orow[u] = acc[u][v];
-        }
-      }
-    }
-  }
-  if (tid == 0 && s_fail) atomicMax(&status[b], (int)TC_ERR_NOT_CONVERGED);
-}
-
 typedef void (*jacobi_fn)(const float*, float*, float*, float*, int, int, float, int, int32_t*, float, float);
 
 static jacobi_fn pick_jacobi(int n) {
@@ -2285,27 +1533,8 @@ static jacobi_fn pick_jacobi(int n) {
 constexpr size_t SMEM_LIMIT = 220 * 1024;  // leaves room for the static shared variables
 
 static void launch_jacobi(const float* H, float* W, float* ZT, float* theta, int n, int batch,
-                          int max_sweeps, float rank_tol, float* scr1, float* scr2, float* scr3,
-                          float* scr4, size_t scr4_stride, int32_t* status, cudaStream_t st,
-                          int nparts = 1, int emit_factors = 0) {
+                          int max_sweeps, float rank_tol, int32_t* status, cudaStream_t st) {
   Scope scope_(KC_JACOBI, st);
-  {
-    const size_t tri = ((size_t)n * (n | 1) + 27 * (size_t)((n + 3) & ~3)) * sizeof(float);
-    if (n >= 3 && tri <= SMEM_LIMIT && scr1 != nullptr) {
-      auto go = [&](auto kernel) {
-        cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri);
-        { kernel<<<batch, 512, tri, st>>>(H, ZT, theta, n, rank_tol, W, scr1, scr2, scr3, scr4, scr4_stride, status, nparts, emit_factors); note_launch(); }
-      };
-      switch (n) {
-        case 128: go(tridiag_eig_kernel<128>); break;
-        case 144: go(tridiag_eig_kernel<144>); break;
-        case 160: go(tridiag_eig_kernel<160>); break;
-        case 192: go(tridiag_eig_kernel<192>); break;
-        default: go(tridiag_eig_kernel<0>); break;
-      }
-      return;
-    }
-  }
   jacobi_fn fn = pick_jacobi(n);
   const size_t need = 2 * (size_t)n * n * sizeof(float);
   const int use_smem = need <= SMEM_LIMIT;
@@ -2320,6 +1549,15 @@ static void launch_jacobi(const float* H, float* W, float* ZT, float* theta, int
   const float floor_rel = 1e-6f;
   const float count_rel = fmaxf(floor_rel, rank_tol * rank_tol);
   { fn<<<batch, 512, smem, st>>>(H, W, ZT, theta, n, max_sweeps, tol, use_smem, status, floor_rel, count_rel); note_launch(); }
+}
+
+// Which solver decomposes an n x n matrix.  Inverse iteration does not orthogonalise eigenvectors
+// against each other, which is fine while the wanted eigenvalues (rank_tol^2 theta_max and up) stand
+// clear of the float32 rounding level of the largest, about 1e-6 of it: from rank_tol = 1e-3 on.
+// Below that the full solve, and a subspace wider than 224, take Jacobi sweeps, whose vectors are
+// orthogonal whatever the spectrum, at a hundred times the time.  Eigenvalues alone need no such care.
+static bool use_tridiag(int n, bool full, bool values_only, float rank_tol) {
+  return eig_tridiag_supported(n) && (values_only || rank_tol >= 1e-3f || (!full && n <= 224));
 }
 
 static void launch_chol_inv(const float* S, float* RinvT, float* Rwork, int k, int batch,
@@ -2512,26 +1750,25 @@ void fill_i32(int32_t* p, int n, int v, cudaStream_t st) {
 // ==========================================================================================
 tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void* O, float* C_out,
                      float* sigma_out, int32_t* rank_out, int32_t* img_status, cudaStream_t st,
-                     float* full_scratch, cudaEvent_t g_ready) {
+                     bool values_only, cudaEvent_t g_ready) {
   // D.B images starting at image b0 of the workspace arrays; O and the outputs already point at
   // image b0.
   const int B = D.B, N = D.N, k = D.k;
   const int q = min(D.N, D.d);
   const size_t sG = (size_t)N * N, sY = (size_t)N * k, sK = (size_t)k * k;
   float* G = (float*)(ws + P.G) + b0 * sG;
-  float* W = (float*)(ws + P.W) + b0 * sK;
+  float* W = (float*)(ws + P.W + b0 * jacobi_work_bytes(k));
   float* ZT = (float*)(ws + P.ZT) + b0 * sK;
   float* theta = (float*)(ws + P.sigma) + (size_t)b0 * k;
 
   if (D.full) {
     if (g_ready) cudaStreamWaitEvent(st, g_ready, 0);
-    // with scratch for it (four N x N arrays per image) the tridiagonal solver takes the full
-    // problem when it fits in shared memory: it has no sweeps that a spectrum without a gap at
-    // the rounding level could keep alive
-    float* fs = full_scratch;
-    launch_jacobi(G, W, ZT, theta, N, B, D.max_sweeps, D.rank_tol, fs, fs ? fs + (size_t)B * sG : nullptr,
-                  fs ? fs + 2 * (size_t)B * sG : nullptr, fs ? fs + 3 * (size_t)B * sG : nullptr, sG,
-                  img_status, st);
+    if (use_tridiag(N, true, values_only, D.rank_tol)) {
+      tc_status e = launch_eig_tridiag(G, sG, N, N, B, D.rank_tol, theta, ZT, sK, N, W, img_status, st);
+      if (e != TC_OK) return e;
+    } else {
+      launch_jacobi(G, W, ZT, theta, N, B, D.max_sweeps, D.rank_tol, img_status, st);
+    }
     Scope scope_(KC_ICS, st);
     { ics_kernel<<<dim3((N + 63) / 64, B), 256, 2 * (size_t)N * sizeof(float), st>>>(
           theta, ZT, C_out, sigma_out, rank_out, img_status, N, N, q, D.rank_tol, 1, nullptr); note_launch(); }
@@ -2567,7 +1804,7 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
     float* Sk = (float*)(ws + P.Sk) + b0 * sK;
     float* Hk = (float*)(ws + P.Hk) + b0 * sK;
     float* Rinv = (float*)(ws + P.Rinv) + b0 * sK;
-    float* Es = (float*)(ws + P.Es) + b0 * 4 * sK;
+    float* Es = (float*)(ws + P.Es + b0 * jacobi_work_bytes(k));
     int32_t* stp = img_status;
     tc_status err = TC_OK;
     auto mm = [&](const float* A_, const float* B_, int M_, int K_, float* c, float* ct, int cls) {
@@ -2596,17 +1833,12 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
     mm(G, At, N, N, nullptr, Bt, KC_GEMM_GQ);
     mm(At, Bt, k, N, Hk, nullptr, KC_GEMM_TN);
     if (err != TC_OK) return err;
-    // The solver leaves the eigenvectors of H as the two factors Z = Q Y (Q from the reduction
-    // to tridiagonal form, Y the eigenvectors of the tridiagonal matrix): Q^T in QTk, Y^T in YTk.
-    float* QTk = Sk;  // the k x k matrices of the passes are free now
-    float* YTk = Es;  // (the solver's first work array, handed back as Y^T)
-    launch_jacobi(Hk, Es, QTk, theta, k, B, D.max_sweeps, D.rank_tol, Es + (size_t)B * sK,
-                  Es + 2 * (size_t)B * sK, Rinv, Es + 3 * (size_t)B * sK, sK, stp, st, 1, 1);
-    // 5. eigenvectors of G in the subspace, U = Q1 Q Y, as two products:
-    //    W = Q1 Q, then PT[p][x] = sum_j Y[j][p] W[x][j] (W Y written transposed)
-    mm(Ar, QTk, N, k, Br, nullptr, KC_GEMM);
+    float* ZT = Sk;  // the k x k matrix of the passes is free now
+    err = launch_eig_tridiag(Hk, sK, k, k, B, D.rank_tol, theta, ZT, sK, k, Es, stp, st);
+    // 5. eigenvectors of G in the subspace, U = Q1 Z, written transposed:
+    //    PT[p][x] = sum_i ZT[p][i] Q1[x][i]
     float* PT = Bt;
-    mm(Br, YTk, N, k, nullptr, PT, KC_GEMM);
+    mm(Ar, ZT, N, k, nullptr, PT, KC_GEMM);
     if (err != TC_OK) return err;
     Scope scope_(KC_ICS, st);
     { ics_kernel<<<dim3((N + 63) / 64, B), 256, 2 * (size_t)k * sizeof(float), st>>>(
@@ -2643,8 +1875,12 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
   // 4. Rayleigh-Ritz:  H = Q1^T G Q1
   gemm<float, float, false, false>(G, Y2, Y1, N, k, N, N, k, k, sG, sY, sY, B, st, KC_GEMM_GQ);   // T = G Q1
   gemm_tn_sym(Y2, Y1, Hm, k, N, sY, sY, B, st, KC_GEMM_TN);   // H = Q1^T T (symmetric)
-  // scratch of the solver: W, Sm, Rinv, Hm (k x k each) and the first k x k of each image's Y1 panel
-  launch_jacobi(Hm, W, ZT, theta, k, B, D.max_sweeps, D.rank_tol, Sm, Rinv, Hm, Y1, sY, img_status, st, parts);
+  if (use_tridiag(k, false, values_only, D.rank_tol)) {
+    tc_status e = launch_eig_tridiag(Hm, sK, k, k, B, D.rank_tol, theta, ZT, sK, k, W, img_status, st);
+    if (e != TC_OK) return e;
+  } else {
+    launch_jacobi(Hm, W, ZT, theta, k, B, D.max_sweeps, D.rank_tol, img_status, st);
+  }
   // 5. eigenvectors of G restricted to the subspace:  PT[p][x] = sum_i ZT[p][i] Q1[x][i]
   gemm<float, float, false, true>(ZT, Y2, Y0, k, N, k, k, k, N, sK, sY, sY, B, st);
   Scope scope_(KC_ICS, st);

@@ -45,7 +45,7 @@ struct Plan {
   size_t G;        // [B, N, N] f32
   size_t Y0, Y1, Y2;  // [B, N, k] f32 each (subspace solve only)
   size_t Sm, Rinv, Hm;  // [B, k, k] f32 each (subspace solve only; Sm, Hm: tn_parts(k) of them)
-  size_t W, ZT;    // [B, k, k] f32: Jacobi work matrix and accumulated rotations (column-major)
+  size_t W, ZT;    // [B] work array of the eigen-solver; [B, k, k] f32 eigenvectors
   size_t setA, setB, best_val, best_dst, msrc, mdst, kept;  // int32 / f32 lists
   size_t rank;     // [B] int32
   size_t flags;    // [B] int32 device status scratch
@@ -55,7 +55,7 @@ struct Plan {
                    // further on, [B][k][N] transposed
   size_t panel_T_off;
   size_t Sk, Hk;   // [B][k][k] f32: Y^T Y (later the eigenvectors) and the projected matrix
-  size_t Es;       // [B][4][k][k] f32 scratch of the tridiagonal solver
+  size_t Es;       // [B] scratch of the tridiagonal solver
   size_t total;
 };
 
@@ -165,13 +165,25 @@ bool gemm_f32x3_supported(int M, int NN, int K);
 tc_status launch_gemm_f32x3(const float* A, const float* B, int M, int NN, int K, int batch,
                             float* C, float* CT, int32_t* status, cudaStream_t st, int cls);
 
+// Eigen-decomposition of the symmetric part of H [batch][n][ldh], 3 <= n <= EIG_TRIDIAG_MAX:
+// theta [batch][n] ascending, ZT [batch][n][ldz] with the eigenvectors in its rows (zero rows for
+// eigenvalues under a quarter of the rank cut-off rank_tol^2 theta_max).  scratch: batch *
+// eig_tridiag_scratch_bytes(n) bytes, 16-byte aligned.
+constexpr int EIG_TRIDIAG_MAX = 768;
+bool eig_tridiag_supported(int n);
+size_t eig_tridiag_scratch_bytes(int n);
+tc_status launch_eig_tridiag(const float* H, size_t sH, int ldh, int n, int batch, float rank_tol, float* theta,
+                             float* ZT, size_t sZ, int ldz, void* scratch, int32_t* status, cudaStream_t st);
+
+// bytes per image of the work array of either eigen-solver (the Jacobi work matrix is k x k)
+inline size_t jacobi_work_bytes(int k) { return align_up(eig_tridiag_scratch_bytes(k), 256); }
+
 // Eigen-decomposition of G and Eq. 3-6:  C, theta (unsorted), then sorted sigma / rank.
 // g_ready: optional event after which G is complete when it is built on another stream (the
 // subspace solve waits for it in front of its first product with G).
-// full_scratch: optional 4 * B * N * N floats; with it a full solve (rank_cap = 0) of a matrix
-// that fits in shared memory goes through the tridiagonal solver instead of Jacobi sweeps.
+// values_only: the caller reads no eigenvectors (C_out), only sigma and the rank.
 tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void* O, float* C_out,
                      float* sigma_out, int32_t* rank_out, int32_t* img_status, cudaStream_t st,
-                     float* full_scratch = nullptr, cudaEvent_t g_ready = nullptr);
+                     bool values_only = false, cudaEvent_t g_ready = nullptr);
 
 }  // namespace tc

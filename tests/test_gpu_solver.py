@@ -1,0 +1,41 @@
+"""The dense linear algebra behind Eq. 3-5 / 3-6 (Sec. 3.3.1) at the sizes where a tile, a register
+layout or a cluster ends, against the float64 oracle, through the C ABI."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import ipgs_oracle as orc
+from paper_2503_10501_b200 import binding as tcb
+import parity_util as pu
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(N, d, rank, seed, batch=2, noise=1e-6):
+    """O of numerical rank `rank` (singular values geometric 1 .. 0.03), and attention."""
+    rng = np.random.default_rng(seed)
+    u = np.linalg.qr(rng.standard_normal((batch, N, rank)))[0]
+    w = np.linalg.qr(rng.standard_normal((batch, d, rank)))[0]
+    s = np.geomspace(100.0, 3.0, rank)
+    O = (u * s) @ w.transpose(0, 2, 1) + noise * rng.standard_normal((batch, N, d))
+    A = rng.random((batch, 1, 3, N))
+    return O.astype(np.float32), A.astype(np.float32)
+
+
+def _check(N, d, rank, rank_cap, seed):
+    O, A = _inputs(N, d, rank, seed)
+    p = tcb.Params(batch=2, n_tokens=N, d_model=d, n_heads=1, head_dim=8, n_query=3, keep=1,
+                   rank_tol=2e-3, dtype="f32", rank_cap=rank_cap)
+    g = tcb.tc_score(p, torch.from_numpy(O).cuda(), torch.from_numpy(A).cuda())
+    torch.cuda.synchronize()
+    assert not g["img_status"].any()
+    for b in range(2):
+        pu.check_scores({k: v[b].cpu().numpy() for k, v in g.items()}, orc.score(O[b], A[b], 0.5, 2e-3), 2e-3)
+
+
+# orders of the tridiagonal solver: the smallest, register layouts and cluster sizes from both sides,
+# and one that no layout fills
+@pytest.mark.parametrize("N", [3, 4, 7, 32, 33, 64, 65, 96, 97, 128, 129, 144, 145, 160, 161, 192, 193, 256,
+                               257, 320, 321, 384, 385, 448, 449, 500, 512, 513, 576, 577, 640, 641, 768])
+def test_full_solve_of_every_layout(N):
+    _check(N, 832, max(2, min(N // 3, 200)), 0, seed=N)
