@@ -50,8 +50,8 @@ Scope::~Scope() {
   g_prof.launches_at_close[slot] = g_launches.load();
 }
 
-tc_status launch_gram_simt(const Dims& D, const void* O, float* G, cudaStream_t st);
-tc_status launch_gram_tc(const Dims& D, const void* O, float* G, int32_t* status, cudaStream_t st);
+tc_status launch_gram_simt(const Dims& D, const void* O, float* G, int ldg, cudaStream_t st);
+tc_status launch_gram_tc(const Dims& D, const void* O, float* G, int ldg, int32_t* status, cudaStream_t st);
 void fill_i32(int32_t* p, int n, int v, cudaStream_t st);
 
 tc_status make_dims(const tc_params* p, Dims* out) {
@@ -92,14 +92,25 @@ tc_status make_dims(const tc_params* p, Dims* out) {
   if (((size_t)D.d * D.esz) % 16 != 0 || ((size_t)D.dh * D.esz) % 16 != 0) return TC_ERR_UNSUPPORTED;
   if (D.N > 4096) return TC_ERR_UNSUPPORTED;
   if (p->rank_cap < 0) return TC_ERR_INVALID_ARG;
+  D.ldn = (D.N + 3) & ~3;
+  D.cap = p->rank_cap;
   D.full = (p->rank_cap == 0) || (p->rank_cap >= D.N);
   D.k = D.full ? D.N : p->rank_cap;
   if (D.k > 1024) return TC_ERR_UNSUPPORTED;  // Jacobi keeps at most 32 elements per lane
   if (!D.full && D.k < 16) return TC_ERR_INVALID_ARG;
-  // the subspace solve runs its products on the tensor cores when the shapes fit its tiles
-  // (the sign sketch keeps one row of signs, d floats, in shared memory)
-  D.tcp = !D.full && (D.N & 3) == 0 && (size_t)D.d * sizeof(float) <= 48 * 1024 &&
-          gemm_f32x3_supported(D.N, D.k, D.N) && gemm_f32x3_supported(D.N, D.k, D.k);
+  // The subspace solve runs its products on the tensor cores, with the subspace widened to a multiple
+  // of 16; where that leaves no subspace, the Gram matrix itself is decomposed.  Above 640 dimensions
+  // it keeps to float32 multiply-adds: the error of the split products, up to 1.5e-6 of sum |a||b|, is
+  // then no longer small against the shifts that the Cholesky factorisations of so wide a basis have.
+  D.tcp = !D.full && D.k <= TCP_MAX;
+  if (D.tcp) {
+    D.k = (D.k + 15) & ~15;
+    if (D.k >= D.N) {
+      D.k = D.N;
+      D.tcp = false;
+      D.full = true;
+    }
+  }
   D.max_sweeps = p->max_sweeps > 0 ? p->max_sweeps : 30;
   D.lambda = p->lambda;
   D.rank_tol = p->rank_tol;
@@ -132,23 +143,23 @@ Plan make_plan(const Dims& D) {
   P.C = take(B * N * 4);
   P.E = take(B * N * 4);
   P.sigma = take(B * k * 4);
-  P.G = take(B * N * N * 4);
+  P.G = take(B * N * (size_t)D.ldn * 4);
   if (D.tcp) {
     P.panel_T_off = align_up(B * N * k * 4, 256);
-    P.PA = take(2 * P.panel_T_off);
-    P.PB = take(2 * P.panel_T_off);
+    P.PA = take(P.panel_T_off + B * k * D.ldn * 4);
+    P.PB = take(P.panel_T_off + B * k * D.ldn * 4);
     P.Sk = take(B * k * k * 4);
     P.Hk = take(B * k * k * 4);
     P.Rinv = take(B * k * k * 4);
+    P.Pk = take(B * chol_panel_floats(D.k) * 4);
     P.Es = take(B * jacobi_work_bytes(D.k));
   } else if (!D.full) {
     P.Y0 = take(B * N * k * 4);
     P.Y1 = take(B * N * k * 4);
     P.Y2 = take(B * N * k * 4);
-    const size_t parts = (size_t)tn_parts(D.k);  // k x k products arrive in this many parts
-    P.Sm = take(B * k * k * 4 * parts);
+    P.Sm = take(B * k * k * 4);
     P.Rinv = take(B * k * k * 4);
-    P.Hm = take(B * k * k * 4 * parts);
+    P.Hm = take(B * k * k * 4);
   }
   if (!D.tcp) {
     P.W = take(B * jacobi_work_bytes(D.k));
@@ -169,9 +180,9 @@ Plan make_plan(const Dims& D) {
 }
 
 // float16 inputs go to the tensor cores; float32 inputs keep full precision on the plain ALUs
-tc_status launch_gram(const Dims& D, const void* O, float* G, int32_t* status, cudaStream_t st) {
-  if (D.f16 || D.bf16) return launch_gram_tc(D, O, G, status, st);
-  return launch_gram_simt(D, O, G, st);
+tc_status launch_gram(const Dims& D, const void* O, float* G, int ldg, int32_t* status, cudaStream_t st) {
+  if (D.f16 || D.bf16) return launch_gram_tc(D, O, G, ldg, status, st);
+  return launch_gram_simt(D, O, G, ldg, st);
 }
 
 static tc_status check_launch() {
@@ -278,15 +289,15 @@ static tc_status enqueue_score(const Ctx& c, const void* O, const void* A, float
     // the sketch and its first Cholesky-QR pass do not read G: with groups, the Gram matrix is
     // built beside them on a stream of its own and joined in front of the first product with G
     cudaEvent_t gram_done = nullptr;
-    float* Gg = (float*)(c.ws + c.P.G) + (size_t)b0 * D.N * D.N;
+    float* Gg = (float*)(c.ws + c.P.G) + (size_t)b0 * D.N * D.ldn;
     if (ng > 1 && !D.full) {
       cudaStreamWaitEvent(gs->s2[g], gs->fork, 0);
       if (late) cudaStreamWaitEvent(gs->s2[g], gs->gram_done[g - per_wave], 0);
-      err = launch_gram(Dg, Og, Gg, img_status + b0, gs->s2[g]);
+      err = launch_gram(Dg, Og, Gg, D.ldn, img_status + b0, gs->s2[g]);
       cudaEventRecord(gs->gram_done[g], gs->s2[g]);
       gram_done = gs->gram_done[g];
     } else {
-      err = launch_gram(Dg, Og, Gg, img_status + b0, st);
+      err = launch_gram(Dg, Og, Gg, D.ldn, img_status + b0, st);
     }
     if (err == TC_OK)
       err = launch_ics(Dg, c.P, c.ws, b0, Og, C + (size_t)b0 * D.N, sigma ? sigma + (size_t)b0 * q : nullptr,
@@ -477,7 +488,7 @@ tc_status tc_carve(const tc_params* p, const void* O, const void* A, const void*
     launch_prune(Dg, E + b * D.N, sA, sB, st);
     if (D.M > 0) {
       if (D.sim_src == 0) {
-        launch_match_gram(Dg, (const float*)(c.ws + c.P.G) + b * D.N * D.N, sA, sB, gbv, gbd, gst, st);
+        launch_match_gram(Dg, (const float*)(c.ws + c.P.G) + b * D.N * D.ldn, D.ldn, sA, sB, gbv, gbd, gst, st);
       } else if (D.sim_src == 1) {
         launch_match_rows(Dg, Xg, sA, sB, gbv, gbd, gst, st);
       } else {
@@ -670,7 +681,7 @@ tc_status tc_gram(const tc_params* p, const void* O, float* G, void* stream) {
   tc_status s = make_dims(p, &D);
   if (s != TC_OK) return s;
   if (!O || !G || misaligned(O) || misaligned(G)) return TC_ERR_INVALID_ARG;
-  s = launch_gram(D, O, G, nullptr, (cudaStream_t)stream);
+  s = launch_gram(D, O, G, D.N, nullptr, (cudaStream_t)stream);
   if (s != TC_OK) return s;
   return check_launch();
 }
@@ -680,10 +691,13 @@ tc_status tc_matmul_f32x3(const float* A, const float* B, float* C, float* CT, i
   if (!A || !B || (!C && !CT) || batch < 1 || M < 1 || NN < 1 || K < 1) return TC_ERR_INVALID_ARG;
   if (misaligned(A) || misaligned(B) || (C && misaligned(C)) || (CT && misaligned(CT)))
     return TC_ERR_INVALID_ARG;
-  if (!gemm_f32x3_supported(M, NN, K)) return TC_ERR_UNSUPPORTED;
+  if ((K & 3) != 0 || (NN != 128 && NN != 144 && NN != 160 && NN != 192)) return TC_ERR_UNSUPPORTED;
   cudaStream_t st = (cudaStream_t)stream;
   if (img_status) fill_i32(img_status, batch, 0, st);
-  tc_status s = launch_gemm_f32x3(A, B, M, NN, K, batch, C, CT, img_status, st, KC_GEMM);
+  F32x3Result R;
+  R.C = C; R.ld = NN; R.stride = (size_t)M * NN;
+  R.CT = CT; R.ldT = M; R.strideT = (size_t)M * NN;
+  tc_status s = launch_gemm_f32x3({A, K, (size_t)M * K}, {B, K, (size_t)NN * K}, M, NN, K, batch, R, img_status, st, KC_GEMM);
   if (s != TC_OK) return s;
   return check_launch();
 }
@@ -734,7 +748,7 @@ tc_status tc_rank(const tc_params* p, const void* O, const int32_t* idx, int32_t
     launch_gather_rows(F, n_sub, O, idx, w + rows_off, img_status, st);
     rows = w + rows_off;
   }
-  s = launch_gram(D, rows, (float*)(w + P.G), img_status, st);
+  s = launch_gram(D, rows, (float*)(w + P.G), D.ldn, img_status, st);
   if (s != TC_OK) return s;
   s = launch_ics(D, P, w, 0, rows, (float*)(w + P.C), sigma, rank, img_status, st, true);
   if (s != TC_OK) return s;

@@ -7,8 +7,9 @@
 // the contraction index K contiguous in both (A [M][K], B [NN][K]); they are split on the way
 // through shared memory.
 //
-// One CTA produces a 128 x NN tile of C for one image (NN = the whole width of C, a multiple of
-// 16; 128, 144, 160 and 192 are built).  Four roles run side by side:
+// One CTA produces a 128 x NN tile of C for one image, NN a multiple of 16 up to 192: the whole width
+// of C up to 192 (every width the solve pads its subspace to has a tile of its own), else the width
+// cut into equal parts.  Four roles run side by side:
 //   - warp 12 (one lane) streams 32-wide K slabs of A and B into a ring of shared-memory stages
 //     with TMA (128-byte swizzle, out-of-range rows / K read as zero);
 //   - warps 8-11 turn a landed slab into its two parts: hi overwrites the value where it lies,
@@ -64,15 +65,21 @@ __device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t da, uint64_t
 }
 
 struct Out {
-  float* plain;    // [batch][M][NN]
-  float* plainT;   // [batch][NN][M]
+  float* plain;    // [batch][M][ld]
+  float* plainT;   // [batch][W][ldT]
+  size_t sC, sT;   // floats per image
+  int ld, ldT;
+  int W;           // columns of C
+  int rows_t;      // rows of C that are written to plainT
+  int sub;         // C -= A B^T instead of C = A B^T, with C taken as zero in rows z0 .. z1 - 1
+  int z0, z1;
 };
 
 // NN: width of C (compile time: it sizes the register tile).
 template <int NN>
 __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_constant__ CUtensorMap mapA,
                                                            const __grid_constant__ CUtensorMap mapB,
-                                                           Out out, int M, int K, int m_tiles,
+                                                           Out out, int M, int K, int m_tiles, int n_tiles,
                                                            int32_t* __restrict__ status) {
   constexpr int STAGES = stages_for(NN);
   constexpr int NCHUNK = NN / 16;            // 16-column chunks of the accumulator
@@ -91,7 +98,8 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
   __shared__ int s_fail;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = blockIdx.x / m_tiles, mt = blockIdx.x % m_tiles;
+  const int b = blockIdx.x / (m_tiles * n_tiles), tile = blockIdx.x % (m_tiles * n_tiles);
+  const int mt = tile % m_tiles, n0 = (tile / m_tiles) * NN;
   const int slabs = (K + BK - 1) / BK;
   const int nchunks = (slabs + DRAIN_SLABS - 1) / DRAIN_SLABS;
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -137,7 +145,7 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
         const uint32_t full = smem_u32(&bar_full[s]);
         mbar_expect_tx(full, HALF);
         tma_load_3d(st_hi(s), &mapA, kb * BK, mt * BM, b, full);
-        tma_load_3d(st_hi(s) + A_B, &mapB, kb * BK, 0, b, full);
+        tma_load_3d(st_hi(s) + A_B, &mapB, kb * BK, n0, b, full);
       }
     }
   } else if (warp == W_MMA) {
@@ -285,25 +293,34 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
     }
     asm volatile("bar.sync 2, 256;" ::: "memory");
     if (s_fail == 0) {
-      const size_t MN = (size_t)M * NN;
+      const int w4 = min(NN, out.W - n0) / 4;   // widths are multiples of four
       if (out.plain != nullptr) {
         for (int rl = warp; rl < BM; rl += EPI_WARPS) {
           const int grow = mt * BM + rl;
           if (grow >= M) break;
           const float4* src = reinterpret_cast<const float4*>(stg + rl * SROW);
-          float4* dst = reinterpret_cast<float4*>(out.plain + (size_t)b * MN + (size_t)grow * NN);
-          for (int v = lane; v < NN / 4; v += 32) dst[v] = src[v];
+          float4* dst = reinterpret_cast<float4*>(out.plain + (size_t)b * out.sC + (size_t)grow * out.ld + n0);
+          const bool keep = out.sub && (grow < out.z0 || grow >= out.z1);
+          for (int v = lane; v < w4; v += 32) {
+            float4 x = src[v];
+            if (out.sub) {
+              const float4 o = keep ? dst[v] : make_float4(0.f, 0.f, 0.f, 0.f);
+              x = make_float4(o.x - x.x, o.y - x.y, o.z - x.z, o.w - x.w);
+            }
+            dst[v] = x;
+          }
         }
       }
       const int row = mt * BM + quad * 32 + lane;
-      if (row < M && out.plainT != nullptr) {
+      if (row < out.rows_t && out.plainT != nullptr) {
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
           const int chunk = 2 * c + half;
           if (chunk >= NCHUNK) continue;
-          float* dst = out.plainT + (size_t)b * MN + (size_t)(chunk * 16) * M + row;
+          float* dst = out.plainT + (size_t)b * out.sT + (size_t)(n0 + chunk * 16) * out.ldT + row;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) dst[(size_t)j * M] = acc[c][j];
+          for (int j = 0; j < 16; ++j)
+            if (n0 + chunk * 16 + j < out.W) dst[(size_t)j * out.ldT] = acc[c][j];
         }
       }
     } else if (status != nullptr && threadIdx.x == 0) {
@@ -319,15 +336,16 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
   }
 }
 
-// [K, rows, batch] float32, box 32 x box_rows x 1, 128-byte swizzle, zero fill
-bool encode_operand(CUtensorMap* map, const float* base, int rows, int K, int batch, int box_rows) {
+// [K, rows, batch] float32 with rows `ld` and images `stride` floats apart, box 32 x box_rows x 1,
+// 128-byte swizzle, zero fill
+bool encode_operand(CUtensorMap* map, const F32x3Operand& o, int rows, int K, int batch, int box_rows) {
   encode_fn enc = get_encode();
   if (enc == nullptr) return false;
   const cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)batch};
-  const cuuint64_t strides[2] = {(cuuint64_t)K * 4, (cuuint64_t)rows * K * 4};
+  const cuuint64_t strides[2] = {(cuuint64_t)o.ld * 4, (cuuint64_t)o.stride * 4};
   const cuuint32_t box[3] = {BK, (cuuint32_t)box_rows, 1};
   const cuuint32_t estr[3] = {1, 1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims, strides, box, estr,
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(o.p), dims, strides, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -339,32 +357,40 @@ tc_status launch_nn(const CUtensorMap& mapA, const CUtensorMap& mapB, const Out&
   if (cudaFuncSetAttribute((const void*)gemm_f32x3_kernel<NN>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return TC_ERR_CUDA;
-  const int m_tiles = (M + BM - 1) / BM;
-  gemm_f32x3_kernel<NN><<<batch * m_tiles, THREADS, smem, st>>>(mapA, mapB, out, M, K, m_tiles, status);
+  const int m_tiles = (M + BM - 1) / BM, n_tiles = (out.W + NN - 1) / NN;
+  gemm_f32x3_kernel<NN><<<batch * m_tiles * n_tiles, THREADS, smem, st>>>(mapA, mapB, out, M, K, m_tiles,
+                                                                         n_tiles, status);
   note_launch();
   return TC_OK;
 }
 
 }  // namespace
 
-bool gemm_f32x3_supported(int M, int NN, int K) {
-  if (M < 1 || K < 4 || (K & 3) != 0) return false;  // TMA rows are whole 16-byte vectors
-  return NN == 128 || NN == 144 || NN == 160 || NN == 192;
-}
-
-// C [batch][M][NN] = A B^T with A [batch][M][K], B [batch][NN][K] float32, 16-byte aligned.
-tc_status launch_gemm_f32x3(const float* A, const float* B, int M, int NN, int K, int batch,
-                            float* C, float* CT, int32_t* status, cudaStream_t st, int cls) {
-  if (!gemm_f32x3_supported(M, NN, K)) return TC_ERR_UNSUPPORTED;
+// C = A B^T; see the declaration.
+tc_status launch_gemm_f32x3(const F32x3Operand& A, const F32x3Operand& B, int M, int W, int K, int batch,
+                            const F32x3Result& R, int32_t* status, cudaStream_t st, int cls) {
+  // TMA rows and 16-byte stores: whole vectors everywhere
+  if (M < 1 || W < 4 || (W & 3) || K < 1 || ((A.ld | B.ld) & 3) || ((A.stride | B.stride) & 3)) return TC_ERR_UNSUPPORTED;
+  if (R.C != nullptr && ((R.ld & 3) || (R.stride & 3))) return TC_ERR_UNSUPPORTED;
+  const int n_tiles = (W + 191) / 192;
+  int nn = ((W + n_tiles - 1) / n_tiles + 15) / 16 * 16;
+  if (nn < 64) nn = 64;
   CUtensorMap mapA, mapB;
-  if (!encode_operand(&mapA, A, M, K, batch, BM) || !encode_operand(&mapB, B, NN, K, batch, NN))
-    return TC_ERR_CUDA;
-  Out out{C, CT};
+  if (!encode_operand(&mapA, A, M, K, batch, BM) || !encode_operand(&mapB, B, W, K, batch, nn)) return TC_ERR_CUDA;
+  Out out;
+  out.plain = R.C; out.plainT = R.CT; out.sC = R.stride; out.sT = R.strideT; out.ld = R.ld; out.ldT = R.ldT;
+  out.W = W; out.rows_t = R.rows_t < 0 ? M : R.rows_t;
+  out.sub = R.subtract ? 1 : 0; out.z0 = R.zero_from; out.z1 = R.zero_to;
   Scope scope_(cls, st);
-  switch (NN) {
+  switch (nn) {
+    case 64: return launch_nn<64>(mapA, mapB, out, M, K, batch, status, st);
+    case 80: return launch_nn<80>(mapA, mapB, out, M, K, batch, status, st);
+    case 96: return launch_nn<96>(mapA, mapB, out, M, K, batch, status, st);
+    case 112: return launch_nn<112>(mapA, mapB, out, M, K, batch, status, st);
     case 128: return launch_nn<128>(mapA, mapB, out, M, K, batch, status, st);
     case 144: return launch_nn<144>(mapA, mapB, out, M, K, batch, status, st);
     case 160: return launch_nn<160>(mapA, mapB, out, M, K, batch, status, st);
+    case 176: return launch_nn<176>(mapA, mapB, out, M, K, batch, status, st);
     case 192: return launch_nn<192>(mapA, mapB, out, M, K, batch, status, st);
     default: return TC_ERR_UNSUPPORTED;
   }

@@ -52,7 +52,7 @@ __device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t da, uint64_t 
 }
 
 __global__ void __launch_bounds__(192) gram_tc_kernel(const __grid_constant__ CUtensorMap map,
-                                                     float* __restrict__ G, int N, int d,
+                                                     float* __restrict__ G, int N, int ldg, int d,
                                                      int tiles_per_image, int bf16,
                                                      int32_t* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
@@ -197,14 +197,14 @@ __global__ void __launch_bounds__(192) gram_tc_kernel(const __grid_constant__ CU
     }
     asm volatile("bar.sync 1, 128;" ::: "memory");
     if (s_fail == 0) {
-      float* Gb = G + (size_t)b * N * N;
+      float* Gb = G + (size_t)b * N * ldg;
       for (int rl = warp; rl < TILE; rl += 4) {
         const int grow = ti * TILE + rl;
         if (grow >= N) break;
         const int col = tj * TILE + 4 * lane;
         const float4 v = *reinterpret_cast<const float4*>(stg + rl * SROW + 4 * lane);
-        float* dst = Gb + (size_t)grow * N + col;
-        if (col + 3 < N && (N & 3) == 0) {
+        float* dst = Gb + (size_t)grow * ldg + col;
+        if (col + 3 < N && (ldg & 3) == 0) {
           *reinterpret_cast<float4*>(dst) = v;
         } else {
           if (col < N) dst[0] = v.x;
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(192) gram_tc_kernel(const __grid_constant__ CU
           const int col0 = tj * TILE + q * 32;
 #pragma unroll
           for (int j = 0; j < 32; ++j)
-            if (col0 + j < N) Gb[(size_t)(col0 + j) * N + row] = acc[q * 32 + j];
+            if (col0 + j < N) Gb[(size_t)(col0 + j) * ldg + row] = acc[q * 32 + j];
         }
       }
     } else if (status != nullptr) {
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(192) gram_tc_kernel(const __grid_constant__ CU
       const int row = ti * TILE + warp * 32 + lane;
       if (row < N)
         for (int j = 0; j < TILE; ++j)
-          if (tj * TILE + j < N) G[((size_t)b * N + row) * N + tj * TILE + j] = __int_as_float(0x7fc00000);
+          if (tj * TILE + j < N) G[((size_t)b * N + row) * ldg + tj * TILE + j] = __int_as_float(0x7fc00000);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(192) gram_tc_kernel(const __grid_constant__ CU
 
 // Returns TC_ERR_UNSUPPORTED when the tensor map cannot be built (caller may not fall back
 // silently: it reports the error).
-tc_status launch_gram_tc(const Dims& D, const void* O, float* G, int32_t* status, cudaStream_t st) {
+tc_status launch_gram_tc(const Dims& D, const void* O, float* G, int ldg, int32_t* status, cudaStream_t st) {
   encode_fn enc = get_encode();
   if (enc == nullptr) return TC_ERR_CUDA;
   CUtensorMap map;
@@ -265,7 +265,7 @@ tc_status launch_gram_tc(const Dims& D, const void* O, float* G, int32_t* status
   const int nt = (D.N + TILE - 1) / TILE;
   const int tiles = nt * (nt + 1) / 2;
   Scope scope_(KC_GRAM, st);
-  gram_tc_kernel<<<D.B * tiles, 192, SMEM_BYTES, st>>>(map, G, D.N, D.d, tiles, D.bf16 ? 1 : 0, status);
+  gram_tc_kernel<<<D.B * tiles, 192, SMEM_BYTES, st>>>(map, G, D.N, ldg, D.d, tiles, D.bf16 ? 1 : 0, status);
   note_launch();
   return TC_OK;
 }

@@ -151,7 +151,7 @@ __device__ inline void warp_best(float& val, int& idx) {
   }
 }
 
-__global__ void __launch_bounds__(128) match_gram_kernel(const float* __restrict__ G,
+__global__ void __launch_bounds__(128) match_gram_kernel(const float* __restrict__ G, int ldg,
                                                         const int32_t* __restrict__ setA,
                                                         const int32_t* __restrict__ setB,
                                                         float* __restrict__ best_val,
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(128) match_gram_kernel(const float* __restrict
   const int jb = blockIdx.x * 4 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (jb >= nB) return;
-  const float* Gb = G + (size_t)b * N * N;
+  const float* Gb = G + (size_t)b * N * ldg;
   const int tb = setB[(size_t)b * nB + jb];
   // a token number outside [0, N) in a caller's list is reported and never used as an address
   if (tb < 0 || tb >= N) {
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(128) match_gram_kernel(const float* __restrict
     }
     return;
   }
-  const float inv_b = inv_norm_from_sq(Gb[(size_t)tb * N + tb]);
+  const float inv_b = inv_norm_from_sq(Gb[(size_t)tb * ldg + tb]);
   float bv = -INFINITY;
   int bi = 0x7fffffff;
   for (int ja = lane; ja < nA; ja += 32) {
@@ -182,8 +182,8 @@ __global__ void __launch_bounds__(128) match_gram_kernel(const float* __restrict
       atomicMax(&status[b], (int)TC_ERR_INVALID_ARG);
       continue;
     }
-    const float inv_a = inv_norm_from_sq(Gb[(size_t)ta * N + ta]);
-    const float c = Gb[(size_t)tb * N + ta] * inv_b * inv_a;
+    const float inv_a = inv_norm_from_sq(Gb[(size_t)ta * ldg + ta]);
+    const float c = Gb[(size_t)tb * ldg + ta] * inv_b * inv_a;
     if (c > bv || (c == bv && ta < bi)) {
       bv = c;
       bi = ta;
@@ -196,12 +196,12 @@ __global__ void __launch_bounds__(128) match_gram_kernel(const float* __restrict
   }
 }
 
-void launch_match_gram(const Dims& D, const float* G, const int32_t* setA, const int32_t* setB,
+void launch_match_gram(const Dims& D, const float* G, int ldg, const int32_t* setA, const int32_t* setB,
                        float* best_val, int32_t* best_dst, int32_t* status, cudaStream_t st) {
   Scope scope_(KC_MATCH, st);
   if (D.nB == 0 || D.nA == 0) return;
   dim3 grid((D.nB + 3) / 4, D.B);
-  { match_gram_kernel<<<grid, 128, 0, st>>>(G, setA, setB, best_val, best_dst, D.N, D.nA, D.nB, status); note_launch(); }
+  { match_gram_kernel<<<grid, 128, 0, st>>>(G, ldg, setA, setB, best_val, best_dst, D.N, D.nA, D.nB, status); note_launch(); }
 }
 
 // ------------------------------------------------------------------------------------------

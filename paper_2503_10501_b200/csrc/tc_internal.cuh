@@ -21,9 +21,12 @@ inline std::atomic<int> g_refuse_encode{0};
 struct Dims {
   int B, N, d, H, dh, T;
   int keep, M, P, nA, nB;
-  int k;          // dimension of the decomposed subspace: rank_cap, or N for the full solve
-  bool full;      // rank_cap == 0
-  bool tcp;       // the subspace solve runs its products on the tensor cores (split panels)
+  int cap;        // rank_cap as given (0 or >= N: none)
+  int k;          // dimension of the decomposition: N for the full solve, else rank_cap, on the tensor
+                  // cores rounded up to a multiple of 16
+  bool full;      // the Gram matrix itself is decomposed
+  bool tcp;       // the subspace solve runs its products on the tensor cores
+  int ldn;        // pitch in floats of G's rows and of transposed panels: N rounded up to a multiple of 4
   int esz;        // bytes per element of O, A, X, K, V
   bool f16;       // float16 storage
   bool bf16;      // bfloat16 storage (neither: float32)
@@ -42,9 +45,9 @@ struct Plan {
   size_t s_part;   // [B, chunks, N] f32   partial column sums of A
   size_t S, C, E;  // [B, N] f32 each
   size_t sigma;    // [B, k] f32 (unsorted eigenvalue norms theta)
-  size_t G;        // [B, N, N] f32
+  size_t G;        // [B, N, ldn] f32
   size_t Y0, Y1, Y2;  // [B, N, k] f32 each (subspace solve only)
-  size_t Sm, Rinv, Hm;  // [B, k, k] f32 each (subspace solve only; Sm, Hm: tn_parts(k) of them)
+  size_t Sm, Rinv, Hm;  // [B, k, k] f32 each (subspace solve only)
   size_t W, ZT;    // [B] work array of the eigen-solver; [B, k, k] f32 eigenvectors
   size_t setA, setB, best_val, best_dst, msrc, mdst, kept;  // int32 / f32 lists
   size_t rank;     // [B] int32
@@ -52,10 +55,11 @@ struct Plan {
   size_t Kmean;    // [B, N, dh] f32: head-mean keys (sim_src == 2 only)
   // tensor-core subspace solve (Dims::tcp)
   size_t PA, PB;   // two sets of tall panels: [B][N][k] row-major and, panel_T_off bytes
-                   // further on, [B][k][N] transposed
+                   // further on, [B][k][ldn] transposed
   size_t panel_T_off;
   size_t Sk, Hk;   // [B][k][k] f32: Y^T Y (later the eigenvectors) and the projected matrix
   size_t Es;       // [B] scratch of the tridiagonal solver
+  size_t Pk;       // [B][chol_panel_floats(k)] f32: panel of the blocked Cholesky factorisation
   size_t total;
 };
 
@@ -67,10 +71,6 @@ __device__ __forceinline__ float tf32_round(float x) {
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
   return __uint_as_float(r);
 }
-
-// Number of parts per image in which the k x k products of the subspace solve are stored
-// (partial sums over chunks of the long dimension, added up by the kernel that reads them).
-int tn_parts(int k);
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -117,7 +117,7 @@ void launch_prune(const Dims& D, const float* E, int32_t* setA, int32_t* setB, c
 // Eq. 3-10 best match per Set-B token, from the Gram matrix or from the rows of O.
 // (status [B]: receives TC_ERR_INVALID_ARG for an image whose lists hold a token number outside
 // [0, N); such an entry is skipped, never used as an address.  The same for the launchers below.)
-void launch_match_gram(const Dims& D, const float* G, const int32_t* setA, const int32_t* setB,
+void launch_match_gram(const Dims& D, const float* G, int ldg, const int32_t* setA, const int32_t* setB,
                        float* best_val, int32_t* best_dst, int32_t* status, cudaStream_t st);
 void launch_match_rows(const Dims& D, const void* O, const int32_t* setA, const int32_t* setB,
                        float* best_val, int32_t* best_dst, int32_t* status, cudaStream_t st);
@@ -156,14 +156,40 @@ tc_status launch_probe(int B, int H, int dh, int L, int n_sys, int n_vis, int pr
                        const void* Q, const void* K, const void* V, void* O, void* A, void* ws,
                        int32_t* status, cudaStream_t st, int bf);
 
-// G = O O^T (float32 out).
-tc_status launch_gram(const Dims& D, const void* O, float* G, int32_t* status, cudaStream_t st);
+// G = O O^T (float32 out, rows ldg floats apart).
+tc_status launch_gram(const Dims& D, const void* O, float* G, int ldg, int32_t* status, cudaStream_t st);
 
-// C [batch][M][NN] = A B^T on the tensor cores, float32-accurate (A [batch][M][K],
-// B [batch][NN][K]); C and / or its transpose CT [batch][NN][M] are written (either may be null).
-bool gemm_f32x3_supported(int M, int NN, int K);
-tc_status launch_gemm_f32x3(const float* A, const float* B, int M, int NN, int K, int batch,
-                            float* C, float* CT, int32_t* status, cudaStream_t st, int cls);
+// C [batch][M][W] = A B^T on the tensor cores, float32-accurate, for A [batch][M][K] and B [batch][W][K]
+// with the contraction index contiguous; W, pitches and strides (in floats) multiples of four, bases
+// 16-byte aligned.  C and / or its transpose CT [batch][W][M] are written (either may be null).
+struct F32x3Operand {
+  const float* p;
+  int ld;          // floats between rows
+  size_t stride;   // floats between images
+};
+struct F32x3Result {
+  float* C;
+  int ld;
+  size_t stride;
+  float* CT;
+  int ldT;
+  size_t strideT;
+  int rows_t = -1;        // rows of C that go to CT (-1: all)
+  bool subtract = false;  // C -= A B^T, C counting as zero in rows zero_from .. zero_to - 1
+  int zero_from = 0, zero_to = 0;
+};
+tc_status launch_gemm_f32x3(const F32x3Operand& A, const F32x3Operand& B, int M, int W, int K, int batch,
+                            const F32x3Result& R, int32_t* status, cudaStream_t st, int cls);
+
+// RinvT [batch][k][k] = L^{-1} (zero above the diagonal) with L L^T = S + shift_rel max_i S_ii I, for
+// S [batch][k][k] symmetric (overwritten), k a multiple of 16.  A pivot well below zero (or no number)
+// is reported as TC_ERR_BREAKDOWN.  Above CHOL_BLOCK_MAX the factorisation is blocked and needs the
+// panel [batch][chol_panel_floats(k)].
+constexpr int CHOL_BLOCK_MAX = 192;
+constexpr int TCP_MAX = 192;  // widest subspace whose products run on the tensor cores
+size_t chol_panel_floats(int k);
+tc_status launch_chol_inv(float* S, float* RinvT, float* panel, int k, int batch, float shift_rel,
+                          int32_t* status, cudaStream_t st);
 
 // Eigen-decomposition of the symmetric part of H [batch][n][ldh], 3 <= n <= EIG_TRIDIAG_MAX:
 // theta [batch][n] ascending, ZT [batch][n][ldz] with the eigenvectors in its rows (zero rows for

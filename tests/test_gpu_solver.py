@@ -11,7 +11,7 @@ import parity_util as pu
 pytestmark = pytest.mark.gpu
 
 
-def _inputs(N, d, rank, seed, batch=2, noise=1e-6):
+def _inputs(N, d, rank, seed, noise, batch=2):
     """O of numerical rank `rank` (singular values geometric 1 .. 0.03), and attention."""
     rng = np.random.default_rng(seed)
     u = np.linalg.qr(rng.standard_normal((batch, N, rank)))[0]
@@ -22,8 +22,8 @@ def _inputs(N, d, rank, seed, batch=2, noise=1e-6):
     return O.astype(np.float32), A.astype(np.float32)
 
 
-def _check(N, d, rank, rank_cap, seed):
-    O, A = _inputs(N, d, rank, seed)
+def _check(N, d, rank, rank_cap, seed, noise=1e-6):
+    O, A = _inputs(N, d, rank, seed, noise)
     p = tcb.Params(batch=2, n_tokens=N, d_model=d, n_heads=1, head_dim=8, n_query=3, keep=1,
                    rank_tol=2e-3, dtype="f32", rank_cap=rank_cap)
     g = tcb.tc_score(p, torch.from_numpy(O).cuda(), torch.from_numpy(A).cuda())
@@ -39,3 +39,12 @@ def _check(N, d, rank, rank_cap, seed):
                                257, 320, 321, 384, 385, 448, 449, 500, 512, 513, 576, 577, 640, 641, 768])
 def test_full_solve_of_every_layout(N):
     _check(N, 832, max(2, min(N // 3, 200)), 0, seed=N)
+
+
+# subspaces: widths that no product tile fills, around one and several Cholesky blocks and the width the
+# float32 chain takes over at; token counts that are no multiple of four; a bound that leaves no
+# subspace once it is rounded up
+@pytest.mark.parametrize("N,rank_cap", [(97, 30), (131, 47), (203, 64), (330, 100), (333, 177), (401, 193), (450, 209),
+                                        (601, 385), (801, 577), (900, 640), (902, 641), (120, 111), (2881, 150)])
+def test_subspace_of_every_width(N, rank_cap):
+    _check(N, 1000, max(8, min(rank_cap - 16, rank_cap * 3 // 4, 200)), rank_cap, seed=N, noise=1e-3)
