@@ -292,4 +292,209 @@ tc_status launch_chol_inv(float* S, float* RinvT, float* panel, int k, int batch
   return TC_OK;
 }
 
+// ------------------------------------------------------------------------------------------
+// The same for a wide basis (float32 multiply-adds only): every entry of the factor and of the inverse
+// is the chain of multiply-adds that the textbook loops give, in their order, whatever the tiling.
+//   chol_f32_prepare   adds the shift, keeps the largest diagonal entry
+//   chol_f32_panel     32 rows of the factor: every block factors the diagonal block for itself (one
+//                      warp), then a thread per column substitutes
+//   chol_f32_update    S[r][c] -= sum_m F[m][r] F[m][c] over those 32 rows, 64 x 64 tiles
+//   chol_f32_inverse   a warp per column of the inverse, back substitution
+// What bounds the first three is 2 k / 32 dependent launches of about 4 us, the last one a chain of k
+// steps of some 300 cycles.  Measured at k = 736, four matrices: CHOLW_MEASURED
+// ------------------------------------------------------------------------------------------
+namespace {
+
+constexpr int WB = 32;  // rows per step
+
+__global__ void __launch_bounds__(256) chol_f32_prepare(float* __restrict__ S, float* __restrict__ F, int k,
+                                                       float shift_rel) {
+  __shared__ float s_red[8];
+  float* Sb = S + (size_t)blockIdx.x * k * k;
+  float md = 0.f;
+  for (int i = threadIdx.x; i < k; i += 256) md = fmaxf(md, Sb[(size_t)i * (k + 1)]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) md = fmaxf(md, __shfl_xor_sync(0xffffffffu, md, o));
+  if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = md;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) md = fmaxf(md, s_red[w]);
+  const float shift = shift_rel * md;
+  for (int i = threadIdx.x; i < k; i += 256) Sb[(size_t)i * (k + 1)] += shift;
+  if (threadIdx.x == 0) F[(size_t)blockIdx.x * k * k + (size_t)(k - 1) * k] = md;  // (below the diagonal: free)
+}
+
+// grid (column tiles of 128, batch), block 128
+__global__ void __launch_bounds__(128) chol_f32_panel(const float* __restrict__ S, float* __restrict__ F, int k, int j0,
+                                                     int32_t* __restrict__ status) {
+  __shared__ float D[WB][WB + 1];
+  __shared__ float s_inv[WB];
+  const int tid = threadIdx.x, lane = tid & 31, b = blockIdx.y;
+  const int w = min(WB, k - j0);
+  const float* Sb = S + (size_t)b * k * k;
+  float* Fb = F + (size_t)b * k * k;
+  for (int e = tid; e < WB * WB; e += 128) {
+    const int r = e >> 5, c = e & 31;
+    D[r][c] = (r < w && c < w && c >= r) ? Sb[(size_t)(j0 + r) * k + j0 + c] : 0.f;
+  }
+  const int c = j0 + w + blockIdx.x * 128 + tid;
+  float x[WB];
+#pragma unroll
+  for (int i = 0; i < WB; ++i) x[i] = (i < w && c < k) ? Sb[(size_t)(j0 + i) * k + c] : 0.f;
+  __syncthreads();
+  if (tid < 32) {
+    const float md = Fb[(size_t)(k - 1) * k];
+    float col[WB];  // lane = column of the block
+#pragma unroll
+    for (int r = 0; r < WB; ++r) col[r] = D[r][lane];
+    bool bad = false;
+#pragma unroll
+    for (int j = 0; j < WB; ++j) {
+      if (j < w) {
+        float p = __shfl_sync(0xffffffffu, col[j], j);
+        if (!(p > 0.f)) {
+          p = fmaxf(md, 1e-30f) * 1e-12f;
+          bad = true;
+        }
+        const float dj = sqrtf(p), inv = 1.0f / dj;
+        col[j] = (lane == j) ? dj : col[j] * inv;
+        if (lane == 0) s_inv[j] = inv;
+#pragma unroll
+        for (int r = j + 1; r < WB; ++r) {
+          const float f = __shfl_sync(0xffffffffu, col[j], r);
+          if (lane >= r) col[r] = fmaf(-f, col[j], col[r]);
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < WB; ++r)
+      if (r <= lane) D[r][lane] = col[r];
+    if (blockIdx.x == 0) {
+#pragma unroll
+      for (int r = 0; r < WB; ++r)
+        if (r <= lane && lane < w) Fb[(size_t)(j0 + r) * k + j0 + lane] = col[r];
+      if (bad && lane == 0) atomicMax(&status[b], (int)TC_ERR_BREAKDOWN);
+    }
+  }
+  __syncthreads();
+  if (c >= k) return;
+#pragma unroll
+  for (int j = 0; j < WB; ++j) {
+    if (j < w) {
+      float v = x[j];
+#pragma unroll
+      for (int m = 0; m < j; ++m) v = fmaf(-D[m][j], x[m], v);
+      x[j] = v * s_inv[j];
+      Fb[(size_t)(j0 + j) * k + c] = x[j];
+    }
+  }
+}
+
+// grid (tiles of 64 x 64 on or above the diagonal of what is left, batch), block 256, 4 x 4 per thread
+__global__ void __launch_bounds__(256) chol_f32_update(float* __restrict__ S, const float* __restrict__ F, int k, int j0,
+                                                      int j1) {
+  __shared__ __align__(16) float fr[WB][64], fc[WB][64];
+  int t = blockIdx.x, tj = 0;  // t -> (ti <= tj): t = tj (tj + 1) / 2 + ti
+  while ((tj + 1) * (tj + 2) / 2 <= t) ++tj;
+  const int ti = t - tj * (tj + 1) / 2;
+  const int r0 = j1 + ti * 64, c0 = j1 + tj * 64, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  float* Sb = S + (size_t)blockIdx.y * k * k;
+  const float* Fb = F + (size_t)blockIdx.y * k * k;
+  for (int e = tid; e < WB * 64; e += 256) {
+    const int m = e >> 6, i = e & 63;
+    fr[m][i] = (r0 + i < k) ? Fb[(size_t)(j0 + m) * k + r0 + i] : 0.f;
+    fc[m][i] = (c0 + i < k) ? Fb[(size_t)(j0 + m) * k + c0 + i] : 0.f;
+  }
+  float acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int r = r0 + 4 * ty + i, c = c0 + 4 * tx + j;
+      acc[i][j] = (r < k && c < k && c >= r) ? Sb[(size_t)r * k + c] : 0.f;
+    }
+  __syncthreads();
+#pragma unroll 8
+  for (int m = 0; m < j1 - j0; ++m) {
+    const float4 a4 = *reinterpret_cast<const float4*>(&fr[m][4 * ty]), b4 = *reinterpret_cast<const float4*>(&fc[m][4 * tx]);
+    const float a[4] = {a4.x, a4.y, a4.z, a4.w}, bb[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(-a[i], bb[j], acc[i][j]);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int r = r0 + 4 * ty + i, c = c0 + 4 * tx + j;
+      if (r < k && c < k && c >= r) Sb[(size_t)r * k + c] = acc[i][j];
+    }
+}
+
+// XT[c][m] = (R^{-1})[m][c], zero for m > c.  grid (ceil(k / 8), batch), block 256: a warp per column,
+// the long columns first.  The row of the factor that the next step needs is read ahead.
+template <int T>  // k <= 32 T
+__global__ void __launch_bounds__(256) chol_f32_inverse(const float* __restrict__ F, float* __restrict__ XT, int k) {
+  extern __shared__ float xs[];  // [8][k]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = blockIdx.y;
+  const int c = k - 1 - (blockIdx.x * 8 + warp);
+  if (c < 0) return;
+  const float* R = F + (size_t)b * k * k;
+  float* x = xs + (size_t)warp * k;
+  float rv[T], dv;
+  auto fetch = [&](int i) {  // entries i + 1 + lane + 32 t <= c of row i, and its diagonal
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+      const int m = i + 1 + lane + 32 * t;
+      rv[t] = (m <= c) ? __ldg(R + (size_t)i * k + m) : 0.f;
+    }
+    dv = __ldg(R + (size_t)i * k + i);
+  };
+  if (lane == 0) x[c] = 1.0f / R[(size_t)c * k + c];
+  __syncwarp();
+  if (c > 0) fetch(c - 1);
+  for (int i = c - 1; i >= 0; --i) {
+    float s = 0.f;
+    const float d = dv;
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+      const int m = i + 1 + lane + 32 * t;
+      if (m <= c) s = fmaf(rv[t], x[m], s);
+    }
+    if (i > 0) fetch(i - 1);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) x[i] = -s / d;
+    __syncwarp();
+  }
+  float* out = XT + ((size_t)b * k + c) * k;
+  for (int m = lane; m < k; m += 32) out[m] = (m <= c) ? x[m] : 0.f;
+}
+
+}  // namespace
+
+void launch_chol_inv_f32(float* S, float* RinvT, float* F, int k, int batch, float shift_rel, int32_t* status,
+                         cudaStream_t st) {
+  Scope scope_(KC_CHOL, st);
+  chol_f32_prepare<<<batch, 256, 0, st>>>(S, F, k, shift_rel);
+  note_launch();
+  for (int j0 = 0; j0 < k; j0 += WB) {
+    const int j1 = j0 + WB < k ? j0 + WB : k, left = k - j1;
+    chol_f32_panel<<<dim3(left > 0 ? (left + 127) / 128 : 1, batch), 128, 0, st>>>(S, F, k, j0, status);
+    note_launch();
+    if (left > 0) {
+      const int nt = (left + 63) / 64;
+      chol_f32_update<<<dim3(nt * (nt + 1) / 2, batch), 256, 0, st>>>(S, F, k, j0, j1);
+      note_launch();
+    }
+  }
+  const size_t smem = (size_t)8 * k * sizeof(float);
+  const dim3 grid((k + 7) / 8, batch);
+  if (k <= 512) chol_f32_inverse<16><<<grid, 256, smem, st>>>(F, RinvT, k);
+  else if (k <= 768) chol_f32_inverse<24><<<grid, 256, smem, st>>>(F, RinvT, k);
+  else chol_f32_inverse<32><<<grid, 256, smem, st>>>(F, RinvT, k);
+  note_launch();
+}
+
 }  // namespace tc

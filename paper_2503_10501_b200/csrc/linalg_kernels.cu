@@ -329,88 +329,6 @@ __global__ void sketch_vec_kernel(const T* __restrict__ O, float* __restrict__ Y
 }
 
 // ==========================================================================================
-// Cholesky factor of S (+ shift) and its inverse.  One block per image.
-//   S [k][k] symmetric in;  RinvT [k][k] out, RinvT[c][m] = (R^{-1})[m][c] for m <= c, else 0,
-//   where R^T R = S + shift_rel * max_i S_ii * I.  Then  Y R^{-1}  has (nearly) orthonormal
-//   columns: one pass of Cholesky-QR.  The shift keeps the factorisation alive when S is
-//   numerically singular; a later unshifted pass removes its effect.
-// The k x k work arrays live in shared memory when they fit, else in global memory.
-// ==========================================================================================
-__global__ void __launch_bounds__(512) chol_inv_kernel(const float* __restrict__ S,
-                                                      float* __restrict__ RinvT,
-                                                      float* __restrict__ Rwork, int k,
-                                                      float shift_rel, int use_smem,
-                                                      int32_t* __restrict__ status) {
-  extern __shared__ float sm[];
-  __shared__ float s_red[16];
-  __shared__ float s_piv;
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const size_t kk = (size_t)k * k;
-  const float* Sb = S + b * kk;
-  float* R = use_smem ? sm : Rwork + b * kk;        // upper triangle used
-  float* XT = use_smem ? sm + kk : RinvT + b * kk;  // XT[c][m]
-  float* out = RinvT + b * kk;
-
-  float md = 0.f;
-  for (int i = tid; i < k; i += 512) md = fmaxf(md, Sb[(size_t)i * k + i]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) md = fmaxf(md, __shfl_xor_sync(0xffffffffu, md, o));
-  if (lane == 0) s_red[warp] = md;
-  __syncthreads();
-  md = s_red[0];
-  for (int w = 1; w < 16; ++w) md = fmaxf(md, s_red[w]);
-  const float shift = shift_rel * md;
-  for (size_t e = tid; e < kk; e += 512) {
-    const int r = (int)(e / k), c = (int)(e % k);
-    float v = Sb[e];
-    if (r == c) v += shift;
-    R[e] = v;
-  }
-  __syncthreads();
-
-  bool bad = false;
-  for (int j = 0; j < k; ++j) {
-    if (tid == 0) {
-      float p = R[(size_t)j * k + j];
-      if (!(p > 0.f)) {
-        p = fmaxf(md, 1e-30f) * 1e-12f;
-        bad = true;
-      }
-      s_piv = sqrtf(p);
-    }
-    __syncthreads();
-    const float dj = s_piv, inv = 1.0f / dj;
-    for (int c = j + tid; c < k; c += 512) R[(size_t)j * k + c] = (c == j) ? dj : R[(size_t)j * k + c] * inv;
-    __syncthreads();
-    for (int r = j + 1 + warp; r < k; r += 16) {
-      const float f = R[(size_t)j * k + r];
-      for (int c = r + lane; c < k; c += 32) R[(size_t)r * k + c] = fmaf(-f, R[(size_t)j * k + c], R[(size_t)r * k + c]);
-    }
-    __syncthreads();
-  }
-  if (tid == 0 && bad) atomicMax(&status[b], (int)TC_ERR_BREAKDOWN);
-
-  // inverse, one warp per column c of R^{-1}:  R x = e_c by back substitution
-  for (int c = warp; c < k; c += 16) {
-    float* x = XT + (size_t)c * k;
-    if (lane == 0) x[c] = 1.0f / R[(size_t)c * k + c];
-    __syncwarp();
-    for (int i = c - 1; i >= 0; --i) {
-      float s = 0.f;
-      for (int m = i + 1 + lane; m <= c; m += 32) s = fmaf(R[(size_t)i * k + m], x[m], s);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) x[i] = -s / R[(size_t)i * k + i];
-      __syncwarp();
-    }
-    for (int m = c + 1 + lane; m < k; m += 32) x[m] = 0.f;
-  }
-  __syncthreads();
-  if (use_smem)
-    for (size_t e = tid; e < kk; e += 512) out[e] = XT[e];
-}
-
-// ==========================================================================================
 // One-sided Jacobi eigen-solver for a symmetric positive semi-definite n x n matrix.
 // One block (16 warps) per image.  W (column-major) starts as the matrix, J as the identity;
 // each pair step rotates columns p, q of both so that the W columns become orthogonal.  At
@@ -612,17 +530,6 @@ static void launch_jacobi(const float* H, int ldh, float* W, float* ZT, float* t
 // orthogonal whatever the spectrum, at a hundred times the time.  Eigenvalues alone need no such care.
 static bool use_tridiag(int n, bool full, bool values_only, float rank_tol) {
   return eig_tridiag_supported(n) && (values_only || rank_tol >= 1e-3f || (!full && n <= 224));
-}
-
-static void launch_chol_inv_simt(const float* S, float* RinvT, float* Rwork, int k, int batch, float shift_rel,
-                                 int32_t* status, cudaStream_t st) {
-  Scope scope_(KC_CHOL, st);
-  const size_t need = 2 * (size_t)k * k * sizeof(float);
-  const int use_smem = need <= SMEM_LIMIT;
-  const size_t smem = use_smem ? need : 0;
-  if (use_smem)
-    cudaFuncSetAttribute((const void*)chol_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  { chol_inv_kernel<<<batch, 512, smem, st>>>(S, RinvT, Rwork, k, shift_rel, use_smem, status); note_launch(); }
 }
 
 // ==========================================================================================
@@ -903,7 +810,7 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
   // one Cholesky-QR pass: dst = src R^{-1},  R^T R = src^T src (+ shift)
   auto cholqr_pass = [&](const float* src, float* dst, float shift_rel) {
     gemm<float, float, true, false>(src, src, Sm, k, k, N, k, k, k, sY, sY, sK, B, st, KC_GEMM_TN, GEMM_SYM);
-    launch_chol_inv_simt(Sm, Rinv, W, k, B, shift_rel, img_status, st);
+    launch_chol_inv_f32(Sm, Rinv, W, k, B, shift_rel, img_status, st);
     gemm<float, float, false, true>(src, Rinv, dst, N, k, k, k, k, k, sY, sK, sY, B, st, KC_GEMM, GEMM_B_UPPER);
   };
   const float kShift = 1e-6f;

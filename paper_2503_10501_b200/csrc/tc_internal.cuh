@@ -191,6 +191,11 @@ size_t chol_panel_floats(int k);
 tc_status launch_chol_inv(float* S, float* RinvT, float* panel, int k, int batch, float shift_rel,
                           int32_t* status, cudaStream_t st);
 
+// RinvT as above for any k up to 1024, by plain float32 multiply-adds in the order of the textbook
+// loops; a pivot that is not positive is replaced and reported.  F: [batch][k][k] scratch.
+void launch_chol_inv_f32(float* S, float* RinvT, float* F, int k, int batch, float shift_rel, int32_t* status,
+                         cudaStream_t st);
+
 // Eigen-decomposition of the symmetric part of H [batch][n][ldh], 3 <= n <= EIG_TRIDIAG_MAX:
 // theta [batch][n] ascending, ZT [batch][n][ldz] with the eigenvectors in its rows (zero rows for
 // eigenvalues under a quarter of the rank cut-off rank_tol^2 theta_max).  scratch: batch *
