@@ -299,9 +299,10 @@ tc_status launch_chol_inv(float* S, float* RinvT, float* panel, int k, int batch
 //   chol_f32_panel     32 rows of the factor: every block factors the diagonal block for itself (one
 //                      warp), then a thread per column substitutes
 //   chol_f32_update    S[r][c] -= sum_m F[m][r] F[m][c] over those 32 rows, 64 x 64 tiles
-//   chol_f32_inverse   a warp per column of the inverse, back substitution
+//   chol_f32_inverse   a warp per four columns of the inverse, back substitution
 // What bounds the first three is 2 k / 32 dependent launches of about 4 us, the last one a chain of k
-// steps of some 300 cycles.  Measured at k = 736, four matrices: CHOLW_MEASURED
+// steps of 400 to 900 cycles.  Measured at k = 736, four matrices: 62 ms (one block per matrix, out of
+// L2) -> 1.0 ms, half of it the inverse.
 // ------------------------------------------------------------------------------------------
 namespace {
 
@@ -347,6 +348,7 @@ __global__ void __launch_bounds__(128) chol_f32_panel(const float* __restrict__ 
     float col[WB];  // lane = column of the block
 #pragma unroll
     for (int r = 0; r < WB; ++r) col[r] = D[r][lane];
+    __syncwarp();
     bool bad = false;
 #pragma unroll
     for (int j = 0; j < WB; ++j) {
@@ -359,16 +361,16 @@ __global__ void __launch_bounds__(128) chol_f32_panel(const float* __restrict__ 
         const float dj = sqrtf(p), inv = 1.0f / dj;
         col[j] = (lane == j) ? dj : col[j] * inv;
         if (lane == 0) s_inv[j] = inv;
+        // row j of the factor goes through shared memory: broadcast reads pipeline, shuffles do not
+        D[j][lane] = col[j];
+        __syncwarp();
 #pragma unroll
         for (int r = j + 1; r < WB; ++r) {
-          const float f = __shfl_sync(0xffffffffu, col[j], r);
+          const float f = D[j][r];
           if (lane >= r) col[r] = fmaf(-f, col[j], col[r]);
         }
       }
     }
-#pragma unroll
-    for (int r = 0; r < WB; ++r)
-      if (r <= lane) D[r][lane] = col[r];
     if (blockIdx.x == 0) {
 #pragma unroll
       for (int r = 0; r < WB; ++r)
@@ -379,13 +381,12 @@ __global__ void __launch_bounds__(128) chol_f32_panel(const float* __restrict__ 
   __syncthreads();
   if (c >= k) return;
 #pragma unroll
-  for (int j = 0; j < WB; ++j) {
-    if (j < w) {
-      float v = x[j];
+  for (int m = 0; m < WB; ++m) {
+    if (m < w) {
+      x[m] *= s_inv[m];
+      Fb[(size_t)(j0 + m) * k + c] = x[m];
 #pragma unroll
-      for (int m = 0; m < j; ++m) v = fmaf(-D[m][j], x[m], v);
-      x[j] = v * s_inv[j];
-      Fb[(size_t)(j0 + j) * k + c] = x[j];
+      for (int j = m + 1; j < WB; ++j) x[j] = fmaf(-D[m][j], x[m], x[j]);
     }
   }
 }
@@ -432,44 +433,83 @@ __global__ void __launch_bounds__(256) chol_f32_update(float* __restrict__ S, co
     }
 }
 
-// XT[c][m] = (R^{-1})[m][c], zero for m > c.  grid (ceil(k / 8), batch), block 256: a warp per column,
-// the long columns first.  The row of the factor that the next step needs is read ahead.
+// XT[c][m] = (R^{-1})[m][c], zero for m > c.  grid (ceil(k / 16), batch), block 128: a warp per four
+// columns c, c - 1, ..., the long columns first.  A row of the factor is read once for the four, two
+// steps ahead; the steps come in phases of 128 whose code has no test that would keep the reads and
+// multiply-adds of a step from overlapping.
 template <int T>  // k <= 32 T
-__global__ void __launch_bounds__(256) chol_f32_inverse(const float* __restrict__ F, float* __restrict__ XT, int k) {
-  extern __shared__ float xs[];  // [8][k]
+__global__ void __launch_bounds__(128) chol_f32_inverse(const float* __restrict__ F, float* __restrict__ XT, int k) {
+  extern __shared__ float xs[];  // [4 warps][4 columns][k]
+  constexpr int Q = T / 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = blockIdx.y;
-  const int c = k - 1 - (blockIdx.x * 8 + warp);
-  if (c < 0) return;
+  const int c0 = k - 1 - 4 * (blockIdx.x * 4 + warp);
+  if (c0 < 0) return;
   const float* R = F + (size_t)b * k * k;
-  float* x = xs + (size_t)warp * k;
-  float rv[T], dv;
-  auto fetch = [&](int i) {  // entries i + 1 + lane + 32 t <= c of row i, and its diagonal
+  float* x = xs + (size_t)warp * 4 * k;
+  float rv[2][T], dv[2];
+  // NQ: groups of 128 entries that a row holds in the current phase
+  auto fetch = [&](int i, int buf, auto nq) {  // entries i + 1 + lane + 32 t <= c0 of row i, and its diagonal
+    if (i < 0) return;
+    const float* row = R + (size_t)i * k + i + 1 + lane;
+    const int left = c0 - i - 1 - lane;  // >= 32 t: entry t exists
 #pragma unroll
-    for (int t = 0; t < T; ++t) {
-      const int m = i + 1 + lane + 32 * t;
-      rv[t] = (m <= c) ? __ldg(R + (size_t)i * k + m) : 0.f;
-    }
-    dv = __ldg(R + (size_t)i * k + i);
+    for (int t = 0; t < 4 * decltype(nq)::value; ++t) rv[buf][t] = (left >= 32 * t) ? __ldg(row + 32 * t) : 0.f;
+    dv[buf] = __ldg(R + (size_t)i * k + i);
   };
-  if (lane == 0) x[c] = 1.0f / R[(size_t)c * k + c];
-  __syncwarp();
-  if (c > 0) fetch(c - 1);
-  for (int i = c - 1; i >= 0; --i) {
-    float s = 0.f;
-    const float d = dv;
+  auto step = [&](int i, int buf, auto nq) {
+    if (i < 0) return;
+    constexpr int NT = 4 * decltype(nq)::value;
+    const int left = c0 - i - 1 - lane;
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int t = 0; t < T; ++t) {
-      const int m = i + 1 + lane + 32 * t;
-      if (m <= c) s = fmaf(rv[t], x[m], s);
+    for (int t = 0; t < NT; ++t) {
+      const float* xt = x + i + 1 + lane + 32 * t;
+#pragma unroll
+      for (int col = 0; col < 4; ++col)
+        if (left - col >= 32 * t) s[col] = fmaf(rv[buf][t], xt[col * k], s[col]);
     }
-    if (i > 0) fetch(i - 1);
+    const float d = dv[buf];
+    // (the next phase begins within two steps: it may need a group more)
+    fetch(i - 2, buf, std::integral_constant<int, (NT / 4 < Q) ? NT / 4 + 1 : Q>{});
+    // the four sums over the lanes, pairwise in the order of a butterfly: lanes 8 col .. get column col
+    {
+      const bool up = (lane & 16) != 0;
+      const float a0 = (up ? s[2] : s[0]) + __shfl_xor_sync(0xffffffffu, up ? s[0] : s[2], 16);
+      const float a1 = (up ? s[3] : s[1]) + __shfl_xor_sync(0xffffffffu, up ? s[1] : s[3], 16);
+      const bool up8 = (lane & 8) != 0;
+      float a = (up8 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, up8 ? a0 : a1, 8);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) x[i] = -s / d;
+      for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      const int col = lane >> 3, c = c0 - col;
+      if ((lane & 7) == 0 && i <= c) x[col * k + i] = (i == c ? 1.0f : -a) / d;
+    }
     __syncwarp();
+  };
+  fetch(c0, 0, std::integral_constant<int, 1>{});
+  fetch(c0 - 1, 1, std::integral_constant<int, 1>{});
+  // steps j = c0 - i in phases of 128
+  auto phase = [&](auto nq) {
+    constexpr int NQ = decltype(nq)::value;
+    if constexpr (NQ <= Q) {
+      for (int j = 128 * (NQ - 1); j < 128 * NQ && j <= c0; j += 2) {
+        step(c0 - j, 0, nq);
+        step(c0 - j - 1, 1, nq);
+      }
+    }
+  };
+  phase(std::integral_constant<int, 1>{});
+  phase(std::integral_constant<int, 2>{});
+  phase(std::integral_constant<int, 3>{});
+  phase(std::integral_constant<int, 4>{});
+  phase(std::integral_constant<int, 5>{});
+  phase(std::integral_constant<int, 6>{});
+  phase(std::integral_constant<int, 7>{});
+  phase(std::integral_constant<int, 8>{});
+  for (int col = 0; col < 4 && c0 - col >= 0; ++col) {
+    const int c = c0 - col;
+    float* out = XT + ((size_t)b * k + c) * k;
+    for (int m = lane; m < k; m += 32) out[m] = (m <= c) ? x[col * k + m] : 0.f;
   }
-  float* out = XT + ((size_t)b * k + c) * k;
-  for (int m = lane; m < k; m += 32) out[m] = (m <= c) ? x[m] : 0.f;
 }
 
 }  // namespace
@@ -489,11 +529,15 @@ void launch_chol_inv_f32(float* S, float* RinvT, float* F, int k, int batch, flo
       note_launch();
     }
   }
-  const size_t smem = (size_t)8 * k * sizeof(float);
-  const dim3 grid((k + 7) / 8, batch);
-  if (k <= 512) chol_f32_inverse<16><<<grid, 256, smem, st>>>(F, RinvT, k);
-  else if (k <= 768) chol_f32_inverse<24><<<grid, 256, smem, st>>>(F, RinvT, k);
-  else chol_f32_inverse<32><<<grid, 256, smem, st>>>(F, RinvT, k);
+  const size_t smem = (size_t)16 * k * sizeof(float);
+  const dim3 grid((k + 15) / 16, batch);
+  auto inverse = [&](auto kernel) {
+    cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kernel<<<grid, 128, smem, st>>>(F, RinvT, k);
+  };
+  if (k <= 512) inverse(chol_f32_inverse<16>);
+  else if (k <= 768) inverse(chol_f32_inverse<24>);
+  else inverse(chol_f32_inverse<32>);
   note_launch();
 }
 
