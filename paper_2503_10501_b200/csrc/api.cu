@@ -60,6 +60,7 @@ tc_status make_dims(const tc_params* p, Dims* out) {
   memset(&D, 0, sizeof(D));
   D.B = p->batch; D.N = p->n_tokens; D.d = p->d_model; D.H = p->n_heads; D.dh = p->head_dim;
   D.T = p->n_query; D.keep = p->keep;
+  D.call_B = D.B;
   if (D.B < 1 || D.N < 1 || D.d < 1 || D.H < 1 || D.dh < 1 || D.T < 1) return TC_ERR_INVALID_ARG;
   if (D.keep < 1 || D.keep > D.N) return TC_ERR_INVALID_ARG;
   if (!(p->lambda >= 0.f && p->lambda <= 1.f)) return TC_ERR_INVALID_ARG;
@@ -220,8 +221,9 @@ struct GroupStreams {
   bool ready = false;
   cudaStream_t s[kMaxGroups];    // a group's sketch -> Cholesky-QR -> eigen-solve chain
   cudaStream_t s2[kMaxGroups];   // its Gram matrix, which the chain needs only from G Q on
+  cudaStream_t attn;             // the attention scores of the whole batch, which are needed last
   cudaEvent_t fork, join[kMaxGroups], gram_done[kMaxGroups];
-  cudaEvent_t attn_done;         // the attention partial sums of the whole batch are written
+  cudaEvent_t attn_done;
 };
 static std::mutex g_groups_mu;
 static GroupStreams g_groups[64];
@@ -238,6 +240,7 @@ static GroupStreams* group_streams() {
       if (cudaEventCreateWithFlags(&g.join[i], cudaEventDisableTiming) != cudaSuccess) return nullptr;
       if (cudaEventCreateWithFlags(&g.gram_done[i], cudaEventDisableTiming) != cudaSuccess) return nullptr;
     }
+    if (cudaStreamCreateWithFlags(&g.attn, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
     if (cudaEventCreateWithFlags(&g.fork, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     if (cudaEventCreateWithFlags(&g.attn_done, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     g.ready = true;
@@ -245,8 +248,8 @@ static GroupStreams* group_streams() {
   return &g;
 }
 
-// score: S partial sums || (Gram -> eigen-solve -> C per image group) -> E
-// A launcher that refuses (tensor map, function attribute) stops the enqueue: the group streams
+// score: S || (Gram || sketch and first pass -> eigen-solve -> C, E) per image group
+// A launcher that refuses (tensor map, function attribute) stops the enqueue: the streams
 // forked so far are joined back, the status words of the images not reached are set, and the
 // caller gets the status.
 // tail: what follows the scores of an image group on that group's stream (images b0 .. b0 + Dg.B),
@@ -261,12 +264,14 @@ static tc_status enqueue_score(const Ctx& c, const void* O, const void* A, float
   int ng = g_n_groups.load();
   if (ng > D.B) ng = D.B;
   std::lock_guard<std::mutex> lk(g_groups_mu);
-  GroupStreams* gs = ng > 1 ? group_streams() : nullptr;
-  if (gs == nullptr) ng = 1;
-  if (ng > 1) cudaEventRecord(gs->fork, c.st);
-  launch_attn_colsum(D, A, (float*)(c.ws + c.P.s_part), c.st);
-  const bool group_tail = (tail != nullptr) && ng > 1;
-  if (group_tail) cudaEventRecord(gs->attn_done, c.st);
+  GroupStreams* gs = group_streams();
+  if (gs == nullptr) return TC_ERR_CUDA;
+  cudaEventRecord(gs->fork, c.st);
+  // the attention scores beside everything else
+  cudaStreamWaitEvent(gs->attn, gs->fork, 0);
+  launch_attn_colsum(D, A, (float*)(c.ws + c.P.s_part), gs->attn);
+  launch_attn_finish(D, (const float*)(c.ws + c.P.s_part), S, gs->attn);
+  cudaEventRecord(gs->attn_done, gs->attn);
   const int base = D.B / ng, extra = D.B % ng;
   int b0 = 0;
   tc_status err = TC_OK;
@@ -285,44 +290,45 @@ static tc_status enqueue_score(const Ctx& c, const void* O, const void* A, float
     if (late) cudaStreamWaitEvent(st, gs->gram_done[g - per_wave], 0);
     Dims Dg = D;
     Dg.B = nb;
-    const char* Og = (const char*)O + (size_t)b0 * D.N * D.d * D.esz;
-    // the sketch and its first Cholesky-QR pass do not read G: with groups, the Gram matrix is
-    // built beside them on a stream of its own and joined in front of the first product with G
-    cudaEvent_t gram_done = nullptr;
-    float* Gg = (float*)(c.ws + c.P.G) + (size_t)b0 * D.N * D.ldn;
-    if (ng > 1 && !D.full) {
+    const size_t o = (size_t)b0 * D.N;
+    const char* Og = (const char*)O + o * D.d * D.esz;
+    float* Gg = (float*)(c.ws + c.P.G) + o * D.ldn;
+    ScoreIo io;
+    io.C = C + o; io.S = S + o; io.E = E + o;
+    io.sigma = sigma ? sigma + (size_t)b0 * q : nullptr;
+    io.rank = rank ? rank + b0 : nullptr;
+    io.status = img_status + b0;
+    io.s_ready = gs->attn_done;
+    // the sketch and its first Cholesky-QR pass do not read G: the Gram matrix is built beside them
+    // on a stream of its own and joined in front of the first product with G
+    if (!D.full) {
       cudaStreamWaitEvent(gs->s2[g], gs->fork, 0);
       if (late) cudaStreamWaitEvent(gs->s2[g], gs->gram_done[g - per_wave], 0);
       err = launch_gram(Dg, Og, Gg, D.ldn, img_status + b0, gs->s2[g]);
       cudaEventRecord(gs->gram_done[g], gs->s2[g]);
-      gram_done = gs->gram_done[g];
+      io.g_ready = gs->gram_done[g];
     } else {
       err = launch_gram(Dg, Og, Gg, D.ldn, img_status + b0, st);
     }
     if (err == TC_OK)
-      err = launch_ics(Dg, c.P, c.ws, b0, Og, C + (size_t)b0 * D.N, sigma ? sigma + (size_t)b0 * q : nullptr,
-                       rank ? rank + b0 : nullptr, img_status + b0, st, false, gram_done);
-    else if (gram_done)
-      cudaStreamWaitEvent(st, gram_done, 0);  // the side stream still joins the group's stream
-    if (group_tail && err == TC_OK) {
-      cudaStreamWaitEvent(st, gs->attn_done, 0);
-      const size_t o = (size_t)b0 * D.N;
-      launch_combine(Dg, (const float*)(c.ws + c.P.s_part) + o * D.chunks, C + o, S + o, E + o, st);
-      (*tail)(Dg, b0, st);
+      err = launch_ics(Dg, c.P, c.ws, b0, Og, io, st);
+    else if (io.g_ready)
+      cudaStreamWaitEvent(st, io.g_ready, 0);  // the side stream still joins the group's stream
+    if (err == TC_OK) {
+      if (D.score_norm == TC_NORM_SUM1) launch_combine(Dg, C + o, S + o, E + o, st);
+      if (tail) (*tail)(Dg, b0, st);
     }
     if (ng > 1) {
       cudaEventRecord(gs->join[g], st);
       cudaStreamWaitEvent(c.st, gs->join[g], 0);
     }
-    if (err != TC_OK) fill_i32(img_status + b0, D.B - b0, (int)err, c.st);
+    if (err != TC_OK) {
+      cudaStreamWaitEvent(c.st, gs->attn_done, 0);
+      fill_i32(img_status + b0, D.B - b0, (int)err, c.st);
+    }
     b0 += nb;
   }
-  if (err != TC_OK) return err;
-  if (!group_tail) {
-    launch_combine(D, (const float*)(c.ws + c.P.s_part), C, S, E, c.st);
-    if (tail) (*tail)(D, 0, c.st);
-  }
-  return TC_OK;
+  return err;
 }
 
 }  // namespace tc
@@ -449,12 +455,14 @@ tc_status tc_stage_status(const tc_params* p, const void* ws, size_t ws_bytes, i
   return TC_OK;
 }
 
-tc_status tc_carve(const tc_params* p, const void* O, const void* A, const void* X, const void* K,
-                   const void* V, void* Xo, void* Ko, void* Vo, int32_t* kept_idx,
-                   int32_t* img_status, void* ws, size_t ws_bytes, void* stream) {
+// call_B: images of the caller's call, of which these are all or a chunk
+static tc_status carve_impl(const tc_params* p, int call_B, const void* O, const void* A, const void* X, const void* K,
+                            const void* V, void* Xo, void* Ko, void* Vo, int32_t* kept_idx,
+                            int32_t* img_status, void* ws, size_t ws_bytes, void* stream) {
   Ctx c;
   tc_status s = open_ctx(p, ws, ws_bytes, stream, &c);
   if (s != TC_OK) return s;
+  c.D.call_B = call_B;
   const Dims& D = c.D;
   if (!O || !A || !X || !Xo || !kept_idx || !img_status) return TC_ERR_INVALID_ARG;
   if (misaligned(O) || misaligned(A) || misaligned(X) || misaligned(Xo)) return TC_ERR_INVALID_ARG;
@@ -508,6 +516,13 @@ tc_status tc_carve(const tc_params* p, const void* O, const void* A, const void*
   s = enqueue_score(c, O, A, E, C, S, nullptr, nullptr, img_status, &tail);
   if (s != TC_OK) return s;
   return check_launch();
+}
+
+tc_status tc_carve(const tc_params* p, const void* O, const void* A, const void* X, const void* K,
+                   const void* V, void* Xo, void* Ko, void* Vo, int32_t* kept_idx,
+                   int32_t* img_status, void* ws, size_t ws_bytes, void* stream) {
+  if (p == nullptr) return TC_ERR_INVALID_ARG;
+  return carve_impl(p, p->batch, O, A, X, K, V, Xo, Ko, Vo, kept_idx, img_status, ws, ws_bytes, stream);
 }
 
 // ---- host-buffer variant: device staging lives at the front of the workspace ---------------
@@ -573,7 +588,7 @@ static HostPlan make_host_plan(const Dims& D, size_t scratch_bytes) {
   };
   const size_t B = D.B, e = D.esz;
   h.O = take(B * D.N * D.d * e);
-  h.A = take(B * D.H * D.T * (size_t)D.N * e);
+  h.A = take(B * D.H * D.T * (size_t)D.N * e + 16);  // (a chunk starts on a 16-byte boundary)
   h.X = take(B * D.N * D.d * e);
   h.K = take(B * D.H * D.N * (size_t)D.dh * e);
   h.V = take(B * D.H * D.N * (size_t)D.dh * e);
@@ -634,7 +649,7 @@ tc_status tc_carve_host(const tc_params* p, const void* O, const void* A, const 
   for (int c = 0; c < nchunk; ++c) {
     const size_t nb = base + (c < extra ? 1 : 0), o = b0;
     ok &= cudaMemcpyAsync(w + h.O + o * iO, (const char*)O + o * iO, nb * iO, cudaMemcpyHostToDevice, cin) == cudaSuccess;
-    ok &= cudaMemcpyAsync(w + h.A + o * iA, (const char*)A + o * iA, nb * iA, cudaMemcpyHostToDevice, cin) == cudaSuccess;
+    ok &= cudaMemcpyAsync(w + h.A + align_up(o * iA, 16), (const char*)A + o * iA, nb * iA, cudaMemcpyHostToDevice, cin) == cudaSuccess;
     ok &= cudaMemcpyAsync(w + h.X + o * iO, (const char*)X + o * iO, nb * iO, cudaMemcpyHostToDevice, cin) == cudaSuccess;
     if (kv) {
       ok &= cudaMemcpyAsync(w + h.K + o * iKV, (const char*)K + o * iKV, nb * iKV, cudaMemcpyHostToDevice, cin) == cudaSuccess;
@@ -650,7 +665,7 @@ tc_status tc_carve_host(const tc_params* p, const void* O, const void* A, const 
     if (nchunk > 1) ok &= cudaStreamWaitEvent(st, hs->in[c], 0) == cudaSuccess;
     tc_params pc = *p;
     pc.batch = (int32_t)nb;
-    s = tc_carve(&pc, w + h.O + o * iO, w + h.A + o * iA, w + h.X + o * iO,
+    s = carve_impl(&pc, D.B, w + h.O + o * iO, w + h.A + align_up(o * iA, 16), w + h.X + o * iO,
                  kv ? w + h.K + o * iKV : nullptr, kv ? w + h.V + o * iKV : nullptr,
                  w + h.Xo + o * iXo, kv ? w + h.Ko + o * iKVo : nullptr,
                  kv ? w + h.Vo + o * iKVo : nullptr, (int32_t*)(w + h.kept) + o * D.keep,
@@ -697,7 +712,7 @@ tc_status tc_matmul_f32x3(const float* A, const float* B, float* C, float* CT, i
   F32x3Result R;
   R.C = C; R.ld = NN; R.stride = (size_t)M * NN;
   R.CT = CT; R.ldT = M; R.strideT = (size_t)M * NN;
-  tc_status s = launch_gemm_f32x3({A, K, (size_t)M * K}, {B, K, (size_t)NN * K}, M, NN, K, batch, R, img_status, st, KC_GEMM);
+  tc_status s = launch_gemm_f32x3({A, K, (size_t)M * K}, {B, K, (size_t)NN * K}, M, NN, K, batch, batch, R, img_status, st, KC_GEMM);
   if (s != TC_OK) return s;
   return check_launch();
 }
@@ -750,7 +765,10 @@ tc_status tc_rank(const tc_params* p, const void* O, const int32_t* idx, int32_t
   }
   s = launch_gram(D, rows, (float*)(w + P.G), D.ldn, img_status, st);
   if (s != TC_OK) return s;
-  s = launch_ics(D, P, w, 0, rows, (float*)(w + P.C), sigma, rank, img_status, st, true);
+  ScoreIo io;
+  io.C = (float*)(w + P.C); io.sigma = sigma; io.rank = rank; io.status = img_status;
+  io.values_only = true;
+  s = launch_ics(D, P, w, 0, rows, io, st);
   if (s != TC_OK) return s;
   return check_launch();
 }

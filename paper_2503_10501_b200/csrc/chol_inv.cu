@@ -237,18 +237,19 @@ void launch_block(const CholArgs& ca, int batch, cudaStream_t st) {
 
 }  // namespace
 
-// Orders above CHOL_BLOCK_MAX go block by block (equal blocks, multiples of 16).  Left of the block
+// Orders above CHOL_BLOCK_MAX go block by block (equal blocks, multiples of 16, up to 160: the widest
+// tile of the product kernel that keeps the cross terms apart).  Left of the block
 // column J that is eliminated, S holds the transposed columns of the inverse so far (from the identity
 // on), right of it what is left of S:
 //   P = S[:, J] L_JJ^{-T}              (block row J of the inverse, transposed, in the rows left of J)
 //   S[:, r] -= P P[r]^T                for the columns r right of J (rows J start from zero)
 static int chol_block(int k) {
-  const int nb = (k + CHOL_BLOCK_MAX - 1) / CHOL_BLOCK_MAX;
+  const int nb = (k + 159) / 160;
   return ((k + nb - 1) / nb + 15) / 16 * 16;
 }
 size_t chol_panel_floats(int k) { return k <= CHOL_BLOCK_MAX ? 0 : (size_t)k * chol_block(k) + 4; }
 
-tc_status launch_chol_inv(float* S, float* RinvT, float* panel, int k, int batch, float shift_rel,
+tc_status launch_chol_inv(float* S, float* RinvT, float* panel, int k, int batch, int of_batch, float shift_rel,
                           int32_t* status, cudaStream_t st) {
   if (k < 1 || (k & 15)) return TC_ERR_UNSUPPORTED;
   const size_t sK = (size_t)k * k;
@@ -277,7 +278,7 @@ tc_status launch_chol_inv(float* S, float* RinvT, float* panel, int k, int batch
     F32x3Result rp;
     rp.C = panel; rp.ld = w; rp.stride = sP;
     rp.CT = RinvT + (size_t)j0 * k; rp.ldT = k; rp.strideT = sK; rp.rows_t = j0;
-    tc_status e = launch_gemm_f32x3({S + j0, k, sK}, {RinvT + (size_t)j0 * (k + 1), k, sK}, k, w, w, batch, rp, status,
+    tc_status e = launch_gemm_f32x3({S + j0, k, sK}, {RinvT + (size_t)j0 * (k + 1), k, sK}, k, w, w, batch, of_batch, rp, status,
                                     st, KC_CHOL);
     if (e != TC_OK) return e;
     if (j1 < k) {
@@ -285,7 +286,7 @@ tc_status launch_chol_inv(float* S, float* RinvT, float* panel, int k, int batch
       rs.C = S + j1; rs.ld = k; rs.stride = sK;
       rs.CT = nullptr; rs.ldT = 0; rs.strideT = 0;
       rs.subtract = true; rs.zero_from = j0; rs.zero_to = j1;
-      e = launch_gemm_f32x3({panel, w, sP}, {panel + (size_t)j1 * w, w, sP}, k, k - j1, w, batch, rs, status, st, KC_CHOL);
+      e = launch_gemm_f32x3({panel, w, sP}, {panel + (size_t)j1 * w, w, sP}, k, k - j1, w, batch, of_batch, rs, status, st, KC_CHOL);
       if (e != TC_OK) return e;
     }
   }

@@ -15,16 +15,23 @@
 //   - warps 8-11 turn a landed slab into its two parts: hi overwrites the value where it lies,
 //     lo goes to the same offset of the stage's second half (the swizzled layout is kept as it
 //     is, so nobody has to know it), then a proxy fence hands both to the tensor core;
-//   - warp 13 (one lane) issues the twelve tcgen05.mma (M = 128, N = NN, K = 8) of the slab into
-//     one of two TMEM accumulators, the small cross terms first, and frees the stage with
-//     tcgen05.commit;
+//   - warp 13 (one lane) issues the twelve tcgen05.mma (M = 128, N = NN, K = 8) of the slab, the
+//     small cross terms into an accumulator of their own (tiles up to 160 columns; three of them fit
+//     TMEM), the others into one of two, and frees the stage with tcgen05.commit;
 //   - warps 0-7 read a finished accumulator back with tcgen05.ld and add it to a float32
 //     register tile: the tensor core adds into its accumulator with truncation, so a fresh
 //     accumulator every DRAIN_SLABS slabs and round-to-nearest adds in registers keep the bias
-//     out.
+//     out.  (The cross terms are 2^-11 of the sum: what is truncated there does not matter.)
+// S CTAs of a cluster share a tile, each with a part of K: at one to sixteen images there are far
+// fewer tiles than SMs, and a tile's K loop is most of a launch.  They exchange their partial tiles
+// through distributed shared memory, each adds up and writes some of the columns.
 // The epilogue writes C row-major and / or transposed, as the consumer needs (the consumer wants
 // K contiguous again).  Every mbarrier wait is bounded; a wait that runs out records an error for
-// the image and the CTA winds down (TMEM is still freed).
+// the image and the CTA winds down (TMEM is still freed, and the cluster's barriers are kept).
+// What bounds the main loop is shared-memory bandwidth: 240 KB per slab of a 128 x 144 tile (operand
+// reads of the twelve MMAs, split, TMA), 1 720 cycles against 940 of tensor work.
+// Measured at one image, k = 160, K = 576 (us for all launches of a carve): 26 -> 19 per Y^T Y and 26 ->
+// 19 per G Q; largest error 1.5e-6 -> 6e-7 of sum |a||b|.
 #include "tc_internal.cuh"
 #include "tcgen05_util.cuh"
 
@@ -42,8 +49,8 @@ constexpr int CONV_WARPS = 4;    // warps 8-11: split of the landed slabs
 constexpr int W_TMA = EPI_WARPS + CONV_WARPS, W_MMA = W_TMA + 1;
 constexpr int THREADS = (W_MMA + 1) * 32;
 constexpr int DRAIN_SLABS = 2;   // slabs accumulated in TMEM before the sum moves to registers
-constexpr uint32_t TMEM_COLS = 512;   // two accumulators of up to 256 columns
-constexpr uint32_t ACC_STRIDE = 256;
+constexpr uint32_t TMEM_COLS = 512;
+constexpr int XROW = 20;         // floats per row of a 16-column chunk in the exchange (padded: no bank is hit twice by a quarter warp)
 
 // a stage holds the A slab (128 rows) and the B slab (NN rows), 128 bytes per row, twice:
 // values / hi parts in its first half, lo parts in its second
@@ -64,6 +71,12 @@ __device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t da, uint64_t
       : "memory");
 }
 
+__device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 struct Out {
   float* plain;    // [batch][M][ld]
   float* plainT;   // [batch][W][ldT]
@@ -75,8 +88,8 @@ struct Out {
   int z0, z1;
 };
 
-// NN: width of C (compile time: it sizes the register tile).
-template <int NN>
+// NN: width of the tile (compile time: it sizes the register tile); S: CTAs that share it.
+template <int NN, int S>
 __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_constant__ CUtensorMap mapA,
                                                            const __grid_constant__ CUtensorMap mapB,
                                                            Out out, int M, int K, int m_tiles, int n_tiles,
@@ -85,6 +98,10 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
   constexpr int NCHUNK = NN / 16;            // 16-column chunks of the accumulator
   constexpr int NCH = (NCHUNK + 1) / 2;      // chunks per thread (two column halves)
   constexpr uint32_t A_B = a_bytes(), HALF = half_bytes(NN), STG = stage_bytes(NN);
+  constexpr bool CROSS = NN <= 160;          // an accumulator for the cross terms
+  constexpr uint32_t ACC_STRIDE = CROSS ? 160 : 256, ACC_X = 2 * ACC_STRIDE;
+  constexpr int LC = (NCHUNK + S - 1) / S;   // chunks of a rank: chunk c belongs to rank c % S
+  static_assert(S == 1 || (uint32_t)(S * LC * BM * XROW * 4) <= STAGES * STG, "exchange buffer");
   // D float32, A and B TF32, both K-major, M = 128, N = NN
   constexpr uint32_t IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(NN >> 3) << 17) |
                              ((uint32_t)(BM >> 4) << 24);
@@ -98,9 +115,11 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
   __shared__ int s_fail;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = blockIdx.x / (m_tiles * n_tiles), tile = blockIdx.x % (m_tiles * n_tiles);
+  const int rank = (S > 1) ? (int)(blockIdx.x % S) : 0, bt = blockIdx.x / S;
+  const int b = bt / (m_tiles * n_tiles), tile = bt % (m_tiles * n_tiles);
   const int mt = tile % m_tiles, n0 = (tile / m_tiles) * NN;
-  const int slabs = (K + BK - 1) / BK;
+  const int all_slabs = (K + BK - 1) / BK, per_rank = (all_slabs + S - 1) / S;
+  const int slab0 = rank * per_rank, slabs = min(all_slabs, slab0 + per_rank) - slab0;   // (at least one: the launcher sees to it)
   const int nchunks = (slabs + DRAIN_SLABS - 1) / DRAIN_SLABS;
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));   // the same place, generic
@@ -144,8 +163,8 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
         }
         const uint32_t full = smem_u32(&bar_full[s]);
         mbar_expect_tx(full, HALF);
-        tma_load_3d(st_hi(s), &mapA, kb * BK, mt * BM, b, full);
-        tma_load_3d(st_hi(s) + A_B, &mapB, kb * BK, n0, b, full);
+        tma_load_3d(st_hi(s), &mapA, (slab0 + kb) * BK, mt * BM, b, full);
+        tma_load_3d(st_hi(s) + A_B, &mapB, (slab0 + kb) * BK, n0, b, full);
       }
     }
   } else if (warp == W_MMA) {
@@ -168,17 +187,19 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
         const uint64_t ah = umma_desc(st_hi(s)), al = umma_desc(st_lo(s));
         const uint64_t bh = umma_desc(st_hi(s) + A_B), bl = umma_desc(st_lo(s) + A_B);
         // 8 floats = 32 bytes further along K inside the swizzled row: +2 in 16-byte units.
-        // The cross terms go first: what the accumulator truncates while they are added is
-        // relative to their own small size.
+        // Without an accumulator of their own the cross terms go first: what is truncated while they
+        // are added is then relative to their own small size.
+        const uint32_t tmem_x = CROSS ? tmem_base + ACC_X : tmem_d;
 #pragma unroll
         for (int k = 0; k < BK / UK; ++k)
-          umma_tf32(tmem_d, al + (uint64_t)(2 * k), bh + (uint64_t)(2 * k), IDESC, (first && k == 0) ? 0u : 1u);
+          umma_tf32(tmem_x, al + (uint64_t)(2 * k), bh + (uint64_t)(2 * k), IDESC,
+                    ((CROSS ? kb == 0 : first) && k == 0) ? 0u : 1u);
 #pragma unroll
         for (int k = 0; k < BK / UK; ++k)
-          umma_tf32(tmem_d, ah + (uint64_t)(2 * k), bl + (uint64_t)(2 * k), IDESC, 1u);
+          umma_tf32(tmem_x, ah + (uint64_t)(2 * k), bl + (uint64_t)(2 * k), IDESC, 1u);
 #pragma unroll
         for (int k = 0; k < BK / UK; ++k)
-          umma_tf32(tmem_d, ah + (uint64_t)(2 * k), bh + (uint64_t)(2 * k), IDESC, 1u);
+          umma_tf32(tmem_d, ah + (uint64_t)(2 * k), bh + (uint64_t)(2 * k), IDESC, (CROSS && first && k == 0) ? 0u : 1u);
         umma_commit(smem_u32(&bar_empty[s]));
         if ((kb % DRAIN_SLABS) == DRAIN_SLABS - 1 || kb == slabs - 1)
           umma_commit(smem_u32(&bar_acc_full[buf]));
@@ -238,15 +259,8 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
     for (int c = 0; c < NCH; ++c)
 #pragma unroll
       for (int j = 0; j < 16; ++j) acc[c][j] = 0.f;
-    bool ok = true;
-    for (int ch = 0; ch < nchunks; ++ch) {
-      const int buf = ch & 1;
-      if (!mbar_wait(smem_u32(&bar_acc_full[buf]), ((uint32_t)ch >> 1) & 1u)) {
-        ok = false;
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)buf * ACC_STRIDE;
+    auto drain = [&](uint32_t col) {
+      const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + col;
       // two loads in flight at a time
 #pragma unroll
       for (int c = 0; c < NCH; c += 2) {
@@ -266,19 +280,31 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
           }
         }
       }
+    };
+    bool ok = true;
+    for (int ch = 0; ch < nchunks; ++ch) {
+      const int buf = ch & 1;
+      if (!mbar_wait(smem_u32(&bar_acc_full[buf]), ((uint32_t)ch >> 1) & 1u)) {
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      drain((uint32_t)buf * ACC_STRIDE);
+      if (CROSS && ch == nchunks - 1) drain(ACC_X);   // (every MMA of the tile has completed)
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0)
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_acc_empty[buf]))
                      : "memory");
     }
+    if (!ok) s_fail = 1;
+    if constexpr (S == 1) {
     // The row-major form leaves through shared memory (the operand ring is free: every MMA that
     // read it has completed): a thread owns a row of the tile, so stores straight from its
     // registers would put every lane into a sector of its own; from the staging tile a warp
     // writes whole rows.  All eight warps come to the barrier whatever their waits returned.
     constexpr int SROW = NN + 4;   // floats per staged row: 16-byte aligned, no bank hit twice by a quarter warp
     float* stg = reinterpret_cast<float*>(smem_gen);
-    if (!ok) s_fail = 1;
     if (out.plain != nullptr) {
       float* srow = stg + (quad * 32 + lane) * SROW;
 #pragma unroll
@@ -313,19 +339,97 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
       }
       const int row = mt * BM + quad * 32 + lane;
       if (row < out.rows_t && out.plainT != nullptr) {
+        float* dst = out.plainT + (size_t)b * out.sT + (size_t)(n0 + half * 16) * out.ldT + row;
+        const size_t ld = out.ldT;
+        const int left = min(NN, out.W - n0);   // columns of the tile that exist
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
-          const int chunk = 2 * c + half;
-          if (chunk >= NCHUNK) continue;
-          float* dst = out.plainT + (size_t)b * out.sT + (size_t)(n0 + chunk * 16) * out.ldT + row;
+          const int c16 = (2 * c + half) * 16;
+          if (c16 + 16 <= left) {
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (n0 + chunk * 16 + j < out.W) dst[(size_t)j * out.ldT] = acc[c][j];
+            for (int j = 0; j < 16; ++j) {
+              *dst = acc[c][j];
+              dst += ld;
+            }
+            dst += 16 * ld;
+          } else if (c16 < left) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              if (c16 + j < left) dst[j * ld] = acc[c][j];
+          }
         }
       }
     } else if (status != nullptr && threadIdx.x == 0) {
       atomicMax(&status[b], (int)TC_ERR_CUDA);
     }
+    } else {
+      // partial tiles to the ranks that own the columns, [source rank][chunk of the owner][row][XROW];
+      // every warp of the cluster comes to both barriers whatever its waits returned
+      float* xb = reinterpret_cast<float*>(smem_gen);
+      const int row = quad * 32 + lane;
+      cluster_sync();   // every rank's MMAs have read its operand ring
+#pragma unroll
+      for (int c = 0; c < NCH; ++c) {
+        const int chunk = 2 * c + half;
+        if (chunk >= NCHUNK) continue;
+        const uint32_t local = smem_u32(xb + ((size_t)(rank * LC + chunk / S) * BM + row) * XROW);
+        uint32_t dst;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(local), "r"(chunk % S));
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst + 16u * j), "f"(acc[c][4 * j]),
+                       "f"(acc[c][4 * j + 1]), "f"(acc[c][4 * j + 2]), "f"(acc[c][4 * j + 3]) : "memory");
+      }
+      cluster_sync();
+      const int grow = mt * BM + row;
+#pragma unroll
+      for (int c = 0; c < (LC + 1) / 2; ++c) {
+        const int lc = 2 * c + half, chunk = lc * S + rank;
+        if (lc >= LC || chunk >= NCHUNK) continue;
+        float* x0 = xb + ((size_t)lc * BM + row) * XROW;
+        float v[16];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) *reinterpret_cast<float4*>(v + 4 * j) = *reinterpret_cast<const float4*>(x0 + 4 * j);
+#pragma unroll
+        for (int t = 1; t < S; ++t)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float4 y = *reinterpret_cast<const float4*>(x0 + (size_t)t * LC * BM * XROW + 4 * j);
+            v[4 * j] += y.x; v[4 * j + 1] += y.y; v[4 * j + 2] += y.z; v[4 * j + 3] += y.w;
+          }
+        if (out.plain != nullptr) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) *reinterpret_cast<float4*>(x0 + 4 * j) = *reinterpret_cast<const float4*>(v + 4 * j);
+        }
+        if (s_fail == 0 && grow < out.rows_t && out.plainT != nullptr) {
+          float* dst = out.plainT + (size_t)b * out.sT + (size_t)(n0 + chunk * 16) * out.ldT + grow;
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            if (n0 + chunk * 16 + j < out.W) dst[(size_t)j * out.ldT] = v[j];
+        }
+      }
+      if (out.plain != nullptr) {
+        asm volatile("bar.sync 2, 256;" ::: "memory");
+        // four lanes per row and chunk: 64 contiguous bytes
+        for (int e = threadIdx.x; e < LC * BM * 4; e += EPI_WARPS * 32) {
+          const int lc = e / (BM * 4), rl = (e >> 2) % BM, v4 = e & 3, chunk = lc * S + rank;
+          const int gr = mt * BM + rl, col = n0 + chunk * 16 + 4 * v4;
+          if (chunk >= NCHUNK || gr >= M || col >= out.W || s_fail != 0) continue;
+          float4 x = *reinterpret_cast<const float4*>(xb + ((size_t)lc * BM + rl) * XROW + 4 * v4);
+          float4* dst = reinterpret_cast<float4*>(out.plain + (size_t)b * out.sC + (size_t)gr * out.ld + col);
+          if (out.sub) {
+            const float4 o = (gr < out.z0 || gr >= out.z1) ? *dst : make_float4(0.f, 0.f, 0.f, 0.f);
+            x = make_float4(o.x - x.x, o.y - x.y, o.z - x.z, o.w - x.w);
+          }
+          *dst = x;
+        }
+      }
+      if (s_fail != 0 && status != nullptr && threadIdx.x == 0) atomicMax(&status[b], (int)TC_ERR_CUDA);
+    }
+  }
+  if (S > 1 && warp >= EPI_WARPS) {   // the other roles' part in the two barriers
+    cluster_sync();
+    cluster_sync();
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -350,29 +454,52 @@ bool encode_operand(CUtensorMap* map, const F32x3Operand& o, int rows, int K, in
              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int NN>
-tc_status launch_nn(const CUtensorMap& mapA, const CUtensorMap& mapB, const Out& out, int M, int K,
-                    int batch, int32_t* status, cudaStream_t st) {
+template <int NN, int S>
+tc_status launch_split(const CUtensorMap& mapA, const CUtensorMap& mapB, const Out& out, int M, int K,
+                       int batch, int32_t* status, cudaStream_t st) {
   constexpr uint32_t smem = (uint32_t)stages_for(NN) * stage_bytes(NN) + 1024;
-  if (cudaFuncSetAttribute((const void*)gemm_f32x3_kernel<NN>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  auto kernel = gemm_f32x3_kernel<NN, S>;
+  if (cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return TC_ERR_CUDA;
   const int m_tiles = (M + BM - 1) / BM, n_tiles = (out.W + NN - 1) / NN;
-  gemm_f32x3_kernel<NN><<<batch * m_tiles * n_tiles, THREADS, smem, st>>>(mapA, mapB, out, M, K, m_tiles,
-                                                                         n_tiles, status);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(batch * m_tiles * n_tiles * S));
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = S;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = S > 1 ? 1 : 0;
+  if (cudaLaunchKernelEx(&cfg, kernel, mapA, mapB, out, M, K, m_tiles, n_tiles, status) != cudaSuccess) return TC_ERR_CUDA;
   note_launch();
   return TC_OK;
+}
+
+template <int NN>
+tc_status launch_nn(const CUtensorMap& mapA, const CUtensorMap& mapB, const Out& out, int M, int K,
+                    int batch, int of_batch, int32_t* status, cudaStream_t st) {
+  // K is split while the tiles of the whole call leave SMs idle, from 12 slabs on (the exchange costs
+  // as much as two of them).  The batch of the call decides, not of this launch: an image's bits then
+  // do not depend on how the call is cut into groups.
+  const int slabs = (K + BK - 1) / BK;
+  const long long tiles = (long long)of_batch * ((M + BM - 1) / BM) * ((out.W + NN - 1) / NN);
+  if (slabs >= 12 && 4 * tiles <= 148) return launch_split<NN, 4>(mapA, mapB, out, M, K, batch, status, st);
+  if (slabs >= 12 && 2 * tiles <= 148) return launch_split<NN, 2>(mapA, mapB, out, M, K, batch, status, st);
+  return launch_split<NN, 1>(mapA, mapB, out, M, K, batch, status, st);
 }
 
 }  // namespace
 
 // C = A B^T; see the declaration.
 tc_status launch_gemm_f32x3(const F32x3Operand& A, const F32x3Operand& B, int M, int W, int K, int batch,
-                            const F32x3Result& R, int32_t* status, cudaStream_t st, int cls) {
+                            int of_batch, const F32x3Result& R, int32_t* status, cudaStream_t st, int cls) {
   // TMA rows and 16-byte stores: whole vectors everywhere
   if (M < 1 || W < 4 || (W & 3) || K < 1 || ((A.ld | B.ld) & 3) || ((A.stride | B.stride) & 3)) return TC_ERR_UNSUPPORTED;
   if (R.C != nullptr && ((R.ld & 3) || (R.stride & 3))) return TC_ERR_UNSUPPORTED;
-  const int n_tiles = (W + 191) / 192;
+  const int n_tiles = W <= 192 ? 1 : (W + 159) / 160;   // (tiles over 160 columns have no accumulator for the cross terms)
   int nn = ((W + n_tiles - 1) / n_tiles + 15) / 16 * 16;
   if (nn < 64) nn = 64;
   CUtensorMap mapA, mapB;
@@ -383,15 +510,15 @@ tc_status launch_gemm_f32x3(const F32x3Operand& A, const F32x3Operand& B, int M,
   out.sub = R.subtract ? 1 : 0; out.z0 = R.zero_from; out.z1 = R.zero_to;
   Scope scope_(cls, st);
   switch (nn) {
-    case 64: return launch_nn<64>(mapA, mapB, out, M, K, batch, status, st);
-    case 80: return launch_nn<80>(mapA, mapB, out, M, K, batch, status, st);
-    case 96: return launch_nn<96>(mapA, mapB, out, M, K, batch, status, st);
-    case 112: return launch_nn<112>(mapA, mapB, out, M, K, batch, status, st);
-    case 128: return launch_nn<128>(mapA, mapB, out, M, K, batch, status, st);
-    case 144: return launch_nn<144>(mapA, mapB, out, M, K, batch, status, st);
-    case 160: return launch_nn<160>(mapA, mapB, out, M, K, batch, status, st);
-    case 176: return launch_nn<176>(mapA, mapB, out, M, K, batch, status, st);
-    case 192: return launch_nn<192>(mapA, mapB, out, M, K, batch, status, st);
+    case 64: return launch_nn<64>(mapA, mapB, out, M, K, batch, of_batch, status, st);
+    case 80: return launch_nn<80>(mapA, mapB, out, M, K, batch, of_batch, status, st);
+    case 96: return launch_nn<96>(mapA, mapB, out, M, K, batch, of_batch, status, st);
+    case 112: return launch_nn<112>(mapA, mapB, out, M, K, batch, of_batch, status, st);
+    case 128: return launch_nn<128>(mapA, mapB, out, M, K, batch, of_batch, status, st);
+    case 144: return launch_nn<144>(mapA, mapB, out, M, K, batch, of_batch, status, st);
+    case 160: return launch_nn<160>(mapA, mapB, out, M, K, batch, of_batch, status, st);
+    case 176: return launch_nn<176>(mapA, mapB, out, M, K, batch, of_batch, status, st);
+    case 192: return launch_nn<192>(mapA, mapB, out, M, K, batch, of_batch, status, st);
     default: return TC_ERR_UNSUPPORTED;
   }
 }

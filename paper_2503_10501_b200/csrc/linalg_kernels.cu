@@ -572,7 +572,8 @@ __global__ void __launch_bounds__(256) ics_kernel(const float* __restrict__ thet
                                                  int32_t* __restrict__ rank_out,
                                                  int32_t* __restrict__ status, int N, int k, int q,
                                                  float rank_tol, int cap,
-                                                 const float* __restrict__ G, int ldg) {
+                                                 const float* __restrict__ G, int ldg,
+                                                 const float* __restrict__ S, float* __restrict__ E, float lambda) {
   // k: vectors in PT (rows ldp floats apart); cap: bound on the rank that the caller gave (0: none):
   // singular values beyond it are reported as zero, and a rank that comes within eight of it as
   // TC_ERR_RANK_CAP.  G (subspace solve only): the Gram matrix, for the energy check below.
@@ -670,8 +671,11 @@ __global__ void __launch_bounds__(256) ics_kernel(const float* __restrict__ thet
   }
   s_part[part][xl] = acc;
   __syncthreads();
-  if (part == 0 && x < N)
-    C[(size_t)b * N + x] = (s_part[0][xl] + s_part[1][xl]) + (s_part[2][xl] + s_part[3][xl]);
+  if (part == 0 && x < N) {
+    const float c = (s_part[0][xl] + s_part[1][xl]) + (s_part[2][xl] + s_part[3][xl]);
+    C[(size_t)b * N + x] = c;
+    if (E != nullptr) E[(size_t)b * N + x] = (1.f - lambda) * c + lambda * S[(size_t)b * N + x];   // Eq. 3-8
+  }
 }
 
 __global__ void fill_i32_kernel(int32_t* p, int n, int v) {
@@ -687,9 +691,9 @@ void fill_i32(int32_t* p, int n, int v, cudaStream_t st) {
 // ==========================================================================================
 // The whole of Eq. 3-5 / 3-6 for a batch, given G in the workspace.
 // ==========================================================================================
-tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void* O, float* C_out,
-                     float* sigma_out, int32_t* rank_out, int32_t* img_status, cudaStream_t st,
-                     bool values_only, cudaEvent_t g_ready) {
+tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void* O, const ScoreIo& io,
+                     cudaStream_t st) {
+  int32_t* img_status = io.status;
   // D.B images starting at image b0 of the workspace arrays; O and the outputs already point at
   // image b0.
   const int B = D.B, N = D.N, k = D.k;
@@ -701,14 +705,16 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
   float* ZT = (float*)(ws + P.ZT) + b0 * sK;
   float* theta = (float*)(ws + P.sigma) + (size_t)b0 * k;
   auto scores = [&](const float* PT, int ldp, const float* Gc) {
+    if (io.s_ready) cudaStreamWaitEvent(st, io.s_ready, 0);
     Scope scope_(KC_ICS, st);
     { ics_kernel<<<dim3((N + 63) / 64, B), 256, 2 * (size_t)k * sizeof(float), st>>>(
-          theta, PT, ldp, C_out, sigma_out, rank_out, img_status, N, k, q, D.rank_tol, cap, Gc, ldn); note_launch(); }
+          theta, PT, ldp, io.C, io.sigma, io.rank, img_status, N, k, q, D.rank_tol, cap, Gc, ldn, io.S,
+          D.score_norm == TC_NORM_NONE ? io.E : nullptr, D.lambda); note_launch(); }
   };
 
   if (D.full) {
-    if (g_ready) cudaStreamWaitEvent(st, g_ready, 0);
-    if (use_tridiag(N, true, values_only, D.rank_tol)) {
+    if (io.g_ready) cudaStreamWaitEvent(st, io.g_ready, 0);
+    if (use_tridiag(N, true, io.values_only, D.rank_tol)) {
       tc_status e = launch_eig_tridiag(G, sG, ldn, N, B, D.rank_tol, theta, ZT, sK, N, W, img_status, st);
       if (e != TC_OK) return e;
     } else {
@@ -755,14 +761,14 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
     const auto small = [&](const float* p) { return F32x3Operand{p, k, sK}; };   // [k][k]
     const F32x3Operand gram{G, ldn, sG};
     auto mm = [&](const F32x3Operand& A_, const F32x3Operand& B_, int M_, int K_, const F32x3Result& R, int cls) {
-      if (err == TC_OK) err = launch_gemm_f32x3(A_, B_, M_, k, K_, B, R, img_status, st, cls);
+      if (err == TC_OK) err = launch_gemm_f32x3(A_, B_, M_, k, K_, B, D.call_B, R, img_status, st, cls);
     };
     const auto tall = [&](float* c, float* ct) { return F32x3Result{c, k, sY, ct, ldn, sT}; };
     const auto square = [&](float* c) { return F32x3Result{c, k, sK, nullptr, 0, 0}; };
     // one Cholesky-QR pass  dst = src R^{-1}  with  R^T R = src^T src + shift
     auto pass = [&](const float* srcR, const float* srcT, float* dstR, float* dstT, float shift_rel) {
       mm(cols(srcT), cols(srcT), k, N, square(Sk), KC_GEMM_TN);
-      if (err == TC_OK) err = launch_chol_inv(Sk, Rinv, Pk, k, B, shift_rel, img_status, st);
+      if (err == TC_OK) err = launch_chol_inv(Sk, Rinv, Pk, k, B, D.call_B, shift_rel, img_status, st);
       mm(rows(srcR), small(Rinv), N, k, tall(dstR, dstT), KC_GEMM);   // (Y R^{-1})[x][c] = Y[x][:] . R^{-T}[c][:]
     };
     // 1. sketch of the column space of O, in both forms
@@ -775,7 +781,7 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
     //    directions under the rank cut-off; the Ritz values above it are unaffected.  The widths of
     //    the package's configurations, chosen close to the rank, stop there; others, which may hold
     //    many directions under the cut-off, take a third so that the values there are right as well.
-    if (g_ready) cudaStreamWaitEvent(st, g_ready, 0);
+    if (io.g_ready) cudaStreamWaitEvent(st, io.g_ready, 0);
     mm(gram, cols(Bt), N, N, tall(Ar, At), KC_GEMM_GQ);
     pass(Ar, At, Br, Bt, 1e-6f);
     if (!((k == 128 || k == 144 || k == 160 || k == 192) && k == D.cap && (N & 3) == 0)) {
@@ -819,7 +825,7 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
   cholqr_pass(Y0, Y1, kShift);
   { float* t = Y0; Y0 = Y1; Y1 = t; }  // Q0 in Y0
   // 3. one multiplication by G sharpens the subspace:  Y1 = G Q0, then orthonormalise
-  if (g_ready) cudaStreamWaitEvent(st, g_ready, 0);
+  if (io.g_ready) cudaStreamWaitEvent(st, io.g_ready, 0);
   gemm<float, float, false, false>(G, Y0, Y1, N, k, N, ldn, k, k, sG, sY, sY, B, st, KC_GEMM_GQ);
   cholqr_pass(Y1, Y2, kShift);
   cholqr_pass(Y2, Y1, kShift);
@@ -827,7 +833,7 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
   // 4. Rayleigh-Ritz:  H = Q1^T G Q1
   gemm<float, float, false, false>(G, Y2, Y1, N, k, N, ldn, k, k, sG, sY, sY, B, st, KC_GEMM_GQ);   // T = G Q1
   gemm<float, float, true, false>(Y2, Y1, Hm, k, k, N, k, k, k, sY, sY, sK, B, st, KC_GEMM_TN);   // H = Q1^T T
-  if (use_tridiag(k, false, values_only, D.rank_tol)) {
+  if (use_tridiag(k, false, io.values_only, D.rank_tol)) {
     tc_status e = launch_eig_tridiag(Hm, sK, k, k, B, D.rank_tol, theta, ZT, sK, k, W, img_status, st);
     if (e != TC_OK) return e;
   } else {

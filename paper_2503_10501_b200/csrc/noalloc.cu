@@ -37,19 +37,6 @@ static tc_status scratch_for_current_device(float** out) {
   return TC_OK;
 }
 
-// S[b][x] = (sum over chunks of part[b][c][x]) / (H T), chunks added in index order.
-__global__ void __launch_bounds__(256) attn_finish_kernel(const float* __restrict__ part,
-                                                         float* __restrict__ S, int N, int chunks,
-                                                         float inv_rows) {
-  const int b = blockIdx.y;
-  const int x = blockIdx.x * 256 + threadIdx.x;
-  if (x >= N) return;
-  const float* pb = part + (size_t)b * chunks * N;
-  float s = 0.f;
-  for (int c = 0; c < chunks; ++c) s += pb[(size_t)c * N + x];
-  S[(size_t)b * N + x] = s * inv_rows;
-}
-
 }  // namespace tc
 
 using namespace tc;
@@ -78,11 +65,6 @@ extern "C" tc_status tc_attn_score_noalloc(const tc_params* p, const void* A, fl
   // Every element of the part of the array this call uses is written by the first kernel before
   // the second reads it, so nothing left over from an earlier call has to be cleared.
   launch_attn_colsum(D, A, scratch, st);
-  {
-    Scope scope_(KC_COMBINE, st);
-    dim3 grid((D.N + 255) / 256, D.B);
-    attn_finish_kernel<<<grid, 256, 0, st>>>(scratch, S, D.N, D.chunks, 1.0f / (float)(D.H * D.T));
-    note_launch();
-  }
+  launch_attn_finish(D, scratch, S, st);
   return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }

@@ -153,8 +153,35 @@ void launch_attn_colsum(const Dims& D, const void* A, float* s_part, cudaStream_
 }
 
 // ------------------------------------------------------------------------------------------
-// Eq. 3-7 second half and Eq. 3-8: S = colsum / (H T);  E = (1 - lambda) C~ + lambda S~.
-// One block per image; all reductions run in a fixed order.
+// Eq. 3-7, second half: S[b][x] = (sum over the chunks of part[b][c][x]) / (H T), chunks added in index
+// order, sixteen loads in flight.  grid (ceil(N / 64), B), block 64.
+// ------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(64) attn_finish_kernel(const float* __restrict__ part, float* __restrict__ S, int N,
+                                                        int chunks, float inv_rows) {
+  const int b = blockIdx.y, x = blockIdx.x * 64 + threadIdx.x;
+  if (x >= N) return;
+  const float* pb = part + (size_t)b * chunks * N + x;
+  float s = 0.f;
+  int c = 0;
+  for (; c + 15 < chunks; c += 16) {
+    float v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) v[u] = pb[(size_t)(c + u) * N];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) s += v[u];
+  }
+  for (; c < chunks; ++c) s += pb[(size_t)c * N];
+  S[(size_t)b * N + x] = s * inv_rows;
+}
+
+void launch_attn_finish(const Dims& D, const float* s_part, float* S, cudaStream_t st) {
+  Scope scope_(KC_COMBINE, st);
+  { attn_finish_kernel<<<dim3((D.N + 63) / 64, D.B), 64, 0, st>>>(s_part, S, D.N, D.chunks, 1.0f / (float)(D.H * D.T)); note_launch(); }
+}
+
+// ------------------------------------------------------------------------------------------
+// Eq. 3-8 on normalised terms (TC_NORM_SUM1): E = (1 - lambda) C / sum(C) + lambda S / sum(S).  (On the
+// raw terms E is formed where C is.)  One block per image; all reductions run in a fixed order.
 // ------------------------------------------------------------------------------------------
 __device__ float block_sum_256(float v, float* sh) {
   const int t = threadIdx.x;
@@ -169,56 +196,27 @@ __device__ float block_sum_256(float v, float* sh) {
   return r;
 }
 
-__global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ part,
-                                                     const float* __restrict__ C,
-                                                     float* __restrict__ S, float* __restrict__ E,
-                                                     int N, int chunks, float inv_rows,
-                                                     float lambda, int sum1) {
+__global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ C, const float* __restrict__ S,
+                                                     float* __restrict__ E, int N, float lambda) {
   __shared__ float sh[256];
-  const int b = blockIdx.x;
-  const float* pb = part + (size_t)b * chunks * N;
+  const size_t o = (size_t)blockIdx.x * N;
   float ls = 0.f, lc = 0.f;
   for (int x = threadIdx.x; x < N; x += 256) {
-    // chunk partials are added in chunk order, eight loads in flight at a time
-    float s = 0.f;
-    int c = 0;
-    for (; c + 7 < chunks; c += 8) {
-      float v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = pb[(size_t)(c + u) * N + x];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) s += v[u];
-    }
-    for (; c < chunks; ++c) s += pb[(size_t)c * N + x];
-    s *= inv_rows;
-    S[(size_t)b * N + x] = s;
-    ls += s;
-    lc += C[(size_t)b * N + x];
+    ls += S[o + x];
+    lc += C[o + x];
   }
-  float cs = 1.f, ss = 1.f;
-  if (sum1) {
-    ss = block_sum_256(ls, sh);
-    cs = block_sum_256(lc, sh);
-    if (!(ss > 0.f)) ss = 1.f;
-    if (!(cs > 0.f)) cs = 1.f;
-  }
-  __syncthreads();
+  float ss = block_sum_256(ls, sh), cs = block_sum_256(lc, sh);
+  if (!(ss > 0.f)) ss = 1.f;
+  if (!(cs > 0.f)) cs = 1.f;
   for (int x = threadIdx.x; x < N; x += 256) {
-    float c = C[(size_t)b * N + x], s = S[(size_t)b * N + x];
-    if (sum1) {
-      c = c / cs;
-      s = s / ss;
-    }
-    E[(size_t)b * N + x] = (1.f - lambda) * c + lambda * s;
+    const float c = C[o + x] / cs, s = S[o + x] / ss;
+    E[o + x] = (1.f - lambda) * c + lambda * s;
   }
 }
 
-void launch_combine(const Dims& D, const float* s_part, const float* C, float* S, float* E,
-                    cudaStream_t st) {
+void launch_combine(const Dims& D, const float* C, const float* S, float* E, cudaStream_t st) {
   Scope scope_(KC_COMBINE, st);
-  const float inv_rows = 1.0f / (float)(D.H * D.T);
-  { combine_kernel<<<D.B, 256, 0, st>>>(s_part, C, S, E, D.N, D.chunks, inv_rows, D.lambda,
-                                      D.score_norm == TC_NORM_SUM1 ? 1 : 0); note_launch(); }
+  { combine_kernel<<<D.B, 256, 0, st>>>(C, S, E, D.N, D.lambda); note_launch(); }
 }
 
 // ------------------------------------------------------------------------------------------

@@ -20,6 +20,7 @@ inline std::atomic<int> g_refuse_encode{0};
 // Counts of Sec. 3.3.1 / Eq. 3-9 plus everything the launchers derive from tc_params.
 struct Dims {
   int B, N, d, H, dh, T;
+  int call_B;     // images of the call (B: of the group at hand)
   int keep, M, P, nA, nB;
   int cap;        // rank_cap as given (0 or >= N: none)
   int k;          // dimension of the decomposition: N for the full solve, else rank_cap, on the tensor
@@ -109,9 +110,10 @@ struct Scope {
 // ---- launchers (each only enqueues on `st`) ---------------------------------------------
 // Eq. 3-7: column means of A over heads and query rows.
 void launch_attn_colsum(const Dims& D, const void* A, float* s_part, cudaStream_t st);
-// Eq. 3-8 (+ the 1/(H T) of Eq. 3-7): S and E from the partial sums and C.
-void launch_combine(const Dims& D, const float* s_part, const float* C, float* S, float* E,
-                    cudaStream_t st);
+// ... and S from them.
+void launch_attn_finish(const Dims& D, const float* s_part, float* S, cudaStream_t st);
+// Eq. 3-8 on normalised terms (score_norm == TC_NORM_SUM1).
+void launch_combine(const Dims& D, const float* C, const float* S, float* E, cudaStream_t st);
 // Stage I prune + Eq. 3-9 split.
 void launch_prune(const Dims& D, const float* E, int32_t* setA, int32_t* setB, cudaStream_t st);
 // Eq. 3-10 best match per Set-B token, from the Gram matrix or from the rows of O.
@@ -162,6 +164,7 @@ tc_status launch_gram(const Dims& D, const void* O, float* G, int ldg, int32_t* 
 // C [batch][M][W] = A B^T on the tensor cores, float32-accurate, for A [batch][M][K] and B [batch][W][K]
 // with the contraction index contiguous; W, pitches and strides (in floats) multiples of four, bases
 // 16-byte aligned.  C and / or its transpose CT [batch][W][M] are written (either may be null).
+// of_batch: images of the whole call that these are a part of.
 struct F32x3Operand {
   const float* p;
   int ld;          // floats between rows
@@ -179,16 +182,16 @@ struct F32x3Result {
   int zero_from = 0, zero_to = 0;
 };
 tc_status launch_gemm_f32x3(const F32x3Operand& A, const F32x3Operand& B, int M, int W, int K, int batch,
-                            const F32x3Result& R, int32_t* status, cudaStream_t st, int cls);
+                            int of_batch, const F32x3Result& R, int32_t* status, cudaStream_t st, int cls);
 
 // RinvT [batch][k][k] = L^{-1} (zero above the diagonal) with L L^T = S + shift_rel max_i S_ii I, for
 // S [batch][k][k] symmetric (overwritten), k a multiple of 16.  A pivot well below zero (or no number)
 // is reported as TC_ERR_BREAKDOWN.  Above CHOL_BLOCK_MAX the factorisation is blocked and needs the
 // panel [batch][chol_panel_floats(k)].
 constexpr int CHOL_BLOCK_MAX = 192;
-constexpr int TCP_MAX = 192;  // widest subspace whose products run on the tensor cores
+constexpr int TCP_MAX = 640;  // widest subspace whose products run on the tensor cores
 size_t chol_panel_floats(int k);
-tc_status launch_chol_inv(float* S, float* RinvT, float* panel, int k, int batch, float shift_rel,
+tc_status launch_chol_inv(float* S, float* RinvT, float* panel, int k, int batch, int of_batch, float shift_rel,
                           int32_t* status, cudaStream_t st);
 
 // RinvT as above for any k up to 1024, by plain float32 multiply-adds in the order of the textbook
@@ -209,12 +212,20 @@ tc_status launch_eig_tridiag(const float* H, size_t sH, int ldh, int n, int batc
 // bytes per image of the work array of either eigen-solver (the Jacobi work matrix is k x k)
 inline size_t jacobi_work_bytes(int k) { return align_up(eig_tridiag_scratch_bytes(k), 256); }
 
-// Eigen-decomposition of G and Eq. 3-6:  C, theta (unsorted), then sorted sigma / rank.
-// g_ready: optional event after which G is complete when it is built on another stream (the
-// subspace solve waits for it in front of its first product with G).
-// values_only: the caller reads no eigenvectors (C_out), only sigma and the rank.
-tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void* O, float* C_out,
-                     float* sigma_out, int32_t* rank_out, int32_t* img_status, cudaStream_t st,
-                     bool values_only = false, cudaEvent_t g_ready = nullptr);
+// Eigen-decomposition of G and Eq. 3-6:  C, theta (unsorted), then sorted sigma / rank; on the raw
+// terms (score_norm == TC_NORM_NONE) Eq. 3-8 as well.  Everything points at image b0 of the batch.
+struct ScoreIo {
+  float* C;                       // out
+  const float* S = nullptr;       // Eq. 3-7, for E
+  float* E = nullptr;             // out, may be null
+  float* sigma = nullptr;         // out, may be null
+  int32_t* rank = nullptr;        // out, may be null
+  int32_t* status;
+  bool values_only = false;       // the caller reads no eigenvectors (C), only sigma and the rank
+  cudaEvent_t g_ready = nullptr;  // after it G is complete, where it is built on another stream
+  cudaEvent_t s_ready = nullptr;  // after it S is
+};
+tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void* O, const ScoreIo& io,
+                     cudaStream_t st);
 
 }  // namespace tc

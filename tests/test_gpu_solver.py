@@ -44,7 +44,7 @@ def test_full_solve_of_every_layout(N):
 # subspaces: widths that no product tile fills, around one and several Cholesky blocks and the width the
 # float32 chain takes over at; token counts that are no multiple of four; a bound that leaves no
 # subspace once it is rounded up
-@pytest.mark.parametrize("N,rank_cap", [(97, 30), (131, 47), (203, 64), (330, 100), (333, 177), (401, 193), (450, 209),
+@pytest.mark.parametrize("N,rank_cap", [(97, 30), (131, 47), (203, 64), (330, 100), (333, 177), (401, 193), (450, 209), (460, 224), (520, 304),
                                         (601, 385), (801, 577), (900, 640), (902, 641), (120, 111), (2881, 150)])
 def test_subspace_of_every_width(N, rank_cap):
     _check(N, 1000, max(8, min(rank_cap - 16, rank_cap * 3 // 4, 200)), rank_cap, seed=N, noise=1e-3)
