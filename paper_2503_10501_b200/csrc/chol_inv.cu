@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(CW * 32, 1) chol_inv_reg_kernel(const CholArgs
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = blockIdx.x;
   const int n = ca.n;
   float* S = ca.S + (size_t)b * ca.sS;
+  pdl_wait();
   auto row_of = [&](int i) { return 16 * (i >> 1) + 2 * warp + (i & 1); };
 
   f2 B[RW][NP];
@@ -202,6 +203,7 @@ __global__ void __launch_bounds__(CW * 32, 1) chol_inv_reg_kernel(const CholArgs
   phase(std::integral_constant<int, 4>{});
   phase(std::integral_constant<int, 5>{});
   __syncthreads();
+  pdl_trigger();
   if (threadIdx.x == 0 && s_bad) atomicMax(&ca.status[b], (int)TC_ERR_BREAKDOWN);
   float* R = ca.R + (size_t)b * ca.sR;
 #pragma unroll
@@ -222,7 +224,7 @@ __global__ void __launch_bounds__(CW * 32, 1) chol_inv_reg_kernel(const CholArgs
 
 template <int NP, int RW>
 void run(const CholArgs& ca, int batch, cudaStream_t st) {
-  chol_inv_reg_kernel<NP, RW><<<batch, CW * 32, 0, st>>>(ca);
+  launch_pdl(chol_inv_reg_kernel<NP, RW>, dim3(batch), dim3(CW * 32), 0, st, 0, ca);
   note_launch();
 }
 
@@ -312,6 +314,8 @@ constexpr int WB = 32;  // rows per step
 __global__ void __launch_bounds__(256) chol_f32_prepare(float* __restrict__ S, float* __restrict__ F, int k,
                                                        float shift_rel) {
   __shared__ float s_red[8];
+  pdl_wait();
+  pdl_trigger();
   float* Sb = S + (size_t)blockIdx.x * k * k;
   float md = 0.f;
   for (int i = threadIdx.x; i < k; i += 256) md = fmaxf(md, Sb[(size_t)i * (k + 1)]);
@@ -333,6 +337,8 @@ __global__ void __launch_bounds__(128) chol_f32_panel(const float* __restrict__ 
   __shared__ float s_inv[WB];
   const int tid = threadIdx.x, lane = tid & 31, b = blockIdx.y;
   const int w = min(WB, k - j0);
+  pdl_wait();
+  pdl_trigger();
   const float* Sb = S + (size_t)b * k * k;
   float* Fb = F + (size_t)b * k * k;
   for (int e = tid; e < WB * WB; e += 128) {
@@ -398,6 +404,8 @@ __global__ void __launch_bounds__(256) chol_f32_update(float* __restrict__ S, co
   __shared__ __align__(16) float fr[WB][64], fc[WB][64];
   int t = blockIdx.x, tj = 0;  // t -> (ti <= tj): t = tj (tj + 1) / 2 + ti
   while ((tj + 1) * (tj + 2) / 2 <= t) ++tj;
+  pdl_wait();
+  pdl_trigger();
   const int ti = t - tj * (tj + 1) / 2;
   const int r0 = j1 + ti * 64, c0 = j1 + tj * 64, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   float* Sb = S + (size_t)blockIdx.y * k * k;
@@ -444,6 +452,8 @@ __global__ void __launch_bounds__(128) chol_f32_inverse(const float* __restrict_
   constexpr int Q = T / 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = blockIdx.y;
   const int c0 = k - 1 - 4 * (blockIdx.x * 4 + warp);
+  pdl_wait();
+  pdl_trigger();
   if (c0 < 0) return;
   const float* R = F + (size_t)b * k * k;
   float* x = xs + (size_t)warp * 4 * k;
@@ -518,15 +528,15 @@ __global__ void __launch_bounds__(128) chol_f32_inverse(const float* __restrict_
 void launch_chol_inv_f32(float* S, float* RinvT, float* F, int k, int batch, float shift_rel, int32_t* status,
                          cudaStream_t st) {
   Scope scope_(KC_CHOL, st);
-  chol_f32_prepare<<<batch, 256, 0, st>>>(S, F, k, shift_rel);
+  launch_pdl(chol_f32_prepare, dim3(batch), dim3(256), 0, st, 0, S, F, k, shift_rel);
   note_launch();
   for (int j0 = 0; j0 < k; j0 += WB) {
     const int j1 = j0 + WB < k ? j0 + WB : k, left = k - j1;
-    chol_f32_panel<<<dim3(left > 0 ? (left + 127) / 128 : 1, batch), 128, 0, st>>>(S, F, k, j0, status);
+    launch_pdl(chol_f32_panel, dim3(left > 0 ? (left + 127) / 128 : 1, batch), dim3(128), 0, st, 0, S, F, k, j0, status);
     note_launch();
     if (left > 0) {
       const int nt = (left + 63) / 64;
-      chol_f32_update<<<dim3(nt * (nt + 1) / 2, batch), 256, 0, st>>>(S, F, k, j0, j1);
+      launch_pdl(chol_f32_update, dim3(nt * (nt + 1) / 2, batch), dim3(256), 0, st, 0, S, F, k, j0, j1);
       note_launch();
     }
   }
@@ -534,7 +544,7 @@ void launch_chol_inv_f32(float* S, float* RinvT, float* F, int k, int batch, flo
   const dim3 grid((k + 15) / 16, batch);
   auto inverse = [&](auto kernel) {
     cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kernel<<<grid, 128, smem, st>>>(F, RinvT, k);
+    launch_pdl(kernel, grid, dim3(128), smem, st, 0, F, RinvT, k);
   };
   if (k <= 512) inverse(chol_f32_inverse<16>);
   else if (k <= 768) inverse(chol_f32_inverse<24>);

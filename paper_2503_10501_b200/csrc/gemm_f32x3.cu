@@ -126,6 +126,10 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
   auto st_hi = [&](int s) { return smem_base + (uint32_t)s * STG; };
   auto st_lo = [&](int s) { return smem_base + (uint32_t)s * STG + HALF; };
 
+  if (threadIdx.x == 32 * W_TMA) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&mapA) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&mapB) : "memory");
+  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(smem_u32(&bar_full[s]), 1);
@@ -150,6 +154,7 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = s_tmem;
+  pdl_wait();
 
   if (warp == W_TMA) {
     // ---- TMA producer ----
@@ -297,6 +302,7 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_acc_empty[buf]))
                      : "memory");
     }
+    pdl_trigger();
     if (!ok) s_fail = 1;
     if constexpr (S == 1) {
     // The row-major form leaves through shared memory (the operand ring is free: every MMA that
@@ -462,18 +468,9 @@ tc_status launch_split(const CUtensorMap& mapA, const CUtensorMap& mapB, const O
   if (cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return TC_ERR_CUDA;
   const int m_tiles = (M + BM - 1) / BM, n_tiles = (out.W + NN - 1) / NN;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(batch * m_tiles * n_tiles * S));
-  cfg.blockDim = dim3(THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = S;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = S > 1 ? 1 : 0;
-  if (cudaLaunchKernelEx(&cfg, kernel, mapA, mapB, out, M, K, m_tiles, n_tiles, status) != cudaSuccess) return TC_ERR_CUDA;
+  if (launch_pdl(kernel, dim3((unsigned)(batch * m_tiles * n_tiles * S)), dim3(THREADS), smem, st, S, mapA, mapB, out, M, K,
+                 m_tiles, n_tiles, status) != cudaSuccess)
+    return TC_ERR_CUDA;
   note_launch();
   return TC_OK;
 }

@@ -44,6 +44,8 @@ __global__ void __launch_bounds__(256) gemm_kernel(const TA* __restrict__ A,
   __shared__ __align__(16) float As[BK][BM + 4];
   __shared__ __align__(16) float Bs[BK][BN + 4];
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  pdl_wait();
+  pdl_trigger();
   if ((flags & GEMM_SYM) && n0 + BN <= m0) return;  // strictly below the diagonal
   A += (size_t)blockIdx.z * sA;
   B += (size_t)blockIdx.z * sB;
@@ -237,7 +239,7 @@ static void gemm_launch(const TA* A, const TB* B, float* C, int M, int N, int K,
                         int ldc, size_t sA, size_t sB, size_t sC, int batch, cudaStream_t st,
                         int flags) {
   dim3 grid((N + 16 * CN - 1) / (16 * CN), (M + 64 * RM - 1) / (64 * RM), batch);
-  { gemm_kernel<TA, TB, TRA, TRB, RM, CN><<<grid, 256, 0, st>>>(A, B, C, M, N, K, lda, ldb, ldc, sA, sB, sC, flags); note_launch(); }
+  { launch_pdl(gemm_kernel<TA, TB, TRA, TRB, RM, CN>, grid, dim3(256), 0, st, 0, A, B, C, M, N, K, lda, ldb, ldc, sA, sB, sC, flags); note_launch(); }
 }
 
 template <typename TA, typename TB, bool TRA, bool TRB>
@@ -280,6 +282,8 @@ __device__ inline float hash_sign(uint32_t c) {
 template <typename T>
 __global__ void sketch_kernel(const T* __restrict__ O, float* __restrict__ Y, int N, int d, int k) {
   const int x = blockIdx.x, b = blockIdx.y, j = threadIdx.x;
+  pdl_wait();
+  pdl_trigger();
   if (j >= k) return;
   const T* row = O + ((size_t)b * N + x) * d;
   float acc = 0.f;
@@ -297,6 +301,8 @@ __global__ void sketch_vec_kernel(const T* __restrict__ O, float* __restrict__ Y
   const int b = blockIdx.y, x = blockIdx.x * blockDim.y + ty;
   for (int c = ty * kg + tx; c < d; c += kg * blockDim.y) sgn[c] = hash_sign((uint32_t)c);
   __syncthreads();
+  pdl_wait();
+  pdl_trigger();
   if (x >= N) return;
   const uint4* row = reinterpret_cast<const uint4*>(O + ((size_t)b * N + x) * d);
   const int ng = d / L;
@@ -541,6 +547,8 @@ __global__ void __launch_bounds__(256) transpose_kernel(const float* __restrict_
   __shared__ float t[32][33];
   const int b = blockIdx.z, r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;
+  pdl_wait();
+  pdl_trigger();
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int r = r0 + ty + 8 * i, c = c0 + tx;
@@ -557,7 +565,7 @@ __global__ void __launch_bounds__(256) transpose_kernel(const float* __restrict_
 static void launch_transpose(const float* in, int R, int C, int batch, float* out, int ldo, cudaStream_t st, int cls) {
   Scope scope_(cls, st);
   dim3 grid((C + 31) / 32, (R + 31) / 32, batch), block(32, 8);
-  { transpose_kernel<<<grid, block, 0, st>>>(in, R, C, out, ldo); note_launch(); }
+  { launch_pdl(transpose_kernel, grid, block, 0, st, 0, in, R, C, out, ldo); note_launch(); }
 }
 
 // ==========================================================================================
@@ -587,6 +595,8 @@ __global__ void __launch_bounds__(256) ics_kernel(const float* __restrict__ thet
   __shared__ float s_part[4][64];
   const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool writer = blockIdx.x == 0;
+  pdl_wait();
+  pdl_trigger();
   float mx = 0.f;
   for (int p = tid; p < k; p += 256) {
     const float s = sqrtf(fmaxf(theta[(size_t)b * k + p], 0.f));
@@ -707,7 +717,7 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
   auto scores = [&](const float* PT, int ldp, const float* Gc) {
     if (io.s_ready) cudaStreamWaitEvent(st, io.s_ready, 0);
     Scope scope_(KC_ICS, st);
-    { ics_kernel<<<dim3((N + 63) / 64, B), 256, 2 * (size_t)k * sizeof(float), st>>>(
+    { launch_pdl(ics_kernel, dim3((N + 63) / 64, B), dim3(256), 2 * (size_t)k * sizeof(float), st, 0,
           theta, PT, ldp, io.C, io.sigma, io.rank, img_status, N, k, q, D.rank_tol, cap, Gc, ldn, io.S,
           D.score_norm == TC_NORM_NONE ? io.E : nullptr, D.lambda); note_launch(); }
   };
@@ -732,13 +742,13 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
       dim3 block(kg, rows), grid((N + rows - 1) / rows, B);
       const size_t smem = (size_t)D.d * sizeof(float);
       TC_WITH_STORAGE_TYPE(D,
-        sketch_vec_kernel<T, 16 / sizeof(T)><<<grid, block, smem, st>>>((const T*)O, Y0, N, D.d, k);
+        launch_pdl(sketch_vec_kernel<T, 16 / sizeof(T)>, grid, block, smem, st, 0, (const T*)O, Y0, N, D.d, k);
         note_launch(););
     } else {
       dim3 grid(N, B);
       const int threads = (k + 31) / 32 * 32;
       TC_WITH_STORAGE_TYPE(D,
-        sketch_kernel<T><<<grid, threads, 0, st>>>((const T*)O, Y0, N, D.d, k);
+        launch_pdl(sketch_kernel<T>, grid, dim3(threads), 0, st, 0, (const T*)O, Y0, N, D.d, k);
         note_launch(););
     }
   };

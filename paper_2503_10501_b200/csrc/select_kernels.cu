@@ -87,6 +87,8 @@ __global__ void __launch_bounds__(SEL_THREADS) prune_kernel(const float* __restr
   __shared__ uint32_t sh_u[2];
   __shared__ int sh_scan[9];
   const int b = blockIdx.x;
+  pdl_wait();
+  pdl_trigger();
   for (int i = threadIdx.x; i < N; i += SEL_THREADS) keys[i] = orderable(E[(size_t)b * N + i]);
   __syncthreads();
   uint32_t thrP, thrA = 0xffffffffu;
@@ -129,7 +131,7 @@ __global__ void __launch_bounds__(SEL_THREADS) prune_kernel(const float* __restr
 
 void launch_prune(const Dims& D, const float* E, int32_t* setA, int32_t* setB, cudaStream_t st) {
   Scope scope_(KC_PRUNE, st);
-  { prune_kernel<<<D.B, SEL_THREADS, (size_t)D.N * sizeof(uint32_t), st>>>(E, setA, setB, D.N, D.P,
+  { launch_pdl(prune_kernel, dim3(D.B), dim3(SEL_THREADS), (size_t)D.N * sizeof(uint32_t), st, 0, E, setA, setB, D.N, D.P,
                                                                        D.nA, D.nB); note_launch(); }
 }
 
@@ -161,6 +163,8 @@ __global__ void __launch_bounds__(128) match_gram_kernel(const float* __restrict
   const int b = blockIdx.y;
   const int jb = blockIdx.x * 4 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  pdl_wait();
+  pdl_trigger();
   if (jb >= nB) return;
   const float* Gb = G + (size_t)b * N * ldg;
   const int tb = setB[(size_t)b * nB + jb];
@@ -201,7 +205,7 @@ void launch_match_gram(const Dims& D, const float* G, int ldg, const int32_t* se
   Scope scope_(KC_MATCH, st);
   if (D.nB == 0 || D.nA == 0) return;
   dim3 grid((D.nB + 3) / 4, D.B);
-  { match_gram_kernel<<<grid, 128, 0, st>>>(G, ldg, setA, setB, best_val, best_dst, D.N, D.nA, D.nB, status); note_launch(); }
+  { launch_pdl(match_gram_kernel, grid, dim3(128), 0, st, 0, G, ldg, setA, setB, best_val, best_dst, D.N, D.nA, D.nB, status); note_launch(); }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -222,6 +226,8 @@ __global__ void __launch_bounds__(256) match_rows_kernel(const T* __restrict__ O
   __shared__ float s_nb;
   const int b = blockIdx.y, jb = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  pdl_wait();
+  pdl_trigger();
   const int tb = setB[(size_t)b * nB + jb];
   const T* Ob = O + (size_t)b * N * d;
   // a token number outside [0, N) in a caller's list is reported and never used as an address
@@ -293,7 +299,7 @@ void launch_match_rows(const Dims& D, const void* O, const int32_t* setA, const 
   dim3 grid(D.nB, D.B);
   size_t smem = (size_t)D.d * sizeof(float);
   TC_WITH_STORAGE_TYPE(D,
-    match_rows_kernel<T><<<grid, 256, smem, st>>>((const T*)O, setA, setB, best_val, best_dst, D.N,
+    launch_pdl(match_rows_kernel<T>, grid, dim3(256), smem, st, 0, (const T*)O, setA, setB, best_val, best_dst, D.N,
                                                   D.d, D.nA, D.nB, status);
     note_launch(););
 }
@@ -304,7 +310,7 @@ void launch_match_rows_f32(const Dims& D, const float* F, int f, const int32_t* 
   Scope scope_(KC_MATCH, st);
   if (D.nB == 0 || D.nA == 0) return;
   dim3 grid(D.nB, D.B);
-  { match_rows_kernel<float><<<grid, 256, (size_t)f * sizeof(float), st>>>(F, setA, setB, best_val, best_dst,
+  { launch_pdl(match_rows_kernel<float>, grid, dim3(256), (size_t)f * sizeof(float), st, 0, F, setA, setB, best_val, best_dst,
                                                                          D.N, f, D.nA, D.nB, status); note_launch(); }
 }
 
@@ -325,6 +331,8 @@ __global__ void __launch_bounds__(SEL_THREADS) merge_select_kernel(
   __shared__ uint32_t sh_u[2];
   __shared__ int sh_scan[9];
   const int b = blockIdx.x;
+  pdl_wait();
+  pdl_trigger();
   // Token numbers come from the caller's lists: one outside [0, N) is reported in the image's
   // status and never used as an address (the kept list then ends in -1 entries).
   auto valid = [&](int t) {
@@ -390,7 +398,7 @@ void launch_merge_select(const Dims& D, const int32_t* setA, const int32_t* setB
                          int32_t* mdst, int32_t* kept, int32_t* status, cudaStream_t st) {
   Scope scope_(KC_MSEL, st);
   size_t smem = (size_t)(D.nB + D.N) * sizeof(uint32_t);
-  { merge_select_kernel<<<D.B, SEL_THREADS, smem, st>>>(setA, setB, best_val, best_dst, msrc, mdst,
+  { launch_pdl(merge_select_kernel, dim3(D.B), dim3(SEL_THREADS), smem, st, 0, setA, setB, best_val, best_dst, msrc, mdst,
                                                      kept, D.N, D.nA, D.nB, D.M, D.keep, status); note_launch(); }
 }
 

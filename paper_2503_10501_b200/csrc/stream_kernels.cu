@@ -159,6 +159,7 @@ void launch_attn_colsum(const Dims& D, const void* A, float* s_part, cudaStream_
 __global__ void __launch_bounds__(64) attn_finish_kernel(const float* __restrict__ part, float* __restrict__ S, int N,
                                                         int chunks, float inv_rows) {
   const int b = blockIdx.y, x = blockIdx.x * 64 + threadIdx.x;
+  pdl_wait();
   if (x >= N) return;
   const float* pb = part + (size_t)b * chunks * N + x;
   float s = 0.f;
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(64) attn_finish_kernel(const float* __restrict
 
 void launch_attn_finish(const Dims& D, const float* s_part, float* S, cudaStream_t st) {
   Scope scope_(KC_COMBINE, st);
-  { attn_finish_kernel<<<dim3((D.N + 63) / 64, D.B), 64, 0, st>>>(s_part, S, D.N, D.chunks, 1.0f / (float)(D.H * D.T)); note_launch(); }
+  { launch_pdl(attn_finish_kernel, dim3((D.N + 63) / 64, D.B), dim3(64), 0, st, 0, s_part, S, D.N, D.chunks, 1.0f / (float)(D.H * D.T)); note_launch(); }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -200,6 +201,8 @@ __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ 
                                                      float* __restrict__ E, int N, float lambda) {
   __shared__ float sh[256];
   const size_t o = (size_t)blockIdx.x * N;
+  pdl_wait();
+  pdl_trigger();
   float ls = 0.f, lc = 0.f;
   for (int x = threadIdx.x; x < N; x += 256) {
     ls += S[o + x];
@@ -216,7 +219,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ 
 
 void launch_combine(const Dims& D, const float* C, const float* S, float* E, cudaStream_t st) {
   Scope scope_(KC_COMBINE, st);
-  { combine_kernel<<<D.B, 256, 0, st>>>(C, S, E, D.N, D.lambda); note_launch(); }
+  { launch_pdl(combine_kernel, dim3(D.B), dim3(256), 0, st, 0, C, S, E, D.N, D.lambda); note_launch(); }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -284,6 +287,7 @@ __global__ void __launch_bounds__(256) compact_kernel(
   __shared__ int s_weighted;
   constexpr int L = Vec16<T>::L;
   const int b = blockIdx.y, j = blockIdx.x;
+  pdl_wait();
   const int a = kept[(size_t)b * keep + j];
   // The lists may come from the caller: a token number outside [0, N) is reported in the
   // image's status and never used as an address.  A bad kept entry gives a row of zeros, a bad
@@ -369,7 +373,7 @@ void launch_compact(const Dims& D, const void* X, const void* K, const void* V,
   dim3 grid(D.keep, D.B);
   size_t smem = (size_t)max(D.M, 1) * sizeof(int) + (size_t)(D.M + 2) * sizeof(float);
   TC_WITH_STORAGE_TYPE(D,
-    compact_kernel<T><<<grid, 256, smem, st>>>((const T*)X, (const T*)K, (const T*)V, kept, msrc, mdst,
+    launch_pdl(compact_kernel<T>, grid, dim3(256), smem, st, 0, (const T*)X, (const T*)K, (const T*)V, kept, msrc, mdst,
                                                (T*)Xo, (T*)Ko, (T*)Vo, D.N, D.d, D.H, D.dh, D.keep,
                                                D.M, E, status);
     note_launch(););
@@ -384,6 +388,8 @@ __global__ void mean_heads_kernel(const T* __restrict__ K, float* __restrict__ K
                                   int dh) {
   const int x = blockIdx.x, b = blockIdx.y;
   const float inv = 1.0f / (float)H;
+  pdl_wait();
+  pdl_trigger();
   for (int c = threadIdx.x; c < dh; c += blockDim.x) {
     float s = 0.f;
     for (int h = 0; h < H; ++h) s += to_f32(K[(((size_t)b * H + h) * N + x) * dh + c]);
@@ -396,7 +402,7 @@ void launch_mean_heads(const Dims& D, const void* K, float* Km, cudaStream_t st)
   dim3 grid(D.N, D.B);
   const int threads = min(256, (D.dh + 31) / 32 * 32);
   TC_WITH_STORAGE_TYPE(D,
-    mean_heads_kernel<T><<<grid, threads, 0, st>>>((const T*)K, Km, D.H, D.N, D.dh);
+    launch_pdl(mean_heads_kernel<T>, grid, dim3(threads), 0, st, 0, (const T*)K, Km, D.H, D.N, D.dh);
     note_launch(););
 }
 

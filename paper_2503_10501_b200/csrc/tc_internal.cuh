@@ -6,6 +6,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "pdl.cuh"
 #include "tokencarve.h"
 
 #include <atomic>
