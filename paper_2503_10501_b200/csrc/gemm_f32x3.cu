@@ -22,6 +22,8 @@
 //     register tile: the tensor core adds into its accumulator with truncation, so a fresh
 //     accumulator every DRAIN_SLABS slabs and round-to-nearest adds in registers keep the bias
 //     out.  (The cross terms are 2^-11 of the sum: what is truncated there does not matter.)
+// For a symmetric C (A = B) lo hi and hi lo each have an accumulator, 512 columns of TMEM with two of
+// 128 for hi hi: entry (i, j) then is the same sum as (j, i), bit for bit.
 // S CTAs of a cluster share a tile, each with a part of K: at one to sixteen images there are far
 // fewer tiles than SMs, and a tile's K loop is most of a launch.  They exchange their partial tiles
 // through distributed shared memory, each adds up and writes some of the columns.
@@ -86,6 +88,7 @@ struct Out {
   int rows_t;      // rows of C that are written to plainT
   int sub;         // C -= A B^T instead of C = A B^T, with C taken as zero in rows z0 .. z1 - 1
   int z0, z1;
+  int sym;         // lo hi and hi lo in accumulators of their own (tiles up to 128 columns)
 };
 
 // NN: width of the tile (compile time: it sizes the register tile); S: CTAs that share it.
@@ -99,7 +102,8 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
   constexpr int NCH = (NCHUNK + 1) / 2;      // chunks per thread (two column halves)
   constexpr uint32_t A_B = a_bytes(), HALF = half_bytes(NN), STG = stage_bytes(NN);
   constexpr bool CROSS = NN <= 160;          // an accumulator for the cross terms
-  constexpr uint32_t ACC_STRIDE = CROSS ? 160 : 256, ACC_X = 2 * ACC_STRIDE;
+  constexpr uint32_t ACC_STRIDE = NN <= 128 ? 128 : CROSS ? 160 : 256, ACC_X = 2 * ACC_STRIDE, ACC_Y = 3 * ACC_STRIDE;
+  const bool sym = NN <= 128 && out.sym != 0;
   constexpr int LC = (NCHUNK + S - 1) / S;   // chunks of a rank: chunk c belongs to rank c % S
   static_assert(S == 1 || (uint32_t)(S * LC * BM * XROW * 4) <= STAGES * STG, "exchange buffer");
   // D float32, A and B TF32, both K-major, M = 128, N = NN
@@ -195,13 +199,14 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
         // Without an accumulator of their own the cross terms go first: what is truncated while they
         // are added is then relative to their own small size.
         const uint32_t tmem_x = CROSS ? tmem_base + ACC_X : tmem_d;
+        const uint32_t tmem_y = sym ? tmem_base + ACC_Y : tmem_x;
 #pragma unroll
         for (int k = 0; k < BK / UK; ++k)
           umma_tf32(tmem_x, al + (uint64_t)(2 * k), bh + (uint64_t)(2 * k), IDESC,
                     ((CROSS ? kb == 0 : first) && k == 0) ? 0u : 1u);
 #pragma unroll
         for (int k = 0; k < BK / UK; ++k)
-          umma_tf32(tmem_x, ah + (uint64_t)(2 * k), bl + (uint64_t)(2 * k), IDESC, 1u);
+          umma_tf32(tmem_y, ah + (uint64_t)(2 * k), bl + (uint64_t)(2 * k), IDESC, (sym && kb == 0 && k == 0) ? 0u : 1u);
 #pragma unroll
         for (int k = 0; k < BK / UK; ++k)
           umma_tf32(tmem_d, ah + (uint64_t)(2 * k), bh + (uint64_t)(2 * k), IDESC, (CROSS && first && k == 0) ? 0u : 1u);
@@ -286,6 +291,20 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
         }
       }
     };
+    auto drain_pair = [&]() {   // entry (j, i) adds the same two sums as (i, j), the other way round
+      const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16);
+#pragma unroll
+      for (int c = 0; c < NCH; ++c) {
+        const int chunk = 2 * c + half;
+        if (chunk >= NCHUNK) continue;
+        uint32_t x[16], y[16];
+        tmem_ld16_issue(taddr + ACC_X + (uint32_t)(chunk * 16), x);
+        tmem_ld16_issue(taddr + ACC_Y + (uint32_t)(chunk * 16), y);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int j = 0; j < 16; ++j) acc[c][j] += __uint_as_float(x[j]) + __uint_as_float(y[j]);
+      }
+    };
     bool ok = true;
     for (int ch = 0; ch < nchunks; ++ch) {
       const int buf = ch & 1;
@@ -295,7 +314,10 @@ __global__ void __launch_bounds__(THREADS) gemm_f32x3_kernel(const __grid_consta
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       drain((uint32_t)buf * ACC_STRIDE);
-      if (CROSS && ch == nchunks - 1) drain(ACC_X);   // (every MMA of the tile has completed)
+      if (CROSS && ch == nchunks - 1) {   // (every MMA of the tile has completed)
+        if (NN <= 128 && sym) drain_pair();
+        else drain(ACC_X);
+      }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0)
@@ -496,15 +518,19 @@ tc_status launch_gemm_f32x3(const F32x3Operand& A, const F32x3Operand& B, int M,
   // TMA rows and 16-byte stores: whole vectors everywhere
   if (M < 1 || W < 4 || (W & 3) || K < 1 || ((A.ld | B.ld) & 3) || ((A.stride | B.stride) & 3)) return TC_ERR_UNSUPPORTED;
   if (R.C != nullptr && ((R.ld & 3) || (R.stride & 3))) return TC_ERR_UNSUPPORTED;
-  const int n_tiles = W <= 192 ? 1 : (W + 159) / 160;   // (tiles over 160 columns have no accumulator for the cross terms)
+  // (tiles over 160 columns have no accumulator for the cross terms, those over 128 not two)
+  const int n_tiles = R.symmetric ? (W + 127) / 128 : W <= 192 ? 1 : (W + 159) / 160;
   int nn = ((W + n_tiles - 1) / n_tiles + 15) / 16 * 16;
   if (nn < 64) nn = 64;
   CUtensorMap mapA, mapB;
-  if (!encode_operand(&mapA, A, M, K, batch, BM) || !encode_operand(&mapB, B, W, K, batch, nn)) return TC_ERR_CUDA;
+  if (!encode_operand(&mapA, A, A.rows < 0 ? M : A.rows, K, batch, BM) ||
+      !encode_operand(&mapB, B, B.rows < 0 ? W : B.rows, K, batch, nn))
+    return TC_ERR_CUDA;
   Out out;
   out.plain = R.C; out.plainT = R.CT; out.sC = R.stride; out.sT = R.strideT; out.ld = R.ld; out.ldT = R.ldT;
   out.W = W; out.rows_t = R.rows_t < 0 ? M : R.rows_t;
   out.sub = R.subtract ? 1 : 0; out.z0 = R.zero_from; out.z1 = R.zero_to;
+  out.sym = R.symmetric ? 1 : 0;
   Scope scope_(cls, st);
   switch (nn) {
     case 64: return launch_nn<64>(mapA, mapB, out, M, K, batch, of_batch, status, st);

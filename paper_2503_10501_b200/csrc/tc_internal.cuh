@@ -170,6 +170,7 @@ struct F32x3Operand {
   const float* p;
   int ld;          // floats between rows
   size_t stride;   // floats between images
+  int rows = -1;   // rows that exist, the others read as zero (-1: all of M or W)
 };
 struct F32x3Result {
   float* C;
@@ -181,6 +182,7 @@ struct F32x3Result {
   int rows_t = -1;        // rows of C that go to CT (-1: all)
   bool subtract = false;  // C -= A B^T, C counting as zero in rows zero_from .. zero_to - 1
   int zero_from = 0, zero_to = 0;
+  bool symmetric = false; // A and B are the same: C is to be symmetric bit for bit
 };
 tc_status launch_gemm_f32x3(const F32x3Operand& A, const F32x3Operand& B, int M, int W, int K, int batch,
                             int of_batch, const F32x3Result& R, int32_t* status, cudaStream_t st, int cls);

@@ -6,6 +6,7 @@ import torch
 
 from oracle import ipgs_oracle as orc
 from paper_2503_10501_b200 import binding as tcb
+from paper_2503_10501_b200 import inputs
 import parity_util as pu
 
 pytestmark = pytest.mark.gpu
@@ -48,3 +49,17 @@ def test_full_solve_of_every_layout(N):
                                         (601, 385), (801, 577), (900, 640), (902, 641), (120, 111), (2881, 150)])
 def test_subspace_of_every_width(N, rank_cap):
     _check(N, 1000, max(8, min(rank_cap - 16, rank_cap * 3 // 4, 200)), rank_cap, seed=N, noise=1e-3)
+
+
+@pytest.mark.parametrize("B,N,d", [(1, 3, 64), (1, 64, 32), (2, 100, 36), (1, 128, 384), (3, 132, 388), (1, 133, 100), (1, 576, 1024), (9, 260, 416)])
+def test_float32_gram(B, N, d):
+    g = torch.Generator().manual_seed(N * d)
+    O = torch.randn(B, N, d, generator=g)
+    O[:, N // 2] = O[:, 0]   # identical rows have identical products
+    p = tcb.Params(batch=B, n_tokens=N, d_model=d, n_heads=1, head_dim=d, n_query=1, keep=1, rank_tol=0.0, dtype="f32")
+    G = tcb.tc_gram(p, O.cuda()).cpu()
+    norm = O.double().norm(dim=2)
+    err = (G.double() - O.double() @ O.double().mT).abs() / (norm[:, :, None] * norm[:, None, :])
+    assert err.max() < 2e-6
+    assert torch.equal(G, G.mT)
+    assert torch.equal(G[:, N // 2], G[:, 0])
