@@ -1,5 +1,6 @@
 // C ABI of libtokencarve: argument checks, workspace planning, and the order in which the
 // kernels of each stage are enqueued.
+#include <cuda.h>
 #include <math.h>
 #include <string.h>
 
@@ -624,6 +625,33 @@ tc_status tc_workspace_bytes_host(const tc_params* p, size_t* bytes) {
   return TC_OK;
 }
 
+// The address under which kernels can read a host buffer, or null unless it lies within one pinned
+// allocation.
+static const void* device_view(const void* host, size_t bytes) {
+  typedef CUresult (*attr_fn)(void*, CUpointer_attribute, CUdeviceptr);
+  static const attr_fn get = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool ok = cudaGetDriverEntryPoint("cuPointerGetAttribute", &f, cudaEnableDefault, &q) == cudaSuccess &&
+                    q == cudaDriverEntryPointSuccess;
+    if (!ok) cudaGetLastError();
+    return ok ? (attr_fn)f : nullptr;
+  }();
+  cudaPointerAttributes at;
+  if (get == nullptr || cudaPointerGetAttributes(&at, host) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (at.type != cudaMemoryTypeHost || at.devicePointer == nullptr) return nullptr;
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  if (get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, (CUdeviceptr)host) != CUDA_SUCCESS ||
+      get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, (CUdeviceptr)host) != CUDA_SUCCESS)
+    return nullptr;
+  const size_t off = (size_t)((CUdeviceptr)host - start);
+  return off < size && bytes <= size - off ? at.devicePointer : nullptr;
+}
+
 tc_status tc_carve_host(const tc_params* p, const void* O, const void* A, const void* X,
                         const void* K, const void* V, void* Xo, void* Ko, void* Vo,
                         int32_t* kept_idx, int32_t* img_status, void* ws, size_t ws_bytes,
@@ -645,6 +673,15 @@ tc_status tc_carve_host(const tc_params* p, const void* O, const void* A, const 
   const size_t iO = (size_t)D.N * D.d * e, iA = (size_t)D.H * D.T * D.N * e;
   const size_t iKV = (size_t)D.H * D.N * D.dh * e;
   const size_t iXo = (size_t)D.keep * D.d * e, iKVo = (size_t)D.H * D.keep * D.dh * e;
+  // Only the survivors' rows of X, K and V are read, P of N, a row at a time, by the gather (and, for
+  // other similarity features, all of X or K by the matching).  From pinned memory the gather reads
+  // them where they lie.  The bus is what bounds this call: of X, K and V a third crosses it at the
+  // usual proportions (8 images of 576 tokens, 4.32 -> 3.49 ms); rows read by a kernel come over it more
+  // slowly than copies, so from three quarters of the tokens on everything is copied.
+  const void* vX = D.sim_src != 1 && 4 * D.P <= 3 * D.N ? device_view(X, D.B * iO) : nullptr;
+  const void* vK = kv && vX && D.sim_src != 2 ? device_view(K, D.B * iKV) : nullptr;
+  const void* vV = kv && vK ? device_view(V, D.B * iKV) : nullptr;
+  const bool direct = vX != nullptr && !misaligned(vX) && (!kv || (vV != nullptr && !misaligned(vK) && !misaligned(vV)));
   // The batch goes through in a few chunks: the upload of chunk c + 1 (copy-in stream) and the
   // download of chunk c - 1 (copy-out stream) run while chunk c is carved on `stream`.
   std::lock_guard<std::mutex> lk(g_host_mu);
@@ -663,26 +700,31 @@ tc_status tc_carve_host(const tc_params* p, const void* O, const void* A, const 
     const size_t nb = base + (c < extra ? 1 : 0), o = b0;
     ok &= cudaMemcpyAsync(w + h.O + o * iO, (const char*)O + o * iO, nb * iO, cudaMemcpyHostToDevice, cin) == cudaSuccess;
     ok &= cudaMemcpyAsync(w + h.A + align_up(o * iA, 16), (const char*)A + o * iA, nb * iA, cudaMemcpyHostToDevice, cin) == cudaSuccess;
-    ok &= cudaMemcpyAsync(w + h.X + o * iO, (const char*)X + o * iO, nb * iO, cudaMemcpyHostToDevice, cin) == cudaSuccess;
-    if (kv) {
-      ok &= cudaMemcpyAsync(w + h.K + o * iKV, (const char*)K + o * iKV, nb * iKV, cudaMemcpyHostToDevice, cin) == cudaSuccess;
-      ok &= cudaMemcpyAsync(w + h.V + o * iKV, (const char*)V + o * iKV, nb * iKV, cudaMemcpyHostToDevice, cin) == cudaSuccess;
+    if (!direct) {
+      ok &= cudaMemcpyAsync(w + h.X + o * iO, (const char*)X + o * iO, nb * iO, cudaMemcpyHostToDevice, cin) == cudaSuccess;
+      if (kv) {
+        ok &= cudaMemcpyAsync(w + h.K + o * iKV, (const char*)K + o * iKV, nb * iKV, cudaMemcpyHostToDevice, cin) == cudaSuccess;
+        ok &= cudaMemcpyAsync(w + h.V + o * iKV, (const char*)V + o * iKV, nb * iKV, cudaMemcpyHostToDevice, cin) == cudaSuccess;
+      }
     }
     if (nchunk > 1) ok &= cudaEventRecord(hs->in[c], cin) == cudaSuccess;
     b0 += (int)nb;
   }
   if (!ok) return TC_ERR_CUDA;
+  const char* dX = direct ? (const char*)vX : w + h.X;
+  const char* dK = direct ? (const char*)vK : w + h.K;
+  const char* dV = direct ? (const char*)vV : w + h.V;
   b0 = 0;
   for (int c = 0; c < nchunk; ++c) {
     const size_t nb = base + (c < extra ? 1 : 0), o = b0;
     if (nchunk > 1) ok &= cudaStreamWaitEvent(st, hs->in[c], 0) == cudaSuccess;
     tc_params pc = *p;
     pc.batch = (int32_t)nb;
-    s = carve_impl(&pc, D.B, w + h.O + o * iO, w + h.A + align_up(o * iA, 16), w + h.X + o * iO,
-                 kv ? w + h.K + o * iKV : nullptr, kv ? w + h.V + o * iKV : nullptr,
-                 w + h.Xo + o * iXo, kv ? w + h.Ko + o * iKVo : nullptr,
-                 kv ? w + h.Vo + o * iKVo : nullptr, (int32_t*)(w + h.kept) + o * D.keep,
-                 (int32_t*)(w + h.status) + o, w + h.scratch, scratch, stream);
+    s = carve_impl(&pc, D.B, w + h.O + o * iO, w + h.A + align_up(o * iA, 16), dX + o * iO,
+                   kv ? dK + o * iKV : nullptr, kv ? dV + o * iKV : nullptr,
+                   w + h.Xo + o * iXo, kv ? w + h.Ko + o * iKVo : nullptr,
+                   kv ? w + h.Vo + o * iKVo : nullptr, (int32_t*)(w + h.kept) + o * D.keep,
+                   (int32_t*)(w + h.status) + o, w + h.scratch, scratch, stream);
     if (s != TC_OK) return s;
     if (nchunk > 1) {
       ok &= cudaEventRecord(hs->done[c], st) == cudaSuccess;

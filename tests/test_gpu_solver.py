@@ -63,3 +63,27 @@ def test_float32_gram(B, N, d):
     assert err.max() < 2e-6
     assert torch.equal(G, G.mT)
     assert torch.equal(G[:, N // 2], G[:, 0])
+
+
+@pytest.mark.parametrize("keep", [40, 97, 98])   # survivors just under, at and above three quarters of the tokens
+@pytest.mark.parametrize("where", ["pinned", "pageable", "middle of a pinned block"])
+def test_host_rows_gathered_or_copied(keep, where):
+    cfg = inputs.tiny_config(n_tokens=195, d_model=64, n_heads=3, head_dim=16, n_query=5, keep=keep, rank=30, dtype="f16",
+                             batch=3, seed=5, noise=0.3, rank_tol=0.0)
+    p = tcb.Params(batch=3, n_tokens=195, d_model=64, n_heads=3, head_dim=16, n_query=5, keep=keep, rank_tol=0.0, dtype="f16")
+    data = inputs.make_batch(cfg)
+    t = [torch.from_numpy(np.ascontiguousarray(data[k])) for k in "OAXKV"]
+    ref = [None if x is None else x.cpu() for x in tcb.tc_carve(p, *(x.cuda() for x in t), ws=tcb.workspace(p))]
+    if where == "pinned":
+        t = [x.pin_memory() for x in t]
+    elif where != "pageable":
+        def inside(x):
+            y = torch.empty(x.numel() + 64, dtype=x.dtype, pin_memory=True)[32:32 + x.numel()].view(x.shape)
+            return y.copy_(x)
+        t = [inside(x) for x in t]
+    out = tuple(torch.empty(r.shape, dtype=r.dtype, pin_memory=True) for r in ref)
+    ws = tcb.workspace(p, host=True)
+    tcb.tc_carve_host(p, *t, out, ws)
+    torch.cuda.synchronize()
+    for a, b in zip(ref, out):
+        assert torch.equal(a, b)
