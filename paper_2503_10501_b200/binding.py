@@ -47,6 +47,10 @@ class TokenCarveError(RuntimeError):
         self.status = status
 
 
+_DTYPES = {"f16": TC_F16, "f32": TC_F32, "bf16": TC_BF16}
+_SIM_FLAGS = {"O": 0, "X": TC_FLAG_SIM_X, "meanK": TC_FLAG_SIM_MEAN_K}
+_TORCH_DTYPES = {"f16": torch.float16, "bf16": torch.bfloat16, "f32": torch.float32}
+
 _lib = None
 
 
@@ -123,15 +127,15 @@ class Params:
     def c(self) -> TcParams:
         return TcParams(self.batch, self.n_tokens, self.d_model, self.n_heads, self.head_dim,
                         self.n_query, self.keep, self.n_merge, self.rho, self.lam, self.rank_tol,
-                        {"f16": TC_F16, "f32": TC_F32, "bf16": TC_BF16}[self.dtype],
+                        _DTYPES[self.dtype],
                         TC_NORM_SUM1 if self.score_norm == "sum1" else TC_NORM_NONE,
                         self.max_sweeps, self.rank_cap,
-                        {"O": 0, "X": TC_FLAG_SIM_X, "meanK": TC_FLAG_SIM_MEAN_K}[self.sim_source]
+                        _SIM_FLAGS[self.sim_source]
                         | (TC_FLAG_WEIGHTED_MERGE if self.weighted_merge else 0))
 
     @property
     def torch_dtype(self):
-        return {"f16": torch.float16, "bf16": torch.bfloat16, "f32": torch.float32}[self.dtype]
+        return _TORCH_DTYPES[self.dtype]
 
 
 def _check(fn: str, status: int) -> None:
@@ -147,7 +151,8 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    # (the handle alone: building torch's stream object takes 3 us, as long as a launch)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def tc_counts(p: Params) -> Tuple[int, int, int, int]:
@@ -210,7 +215,7 @@ def tc_rope_tables(pos: torch.Tensor, head_dim: int, base: float = 10000.0):
     assert pos.dtype == torch.int32
     shape = tuple(pos.shape) + (head_dim // 2,)
     cos = torch.empty(shape, dtype=torch.float32, device=pos.device)
-    sin = torch.empty(shape, dtype=torch.float32, device=pos.device)
+    sin = torch.empty_like(cos)
     _check("tc_rope_tables", lib().tc_rope_tables(_ptr(pos), pos.numel(), head_dim, base, _ptr(cos),
                                                   _ptr(sin), _stream()))
     return cos, sin
