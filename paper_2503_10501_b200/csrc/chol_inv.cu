@@ -6,15 +6,15 @@
 // Elimination of S next to the identity: step j subtracts multiples of row j from the rows below, in S
 // (columns right of j) and in what was the identity (columns left of j), which takes the place of the
 // columns of S that are finished.  A row is scaled by the root of its pivot at the end.
-// What bounds it is the latency of a step, in a chain of n: the matrix lives in registers (rows dealt
-// cyclically over eight warps, two neighbouring columns of each 64 per lane), two steps at a time
-// exchange their two rows through shared memory, behind one barrier, and the warp that owns the next
-// two rows updates and publishes them before it goes on with its other rows.
-// The steps come in phases of 32: the code of a phase covers, without any test, the rows that are not
-// finished when it begins.
-// Measured, 16 matrices: order 144 and 160, 53 and 62 us with the matrix in shared memory and blocks of
-// 16 columns -> 39 and 47 us here; a pair of steps takes 1000 cycles at order 160, of which the
-// multiply-adds are 240.
+// What bounds it is the chain of n steps.  So 16 rows are taken at a time (a panel), and the chain runs
+// in one warp: it factors the panel's diagonal block (a lane per column, two steps at a time, 200 cycles),
+// then a thread per column eliminates the panel's rows among themselves.  Eight other warps meanwhile
+// subtract the panel before from the rows below it, which they hold in registers (all columns of a row in
+// one warp: a multiplier costs a cycle of shared memory per warp that reads it); the next panel's rows
+// come first and are handed over.
+// Measured, 16 matrices: order 144 and 160, 53 and 62 us with the matrix in shared memory, 39 and 47 us
+// with all warps in step and two rows per barrier, 25 and 28 us here.  The first panels are bound by the
+// subtraction (5 000 cycles, 3 000 of them multiply-adds), the last ones by the chain (4 600).
 #include "pair_math.cuh"
 #include "tc_internal.cuh"
 
@@ -24,7 +24,13 @@ namespace tc {
 
 namespace {
 
-constexpr int CW = 8;  // warps
+constexpr int UW = 8;    // warps that hold the matrix
+constexpr int WARPS = 16;  // and those of the panels (two warpgroups each)
+constexpr int PB = 16;   // rows of a panel
+// registers of a thread where the matrix fills them (three column groups); together the 512 x 128 of the launch
+constexpr int REGS_MATRIX = 176, REGS_PANEL = 80;
+static_assert(REGS_MATRIX * UW + REGS_PANEL * (WARPS - UW) <= 128 * WARPS, "registers of a block");
+constexpr int XT_ROW = PB + 4;   // padded: a quarter warp's 16-byte accesses meet no bank twice
 
 struct CholArgs {
   float* S;          // [batch][..][ldS], order n; see `first`
@@ -44,197 +50,250 @@ struct CholArgs {
   int32_t* status;
 };
 
-// NP: 64-column groups, RW: rows per warp (n <= 8 RW).  Rows go to the warps in pairs: row 16 i' + 2 w + u
-// is row 2 i' + u of warp w.
-template <int NP, int RW>
-__global__ void __launch_bounds__(CW * 32, 1) chol_inv_reg_kernel(const CholArgs ca) {
-  constexpr int NC = 64 * NP;
-  constexpr int NPH = (RW + 3) / 4;                       // phases of 32 columns = 4 rows of a warp
-  __shared__ __align__(16) float rowp[2][2][NC];          // rows j, j + 1 as the others subtract them
-  __shared__ __align__(16) float rowr[2][2][CW][(RW + 3) & ~3];  // their entries below the pivots, by owner of the row of that number
-  __shared__ float2 s_piv[2];
-  __shared__ float s_pv[NC];                              // pivots
-  __shared__ float s_red[CW];
+// NP: 64-column groups, P: panels (n = 16 P <= 64 NP).
+template <int NP, int P>
+__global__ void __launch_bounds__(WARPS * 32, 1) chol_inv_kernel(const CholArgs ca) {
+  constexpr int NC = 64 * NP, PW = 2 * NP, THREADS = (UW + PW) * 32, n = PB * P;
+  constexpr int RW = 2 * P;                    // rows of a warp: 16 q + 2 w, + 1 of panel q
+  extern __shared__ __align__(16) uint8_t chol_smem[];
+  typedef float Rows[PB][NC];
+  typedef float Cols[NC][XT_ROW];
+  Rows& raw = *reinterpret_cast<Rows*>(chol_smem);   // rows of the next panel as the warps hand them over
+  Rows* xs = reinterpret_cast<Rows*>(chol_smem) + 1;   // [2]: rows of a panel, eliminated among themselves
+  Cols* xt = reinterpret_cast<Cols*>(xs + 2);          // [2]: the same by columns, times -1 / pivot: multipliers of the rows below
+  __shared__ __align__(16) float db[PB][PB], lt[PB][PB];
+  __shared__ float s_ninv[PB], s_rs[PB];
+  __shared__ float s_red[WARPS];
   __shared__ int s_bad;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = blockIdx.x;
-  const int n = ca.n;
   float* S = ca.S + (size_t)b * ca.sS;
   pdl_wait();
-  auto row_of = [&](int i) { return 16 * (i >> 1) + 2 * warp + (i & 1); };
-
-  f2 B[RW][NP];
-#pragma unroll
-  for (int i = 0; i < RW; ++i)
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      const int r = row_of(i), c = 2 * lane + 64 * p;
-      B[i][p] = (r < n && c < n) ? *reinterpret_cast<const f2*>(S + (size_t)r * ca.ldS + c) : 0ull;
-    }
   float md = 0.f;
-  for (int i = threadIdx.x; i < n + ca.n_rest; i += CW * 32) md = fmaxf(md, S[(size_t)i * (ca.ldS + 1)]);
+  for (int i = threadIdx.x; i < n + ca.n_rest; i += WARPS * 32) md = fmaxf(md, S[(size_t)i * (ca.ldS + 1)]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) md = fmaxf(md, __shfl_xor_sync(0xffffffffu, md, o));
   if (lane == 0) s_red[warp] = md;
   if (threadIdx.x == 0) s_bad = 0;
+
+  if (warp < UW) {
+    if constexpr (NP == 3) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_MATRIX));
+    const int w = warp;
+    auto row_of = [&](int i) { return PB * (i >> 1) + 2 * w + (i & 1); };
+    f2 B[RW][NP];
+#pragma unroll
+    for (int i = 0; i < RW; ++i)
+#pragma unroll
+      for (int g = 0; g < NP; ++g) {
+        const int c = 2 * lane + 64 * g;
+        B[i][g] = c < n ? *reinterpret_cast<const f2*>(S + (size_t)row_of(i) * ca.ldS + c) : 0ull;
+      }
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v < WARPS; ++v) md = fmaxf(md, s_red[v]);
+    if (ca.blocked && !ca.first) md = ca.largest[(size_t)b * ca.sL];
+    const float shift = ca.first ? ca.shift_rel * md : 0.f;
+#pragma unroll
+    for (int i = 0; i < RW; ++i)
+#pragma unroll
+      for (int g = 0; g < NP; ++g) {
+        const int r = row_of(i), c = 2 * lane + 64 * g;
+        float2 t = upk(B[i][g]);
+        if (c == r) t.x += shift;
+        if (c + 1 == r) t.y += shift;
+        B[i][g] = pk(t.x, t.y);
+      }
+    auto hand_over = [&](auto qc) {   // rows of panel q
+      constexpr int q = decltype(qc)::value;
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int g = 0; g < NP; ++g) *reinterpret_cast<f2*>(&raw[2 * w + u][2 * lane + 64 * g]) = B[2 * q + u][g];
+      asm volatile("bar.arrive 1, %0;" ::"n"(THREADS) : "memory");
+    };
+    // rows i0 .. i1 - 1 -= multipliers times the rows of panel p
+    auto subtract = [&](auto pc, auto ac, auto bc) {
+      constexpr int p = decltype(pc)::value, i0 = decltype(ac)::value, i1 = decltype(bc)::value;
+      constexpr int buf = p & 1;
+      // the panel's columns of the rows below start over as columns of the inverse
+      const bool zero = ((2 * lane + 64 * (p / 4)) >> 4) == p;
+#pragma unroll
+      for (int i = i0; i < i1; ++i) B[i][p / 4] = zero ? 0ull : B[i][p / 4];
+#pragma unroll(i1 - i0 <= 2 ? 4 : P <= 10 ? 2 : 1)   // (as far as the registers go)
+      for (int m = 0; m < PB; m += 2) {
+        f2 x[2][NP];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int g = 0; g < NP; ++g) x[u][g] = *reinterpret_cast<const f2*>(&xs[buf][m + u][2 * lane + 64 * g]);
+#pragma unroll
+        for (int i = i0; i < i1; ++i) {
+          const float2 l = *reinterpret_cast<const float2*>(&xt[buf][row_of(i)][m]);
+          const f2 l0 = pk(l.x, l.x), l1 = pk(l.y, l.y);
+#pragma unroll
+          for (int g = 0; g < NP; ++g) B[i][g] = fma2(l1, x[1][g], fma2(l0, x[0][g], B[i][g]));
+        }
+      }
+    };
+    hand_over(std::integral_constant<int, 0>{});
+    auto panel = [&](auto pc) {
+      constexpr int p = decltype(pc)::value;
+      if constexpr (p + 1 < P) {
+        asm volatile("bar.sync 3, %0;" ::"n"(THREADS) : "memory");   // panel p is there
+        subtract(pc, std::integral_constant<int, 2 * p + 2>{}, std::integral_constant<int, 2 * p + 4>{});
+        hand_over(std::integral_constant<int, p + 1>{});
+        if constexpr (p + 2 < P) {
+          subtract(pc, std::integral_constant<int, 2 * p + 4>{}, std::integral_constant<int, RW>{});
+        }
+      }
+    };
+    panel(std::integral_constant<int, 0>{});
+    panel(std::integral_constant<int, 1>{});
+    panel(std::integral_constant<int, 2>{});
+    panel(std::integral_constant<int, 3>{});
+    panel(std::integral_constant<int, 4>{});
+    panel(std::integral_constant<int, 5>{});
+    panel(std::integral_constant<int, 6>{});
+    panel(std::integral_constant<int, 7>{});
+    panel(std::integral_constant<int, 8>{});
+    panel(std::integral_constant<int, 9>{});
+    panel(std::integral_constant<int, 10>{});
+    return;
+  }
+
+  // ---- the panels ----
+  if constexpr (NP == 3) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_PANEL));
   __syncthreads();
 #pragma unroll
-  for (int w = 0; w < CW; ++w) md = fmaxf(md, s_red[w]);
+  for (int v = 0; v < WARPS; ++v) md = fmaxf(md, s_red[v]);
   if (ca.blocked && !ca.first) md = ca.largest[(size_t)b * ca.sL];
-  const float shift = ca.first ? ca.shift_rel * md : 0.f;
   // A direction of S under the rounding level of its entries can leave any pivot: one below 2.5e-7 of
   // the largest entry is raised to that.  Only a pivot that is negative by far more than rounding (or
   // no number) says that S is not what it should be.
   const float floor_p = 2.5e-7f * fmaxf(md, 1e-30f);
   const float bad_p = -1e-5f * md;
-#pragma unroll
-  for (int i = 0; i < RW; ++i)
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      const int r = row_of(i), c = 2 * lane + 64 * p;
-      float2 t = upk(B[i][p]);
-      if (c == r) t.x += shift;
-      if (c + 1 == r) t.y += shift;
-      B[i][p] = pk(t.x, t.y);
-    }
-  if (ca.blocked) {
-#pragma unroll
-    for (int i = 0; i < RW; ++i) {
-      const int r = row_of(i);
-      for (int c = lane; c < n && r < n; c += 32) S[(size_t)r * ca.ldS + c] = (c == r) ? 1.f : 0.f;
-    }
-    if (ca.first) {
-      if (threadIdx.x == 0) ca.largest[(size_t)b * ca.sL] = md;
-      for (int i = n + threadIdx.x; i < n + ca.n_rest; i += CW * 32) S[(size_t)i * (ca.ldS + 1)] += shift;
-    }
-  }
-
-  // rows j, j + 1 (j even) by their owner; their register indices lie in [I, I + 6).  Row j + 1 is
-  // published with step j applied to it (the owner's registers get that like everyone's, later).
-  auto publish = [&](int j, auto ic) {
-    constexpr int I = decltype(ic)::value;
-    if (((j >> 1) & (CW - 1)) == warp && j < n) {
-      f2 ra[NP], rb[NP];
-      const uint32_t at = 1u << (2 * (j >> 4)), atp = 1u << (j >> 6);
-      f2 ap = 0ull, bp = 0ull;  // columns j, j + 1 of both
-#pragma unroll
-      for (int i = I; i < I + 6 && i + 1 < RW; i += 2)
-        if ((at >> i) & 1u) {
-#pragma unroll
-          for (int p = 0; p < NP; ++p) {
-            ra[p] = B[i][p];
-            rb[p] = B[i + 1][p];
-            if ((atp >> p) & 1u) {
-              ap = ra[p];
-              bp = rb[p];
-            }
-          }
-        }
-      const int src = (j & 63) >> 1;
-      const float2 a2 = upk(ap), b2 = upk(bp);
-      const float pj = __shfl_sync(0xffffffffu, a2.x, src), sj = __shfl_sync(0xffffffffu, a2.y, src);
-      const float qj = __shfl_sync(0xffffffffu, b2.y, src);
-      const float m = -sj * rcp_newton(fmaxf(pj, floor_p));
-      const f2 m2 = pk(m, m);
-#pragma unroll
-      for (int p = 0; p < NP; ++p) {
-        const int c = 2 * lane + 64 * p;
-        const float2 x = upk(ra[p]), y = upk(fma2(m2, ra[p], rb[p]));
-        const bool here = c == j, right = c > j;
-        *reinterpret_cast<float2*>(&rowp[(j >> 1) & 1][0][c]) = make_float2(here ? 1.f : x.x, here ? 0.f : x.y);
-        *reinterpret_cast<float2*>(&rowp[(j >> 1) & 1][1][c]) = make_float2(here ? m : y.x, here ? 1.f : y.y);
-        if (c < 8 * RW) {
-          const int w = (c >> 1) & (CW - 1), i = 2 * (c >> 4);
-          *reinterpret_cast<float2*>(&rowr[(j >> 1) & 1][0][w][i]) = make_float2(right ? x.x : 0.f, here || right ? x.y : 0.f);
-          *reinterpret_cast<float2*>(&rowr[(j >> 1) & 1][1][w][i]) = make_float2(right ? y.x : 0.f, right ? y.y : 0.f);
-        }
-      }
-      if (lane == 0) s_piv[(j >> 1) & 1] = make_float2(pj, fmaf(m, sj, qj));
-    }
-  };
-  publish(0, std::integral_constant<int, 0>{});
-  int j = 0;
-  auto phase = [&](auto fc) {
-    constexpr int F = decltype(fc)::value, I0 = 4 * F, PJ = F / 2;
-    if constexpr (F < NPH) {
-      for (; j < n && j < 32 * (F + 1); j += 2) {
-        __syncthreads();  // rows j, j + 1 are there, and everyone has read the two before
-        const int buf = (j >> 1) & 1;
-        const float2 piv = s_piv[buf];
-        const float pa = fmaxf(piv.x, floor_p), pb = fmaxf(piv.y, floor_p);
-        const float ma = -rcp_newton(pa), mb = -rcp_newton(pb);
-        f2 xa[NP], xb[NP];
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-          xa[p] = *reinterpret_cast<const f2*>(&rowp[buf][0][2 * lane + 64 * p]);
-          xb[p] = *reinterpret_cast<const f2*>(&rowp[buf][1][2 * lane + 64 * p]);
-        }
-        // columns j, j + 1 of the rows below start over as columns of the inverse
-        const f2 keep = (2 * lane + 64 * PJ == j) ? 0ull : pk(1.f, 1.f);
-        auto update = [&](int i, float la, float lb) {
-          const float ua = la * ma, ub = lb * mb;
-          const f2 ua2 = pk(ua, ua), ub2 = pk(ub, ub);
-#pragma unroll
-          for (int p = 0; p < NP; ++p)
-            B[i][p] = fma2(ub2, xb[p], fma2(ua2, xa[p], p == PJ ? mul2(keep, B[i][p]) : B[i][p]));
-        };
-        auto update2 = [&](int i) {  // rows i, i + 1
-          const float2 la = *reinterpret_cast<const float2*>(&rowr[buf][0][warp][i]);
-          const float2 lb = *reinterpret_cast<const float2*>(&rowr[buf][1][warp][i]);
-          update(i, la.x, lb.x);
-          update(i + 1, la.y, lb.y);
-        };
-#pragma unroll
-        for (int i = I0; i < I0 + 6 && i < RW; i += 2) update2(i);
-        publish(j + 2, std::integral_constant<int, I0>{});
-#pragma unroll
-        for (int i = I0 + 6; i < RW; i += 2) update2(i);
-        if (threadIdx.x == 32 * (CW - 1)) {
-          s_pv[j] = pa;
-          s_pv[j + 1] = pb;
-          if (!(piv.x > bad_p) || !(piv.y > bad_p)) s_bad = 1;
-        }
-      }
-    }
-  };
-  phase(std::integral_constant<int, 0>{});
-  phase(std::integral_constant<int, 1>{});
-  phase(std::integral_constant<int, 2>{});
-  phase(std::integral_constant<int, 3>{});
-  phase(std::integral_constant<int, 4>{});
-  phase(std::integral_constant<int, 5>{});
-  __syncthreads();
-  pdl_trigger();
-  if (threadIdx.x == 0 && s_bad) atomicMax(&ca.status[b], (int)TC_ERR_BREAKDOWN);
+  const int c = threadIdx.x - UW * 32;
+  if (c >= NC) return;
   float* R = ca.R + (size_t)b * ca.sR;
+  bool bad = false;
+#pragma unroll 1
+  for (int q = 0; q < P; ++q) {
+    const int j0 = PB * q, buf = q & 1;
+    asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");   // its rows have been handed over
+    float x[PB];
+    if (warp == UW) {
+      const int cl = lane & (PB - 1);
+      float own_p = 1.f, own_inv = 1.f;
 #pragma unroll
-  for (int i = 0; i < RW; ++i) {
-    const int r = row_of(i);
-    if (r >= n) continue;
-    const float rs = rsqrtf(s_pv[r]);
+      for (int i = 0; i < PB; ++i) x[i] = raw[i][j0 + cl];
 #pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      const int c = 2 * lane + 64 * p;
-      const float2 t = upk(B[i][p]);
-      if (c < n)
-        *reinterpret_cast<float2*>(R + (size_t)r * ca.ldR + c) =
-            make_float2(c < r ? t.x * rs : (c == r ? rs : 0.f), c + 1 < r ? t.y * rs : (c + 1 == r ? rs : 0.f));
+      for (int m = 0; m < PB; m += 2) {   // two steps: rows m and m + 1, the second with the first one applied
+        db[m][cl] = x[m];
+        db[m + 1][cl] = x[m + 1];
+        const float piv = __shfl_sync(0xffffffffu, x[m], m), off = __shfl_sync(0xffffffffu, x[m + 1], m);
+        const float piv1 = __shfl_sync(0xffffffffu, x[m + 1], m + 1);
+        __syncwarp();
+        const float pa = fmaxf(piv, floor_p), ia = rcp_newton(pa), g = -off * ia, ta = x[m] * ia;
+        const float qb = fmaf(g, off, piv1), pb = fmaxf(qb, floor_p), ib = rcp_newton(pb);
+        const float tb = fmaf(g, x[m], x[m + 1]) * ib;
+        bad |= !(piv > bad_p) | !(qb > bad_p);
+        lt[m][cl] = ta;
+        lt[m + 1][cl] = tb;
+        if (cl == m) {
+          own_p = pa;
+          own_inv = ia;
+        }
+        if (cl == m + 1) {
+          own_p = pb;
+          own_inv = ib;
+        }
+        auto next = [&](int i, float r0, float r1) { x[i] = fmaf(-fmaf(g, r0, r1), tb, fmaf(-r0, ta, x[i])); };
+#pragma unroll
+        for (int i4 = (m + 2) & ~3; i4 < PB; i4 += 4) {
+          const float4 r0 = *reinterpret_cast<const float4*>(&db[m][i4]), r1 = *reinterpret_cast<const float4*>(&db[m + 1][i4]);
+          if (i4 > m + 1) {
+            next(i4, r0.x, r1.x);
+            next(i4 + 1, r0.y, r1.y);
+          }
+          next(i4 + 2, r0.z, r1.z);
+          next(i4 + 3, r0.w, r1.w);
+        }
+      }
+      s_ninv[cl] = -own_inv;
+      s_rs[cl] = rsqrtf(own_p);
+    }
+    const bool mine = (c >> 4) == q;   // a column of the panel starts over as one of the identity
+#pragma unroll
+    for (int i = 0; i < PB; ++i) x[i] = mine ? (c == j0 + i ? 1.f : 0.f) : raw[i][c];
+    asm volatile("bar.sync 2, %0;" ::"n"(PW * 32) : "memory");   // the block's factor is there
+#pragma unroll
+    for (int m = 0; m < PB - 1; ++m) {
+#pragma unroll
+      for (int i4 = (m + 1) & ~3; i4 < PB; i4 += 4) {
+        const float4 l = *reinterpret_cast<const float4*>(&lt[m][i4]);
+        if (i4 > m) x[i4] = fmaf(-l.x, x[m], x[i4]);
+        if (i4 + 1 > m) x[i4 + 1] = fmaf(-l.y, x[m], x[i4 + 1]);
+        if (i4 + 2 > m) x[i4 + 2] = fmaf(-l.z, x[m], x[i4 + 2]);
+        if (i4 + 3 > m) x[i4 + 3] = fmaf(-l.w, x[m], x[i4 + 3]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < PB; ++i) xs[buf][i][c] = x[i];
+#pragma unroll
+    for (int i = 0; i < PB; i += 4)
+      *reinterpret_cast<float4*>(&xt[buf][c][i]) = make_float4(x[i] * s_ninv[i], x[i + 1] * s_ninv[i + 1],
+                                                               x[i + 2] * s_ninv[i + 2], x[i + 3] * s_ninv[i + 3]);
+    if (q + 1 < P) asm volatile("bar.arrive 3, %0;" ::"n"(THREADS) : "memory");
+    if (c < n) {
+#pragma unroll
+      for (int i = 0; i < PB; ++i) R[(size_t)(j0 + i) * ca.ldR + c] = c <= j0 + i ? x[i] * s_rs[i] : 0.f;
     }
   }
+  if (bad) atomicMax(&ca.status[b], (int)TC_ERR_BREAKDOWN);
+  if (ca.blocked) {
+    for (int i = warp - UW; i < n; i += PW)
+      for (int k = lane; k < n; k += 32) S[(size_t)i * ca.ldS + k] = (k == i) ? 1.f : 0.f;
+    if (ca.first) {
+      if (c == 0) ca.largest[(size_t)b * ca.sL] = md;
+      for (int i = n + c; i < n + ca.n_rest; i += PW * 32) S[(size_t)i * (ca.ldS + 1)] += ca.shift_rel * md;
+    }
+  }
+  pdl_trigger();
 }
 
-template <int NP, int RW>
-void run(const CholArgs& ca, int batch, cudaStream_t st) {
-  launch_pdl(chol_inv_reg_kernel<NP, RW>, dim3(batch), dim3(CW * 32), 0, st, 0, ca);
+template <int NP, int P>
+tc_status run(const CholArgs& ca, int batch, cudaStream_t st) {
+  constexpr int smem = (3 * PB + 2 * XT_ROW) * 64 * NP * 4;
+  auto kernel = chol_inv_kernel<NP, P>;
+  if (NP == 3) {   // the split of the registers counts on what the launch brings
+    static const int regs = [&] {
+      cudaFuncAttributes a;
+      return cudaFuncGetAttributes(&a, (const void*)kernel) == cudaSuccess ? a.numRegs : 0;
+    }();
+    if (regs != 128) return TC_ERR_CUDA;
+    if (cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return TC_ERR_CUDA;
+  }
+  static_assert(NP == 3 || smem <= 48 * 1024, "shared memory without opting in");
+  if (launch_pdl(kernel, dim3(batch), dim3(WARPS * 32), smem, st, 0, ca) != cudaSuccess) return TC_ERR_CUDA;
   note_launch();
+  return TC_OK;
 }
 
-void launch_block(const CholArgs& ca, int batch, cudaStream_t st) {
-  if (ca.n <= 64) run<1, 8>(ca, batch, st);
-  else if (ca.n <= 96) run<2, 12>(ca, batch, st);
-  else if (ca.n <= 128) run<2, 16>(ca, batch, st);
-  else if (ca.n <= 144) run<3, 18>(ca, batch, st);
-  else if (ca.n <= 160) run<3, 20>(ca, batch, st);
-  else run<3, 24>(ca, batch, st);
+tc_status launch_block(const CholArgs& ca, int batch, cudaStream_t st) {
+  switch (ca.n / PB) {
+    case 1: return run<1, 1>(ca, batch, st);
+    case 2: return run<1, 2>(ca, batch, st);
+    case 3: return run<1, 3>(ca, batch, st);
+    case 4: return run<1, 4>(ca, batch, st);
+    case 5: return run<2, 5>(ca, batch, st);
+    case 6: return run<2, 6>(ca, batch, st);
+    case 7: return run<2, 7>(ca, batch, st);
+    case 8: return run<2, 8>(ca, batch, st);
+    case 9: return run<3, 9>(ca, batch, st);
+    case 10: return run<3, 10>(ca, batch, st);
+    case 11: return run<3, 11>(ca, batch, st);
+    case 12: return run<3, 12>(ca, batch, st);
+    default: return TC_ERR_UNSUPPORTED;
+  }
 }
 
 }  // namespace
@@ -261,8 +320,7 @@ tc_status launch_chol_inv(float* S, float* RinvT, float* panel, int k, int batch
     Scope scope_(KC_CHOL, st);
     ca.S = S; ca.R = RinvT; ca.n = k;
     ca.blocked = false; ca.first = true; ca.n_rest = 0; ca.largest = nullptr; ca.sL = 0;
-    launch_block(ca, batch, st);
-    return TC_OK;
+    return launch_block(ca, batch, st);
   }
   const int nb = chol_block(k);
   const size_t sP = chol_panel_floats(k);
@@ -274,7 +332,8 @@ tc_status launch_chol_inv(float* S, float* RinvT, float* panel, int k, int batch
       ca.S = S + (size_t)j0 * (k + 1); ca.R = RinvT + (size_t)j0 * (k + 1); ca.n = w;
       ca.blocked = true; ca.first = j0 == 0; ca.n_rest = j0 == 0 ? k - w : 0;
       ca.largest = panel + (size_t)k * nb; ca.sL = sP;
-      launch_block(ca, batch, st);
+      const tc_status e = launch_block(ca, batch, st);
+      if (e != TC_OK) return e;
     }
     if (j0 == 0 && j1 == k) break;
     F32x3Result rp;
