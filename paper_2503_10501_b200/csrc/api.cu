@@ -195,6 +195,20 @@ tc_status launch_gram(const Dims& D, const void* O, float* G, int ldg, int32_t* 
   return launch_gemm_f32x3(op, op, D.N, ldg, D.d, D.B, D.call_B, R, status, st, KC_GRAM);
 }
 
+// Eq. 3-10 on the rows of F [B, N, f]: all products of two tokens on the tensor cores, of which the
+// matching reads its own.  (A warp per pair of tokens, on the plain ALUs, took four times as long at
+// 8 images of 576 tokens and d = 4096: 245 us, 64 for both launches here.)
+static tc_status match_features(const Dims& D, const void* F, bool f32, int f, float* G, const int32_t* setA,
+                                const int32_t* setB, float* best_val, int32_t* best_dst, int32_t* status,
+                                cudaStream_t st) {
+  Dims Df = D;
+  Df.d = f;
+  if (f32) Df.f16 = Df.bf16 = false;
+  const tc_status s = launch_gram(Df, F, G, D.ldn, status, st);
+  if (s == TC_OK) launch_match_gram(D, G, D.ldn, setA, setB, best_val, best_dst, status, st);
+  return s;
+}
+
 static tc_status check_launch() {
   return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
@@ -410,14 +424,16 @@ tc_status tc_merge(const tc_params* p, const void* O, const int32_t* setA, const
   int32_t* flags = (int32_t*)(c.ws + c.P.flags);
   fill_i32(flags, D.B, 0, c.st);
   if (D.M > 0) {
+    float* G = (float*)(c.ws + c.P.G);
     if (D.sim_src == 2) {
       // the features are the head-mean keys: `O` is K [B, H, N, dh]
       float* Km = (float*)(c.ws + c.P.Kmean);
       launch_mean_heads(D, O, Km, c.st);
-      launch_match_rows_f32(D, Km, D.dh, setA, setB, bv, bd, flags, c.st);
+      s = match_features(D, Km, true, D.dh, G, setA, setB, bv, bd, flags, c.st);
     } else {
-      launch_match_rows(D, O, setA, setB, bv, bd, flags, c.st);  // rows of O, or of X
+      s = match_features(D, O, false, D.d, G, setA, setB, bv, bd, flags, c.st);  // rows of O, or of X
     }
+    if (s != TC_OK) return s;
   }
   launch_merge_select(D, setA, setB, bv, bd, merge_src, merge_dst, kept_idx, flags, c.st);
   return check_launch();
@@ -496,6 +512,7 @@ static tc_status carve_impl(const tc_params* p, int call_B, const void* O, const
   int32_t* msrc = (int32_t*)(c.ws + c.P.msrc);
   int32_t* mdst = (int32_t*)(c.ws + c.P.mdst);
   // selection and gather of images b0 .. b0 + Dg.B on the stream their scores were computed on
+  tc_status tail_err = TC_OK;
   const GroupTail tail = [&](const Dims& Dg, int b0, cudaStream_t st) {
     const size_t b = (size_t)b0, esz = D.esz;
     const size_t kv_in = (size_t)D.H * D.N * D.dh * esz, kv_out = (size_t)D.H * D.keep * D.dh * esz;
@@ -509,15 +526,18 @@ static tc_status carve_impl(const tc_params* p, int call_B, const void* O, const
     const char* Vg = kv ? (const char*)V + b * kv_in : nullptr;
     launch_prune(Dg, E + b * D.N, sA, sB, st);
     if (D.M > 0) {
+      float* Gg = (float*)(c.ws + c.P.G) + b * D.N * D.ldn;   // (the scores are done with it)
+      tc_status e = TC_OK;
       if (D.sim_src == 0) {
-        launch_match_gram(Dg, (const float*)(c.ws + c.P.G) + b * D.N * D.ldn, D.ldn, sA, sB, gbv, gbd, gst, st);
+        launch_match_gram(Dg, Gg, D.ldn, sA, sB, gbv, gbd, gst, st);
       } else if (D.sim_src == 1) {
-        launch_match_rows(Dg, Xg, sA, sB, gbv, gbd, gst, st);
+        e = match_features(Dg, Xg, false, D.d, Gg, sA, sB, gbv, gbd, gst, st);
       } else {
         float* Km = (float*)(c.ws + c.P.Kmean) + b * D.N * D.dh;
         launch_mean_heads(Dg, Kg, Km, st);
-        launch_match_rows_f32(Dg, Km, D.dh, sA, sB, gbv, gbd, gst, st);
+        e = match_features(Dg, Km, true, D.dh, Gg, sA, sB, gbv, gbd, gst, st);
       }
+      if (e != TC_OK) tail_err = e;
     }
     int32_t* gms = msrc + b * D.M;
     int32_t* gmd = mdst + b * D.M;
@@ -528,6 +548,7 @@ static tc_status carve_impl(const tc_params* p, int call_B, const void* O, const
                    D.wmerge ? E + b * D.N : nullptr, gst, st);
   };
   s = enqueue_score(c, O, A, E, C, S, nullptr, nullptr, img_status, &tail);
+  if (s == TC_OK) s = tail_err;
   if (s != TC_OK) return s;
   return check_launch();
 }

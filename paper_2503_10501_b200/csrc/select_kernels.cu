@@ -209,112 +209,6 @@ void launch_match_gram(const Dims& D, const float* G, int ldg, const int32_t* se
 }
 
 // ------------------------------------------------------------------------------------------
-// Eq. 3-10 from the rows of O (stand-alone Stage II): one block per Set-B token keeps its row
-// in shared memory as float32; each warp takes Set-A rows in turn.
-// ------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(256) match_rows_kernel(const T* __restrict__ O,
-                                                        const int32_t* __restrict__ setA,
-                                                        const int32_t* __restrict__ setB,
-                                                        float* __restrict__ best_val,
-                                                        int32_t* __restrict__ best_dst, int N,
-                                                        int d, int nA, int nB,
-                                                        int32_t* __restrict__ status) {
-  extern __shared__ float rowb[];  // [d]
-  __shared__ float sv[8];
-  __shared__ int si[8];
-  __shared__ float s_nb;
-  const int b = blockIdx.y, jb = blockIdx.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  pdl_wait();
-  pdl_trigger();
-  const int tb = setB[(size_t)b * nB + jb];
-  const T* Ob = O + (size_t)b * N * d;
-  // a token number outside [0, N) in a caller's list is reported and never used as an address
-  if (tb < 0 || tb >= N) {
-    if (threadIdx.x == 0) {
-      atomicMax(&status[b], (int)TC_ERR_INVALID_ARG);
-      best_val[(size_t)b * nB + jb] = -INFINITY;
-      best_dst[(size_t)b * nB + jb] = -1;
-    }
-    return;
-  }
-  for (int c = threadIdx.x; c < d; c += 256) rowb[c] = (float)Ob[(size_t)tb * d + c];
-  __syncthreads();
-  if (warp == 0) {
-    float s = 0.f;
-    for (int c = lane; c < d; c += 32) s += rowb[c] * rowb[c];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) s_nb = s;
-  }
-  __syncthreads();
-  const float inv_b = inv_norm_from_sq(s_nb);
-  float bv = -INFINITY;
-  int bi = 0x7fffffff;
-  for (int ja = warp; ja < nA; ja += 8) {
-    const int ta = setA[(size_t)b * nA + ja];
-    if (ta < 0 || ta >= N) {
-      if (lane == 0) atomicMax(&status[b], (int)TC_ERR_INVALID_ARG);
-      continue;
-    }
-    const T* ra = Ob + (size_t)ta * d;
-    float dot = 0.f, na = 0.f;
-    for (int c = lane; c < d; c += 32) {
-      const float v = (float)ra[c];
-      dot += v * rowb[c];
-      na += v * v;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      dot += __shfl_xor_sync(0xffffffffu, dot, o);
-      na += __shfl_xor_sync(0xffffffffu, na, o);
-    }
-    const float c = dot * inv_b * inv_norm_from_sq(na);
-    if (c > bv || (c == bv && ta < bi)) {
-      bv = c;
-      bi = ta;
-    }
-  }
-  if (lane == 0) {
-    sv[warp] = bv;
-    si[warp] = bi;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w)
-      if (sv[w] > bv || (sv[w] == bv && si[w] < bi)) {
-        bv = sv[w];
-        bi = si[w];
-      }
-    best_val[(size_t)b * nB + jb] = bv;
-    best_dst[(size_t)b * nB + jb] = (bi == 0x7fffffff) ? -1 : bi;
-  }
-}
-
-void launch_match_rows(const Dims& D, const void* O, const int32_t* setA, const int32_t* setB,
-                       float* best_val, int32_t* best_dst, int32_t* status, cudaStream_t st) {
-  Scope scope_(KC_MATCH, st);
-  if (D.nB == 0 || D.nA == 0) return;
-  dim3 grid(D.nB, D.B);
-  size_t smem = (size_t)D.d * sizeof(float);
-  TC_WITH_STORAGE_TYPE(D,
-    launch_pdl(match_rows_kernel<T>, grid, dim3(256), smem, st, 0, (const T*)O, setA, setB, best_val, best_dst, D.N,
-                                                  D.d, D.nA, D.nB, status);
-    note_launch(););
-}
-
-void launch_match_rows_f32(const Dims& D, const float* F, int f, const int32_t* setA,
-                           const int32_t* setB, float* best_val, int32_t* best_dst,
-                           int32_t* status, cudaStream_t st) {
-  Scope scope_(KC_MATCH, st);
-  if (D.nB == 0 || D.nA == 0) return;
-  dim3 grid(D.nB, D.B);
-  { launch_pdl(match_rows_kernel<float>, grid, dim3(256), (size_t)f * sizeof(float), st, 0, F, setA, setB, best_val, best_dst,
-                                                                         D.N, f, D.nA, D.nB, status); note_launch(); }
-}
-
-// ------------------------------------------------------------------------------------------
 // Choice of the M merged Set-B tokens (highest best-similarity, ties to the lower token; Set B
 // is in ascending token order so list position is token order), merge lists, kept list.
 // One block per image.

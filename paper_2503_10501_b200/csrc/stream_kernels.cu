@@ -381,28 +381,38 @@ void launch_compact(const Dims& D, const void* X, const void* K, const void* V,
 
 // ------------------------------------------------------------------------------------------
 // Km[b][x][:] = mean over the heads h of K[b][h][x][:], float32 (the features ToMe matches on).
-// grid (N, B), block dh (rounded up to a warp).
+// K is read once, so loads in flight are what counts: a thread per 16-byte vector of a row, the heads
+// one after the other, eight loads ahead.  grid (blocks of N * dh, B).
 // ------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void mean_heads_kernel(const T* __restrict__ K, float* __restrict__ Km, int H, int N,
-                                  int dh) {
-  const int x = blockIdx.x, b = blockIdx.y;
+__global__ void __launch_bounds__(128) mean_heads_kernel(const T* __restrict__ K, float* __restrict__ Km, int H,
+                                                         int n_vec) {
+  constexpr int L = 16 / sizeof(T);
+  const int v = blockIdx.x * 128 + threadIdx.x, b = blockIdx.y;   // vector of the image's N x dh
   const float inv = 1.0f / (float)H;
   pdl_wait();
   pdl_trigger();
-  for (int c = threadIdx.x; c < dh; c += blockDim.x) {
-    float s = 0.f;
-    for (int h = 0; h < H; ++h) s += to_f32(K[(((size_t)b * H + h) * N + x) * dh + c]);
-    Km[((size_t)b * N + x) * dh + c] = s * inv;
+  if (v >= n_vec) return;
+  const uint4* src = reinterpret_cast<const uint4*>(K) + (size_t)b * H * n_vec + v;
+  float s[L] = {};
+#pragma unroll 8
+  for (int h = 0; h < H; ++h) {
+    const uint4 x = __ldg(src + (size_t)h * n_vec);
+    const T* e = reinterpret_cast<const T*>(&x);
+#pragma unroll
+    for (int i = 0; i < L; ++i) s[i] += to_f32(e[i]);
   }
+  float4* dst = reinterpret_cast<float4*>(Km + ((size_t)b * n_vec + v) * L);
+#pragma unroll
+  for (int i = 0; i < L; i += 4) dst[i / 4] = make_float4(s[i] * inv, s[i + 1] * inv, s[i + 2] * inv, s[i + 3] * inv);
 }
 
 void launch_mean_heads(const Dims& D, const void* K, float* Km, cudaStream_t st) {
   Scope scope_(KC_MATCH, st);
-  dim3 grid(D.N, D.B);
-  const int threads = min(256, (D.dh + 31) / 32 * 32);
+  const int n_vec = (int)((size_t)D.N * D.dh * D.esz / 16);
+  dim3 grid((n_vec + 127) / 128, D.B);
   TC_WITH_STORAGE_TYPE(D,
-    launch_pdl(mean_heads_kernel<T>, grid, dim3(threads), 0, st, 0, (const T*)K, Km, D.H, D.N, D.dh);
+    launch_pdl(mean_heads_kernel<T>, grid, dim3(128), 0, st, 0, (const T*)K, Km, D.H, n_vec);
     note_launch(););
 }
 

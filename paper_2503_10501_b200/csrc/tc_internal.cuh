@@ -117,12 +117,10 @@ void launch_attn_finish(const Dims& D, const float* s_part, float* S, cudaStream
 void launch_combine(const Dims& D, const float* C, const float* S, float* E, cudaStream_t st);
 // Stage I prune + Eq. 3-9 split.
 void launch_prune(const Dims& D, const float* E, int32_t* setA, int32_t* setB, cudaStream_t st);
-// Eq. 3-10 best match per Set-B token, from the Gram matrix or from the rows of O.
+// Eq. 3-10 best match per Set-B token, from the Gram matrix.
 // (status [B]: receives TC_ERR_INVALID_ARG for an image whose lists hold a token number outside
 // [0, N); such an entry is skipped, never used as an address.  The same for the launchers below.)
 void launch_match_gram(const Dims& D, const float* G, int ldg, const int32_t* setA, const int32_t* setB,
-                       float* best_val, int32_t* best_dst, int32_t* status, cudaStream_t st);
-void launch_match_rows(const Dims& D, const void* O, const int32_t* setA, const int32_t* setB,
                        float* best_val, int32_t* best_dst, int32_t* status, cudaStream_t st);
 // top-M of the best similarities, merge lists, kept list.
 void launch_merge_select(const Dims& D, const int32_t* setA, const int32_t* setB,
@@ -135,10 +133,6 @@ void launch_compact(const Dims& D, const void* X, const void* K, const void* V,
                     void* Ko, void* Vo, const float* E, int32_t* status, cudaStream_t st);
 // Km [B, N, dh] float32 = mean over the heads of K [B, H, N, dh].
 void launch_mean_heads(const Dims& D, const void* K, float* Km, cudaStream_t st);
-// launch_match_rows on float32 features F [B, N, f] whatever the storage type of the call.
-void launch_match_rows_f32(const Dims& D, const float* F, int f, const int32_t* setA,
-                           const int32_t* setB, float* best_val, int32_t* best_dst,
-                           int32_t* status, cudaStream_t st);
 
 // Sec. 3.2: rows idx[b][0..n_sub) of O gathered into Os [B, n_sub, d] (D describes O).
 void launch_gather_rows(const Dims& D, int n_sub, const void* O, const int32_t* idx, void* Os,
