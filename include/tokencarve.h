@@ -311,8 +311,8 @@ tc_status tc_reassemble(const tc_params* p, int32_t n_sys, int32_t n_text, const
  *   The attention is causal (row i sees the keys j <= i); a visual token a probe row cannot see
  *   gets probability 0.  float32 scores and sums, probabilities rounded to the storage type
  *   before they multiply V.
- *   img_status [B] as in tc_score.  ws: device scratch of tc_probe_workspace_bytes() bytes (the
- *   transposed V), owned by the caller; nothing is allocated; asynchronous on `stream`.
+ *   img_status [B] as in tc_score.  ws: device scratch of tc_probe_workspace_bytes() bytes,
+ *   owned by the caller; nothing is allocated; asynchronous on `stream`.
  * Returns TC_ERR_UNSUPPORTED for float32 storage or head_dim != 128.
  */
 tc_status tc_probe_workspace_bytes(const tc_params* p, int32_t n_sys, int32_t n_text, size_t* bytes);

@@ -4,24 +4,10 @@
 // probe rows pay to the visual tokens (the slice Eq. 3-7 averages).  The probability matrix is
 // never written out in full.
 //
-// Both products run on the 5th-generation tensor cores (tcgen05.mma kind::f16, M = N = 128,
-// float32 accumulators in TMEM, operands staged by TMA with the 128-byte swizzle).  One CTA owns
-// 128 query rows of one head of one image and walks the keys in blocks of 128:
-//   - warp 8 (one lane): TMA loads of the query tile (once), then per block the key tile and,
-//     when Z is wanted, the tile of V^T (V is transposed into the workspace first, so that both
-//     operands of P V have their contraction index contiguous);
-//   - warp 9 (one lane): S = Q K^T into TMEM; later O_blk = P V into a second accumulator;
-//   - warps 0-7: two threads per query row, each with half of the block's 128 columns (and half
-//     of the row of Z).  The scores come back with tcgen05.ld, get the causal mask, and feed an
-//     online softmax in the exp2 domain (the two halves of a row exchange their block maxima
-//     through shared memory); the probabilities are written as
-//     float16 / bfloat16 into a shared-memory tile of their own (in the swizzled layout the
-//     tensor core expects), and the block's P V is folded into a float32 row of Z held in
-//     registers, rescaled when the running maximum moves.
-// The scores have two accumulators and V^T two tiles: while the softmax warps work on block i the
-// tensor core already forms the scores of block i + 1, and the loads of block i + 1 are in flight.
-// The probe rows take two passes over the keys instead (first the row maxima and sums, then the
-// normalised probabilities of the visual columns) and need no V.
+// Both products run on the 5th-generation tensor cores (tcgen05.mma kind::f16, float32 accumulators in
+// TMEM, operands staged by TMA with the 128-byte swizzle), 128 query rows at a time against blocks of
+// keys, with an online softmax in the exp2 domain.  V is read as it lies: the contraction index is the
+// row there.
 // Every mbarrier wait is bounded; a wait that runs out records an error for the image and the
 // CTA winds down (TMEM is still freed).
 #include "tc_internal.cuh"
@@ -35,18 +21,18 @@ using namespace t5;
 
 constexpr int QT = 128;          // query rows per CTA
 constexpr int KB = 128;          // keys per block
+constexpr int SB = 64;           // keys per softmax step of the rows of Z
 constexpr int DH = 128;          // head dimension the kernel is built for
 constexpr uint32_t ATOM = 128 * 128;        // bytes of one 128-row x 64-element swizzle atom
 constexpr uint32_t TILE_B = 2 * ATOM;       // a 128 x 128 tile of 16-bit elements
-constexpr uint32_t SMEM_O = 6 * TILE_B + 1024;   // Q, K, two tiles of P, two tiles of V^T
-constexpr uint32_t STG_ROW = 2 * KB + 16;         // bytes of a row of the staging tile (padded: no bank is hit twice by a quarter warp)
-constexpr uint32_t SMEM_A = 2 * TILE_B + QT * STG_ROW + 1024;   // Q, K, staging tile of the probabilities
-constexpr uint32_t TMEM_COLS_O = 512;            // two score accumulators and two for the blocks' P V
-constexpr uint32_t TMEM_COLS_A = 256;            // two score accumulators
+constexpr uint32_t SMEM_Z = 6 * TILE_B + 1024;                      // two of Q, K and V each
+constexpr uint32_t SMEM_P = 3 * TILE_B + 4 * 32 * 64 + 1024;        // Q, two of K, staging of the probabilities
+constexpr uint32_t TMEM_COLS_Z = 512;                               // two of the scores and two of Z
+constexpr uint32_t TMEM_COLS_P = 256;                               // two of the scores
 
-// D float32, A and B float16 (bf = 0) or bfloat16 (bf = 1), both K-major, M = N = 128
-__device__ __forceinline__ uint32_t idesc(int bf) {
-  return (1u << 4) | (bf ? ((1u << 7) | (1u << 10)) : 0u) | ((uint32_t)(128 >> 3) << 17) |
+// D float32, A and B float16 (bf = 0) or bfloat16 (bf = 1), both K-major, M = 128, N = n
+__device__ __forceinline__ uint32_t idesc(int bf, int n = 128) {
+  return (1u << 4) | (bf ? ((1u << 7) | (1u << 10)) : 0u) | ((uint32_t)(n >> 3) << 17) |
          ((uint32_t)(128 >> 4) << 24);
 }
 
@@ -60,7 +46,7 @@ __device__ __forceinline__ void umma_16(uint32_t tmem_d, uint64_t da, uint64_t d
       : "memory");
 }
 
-// the eight tcgen05.mma of a 128 x 128 x 128 product of two swizzled 16-bit tiles
+// the eight tcgen05.mma of a product over dh of two swizzled 16-bit tiles
 __device__ __forceinline__ void mma_tile(uint32_t tmem_d, uint32_t a_base, uint32_t b_base, uint32_t id) {
 #pragma unroll
   for (int ks = 0; ks < 8; ++ks) {
@@ -68,6 +54,24 @@ __device__ __forceinline__ void mma_tile(uint32_t tmem_d, uint32_t a_base, uint3
     umma_16(tmem_d, umma_desc(a_base + atom) + (uint64_t)(2 * (ks & 3)),
             umma_desc(b_base + atom) + (uint64_t)(2 * (ks & 3)), id, ks > 0 ? 1u : 0u);
   }
+}
+
+// Descriptor of a tile whose rows of 128 bytes run along the operand's N, 128-byte swizzle: eight rows
+// (K) are 1024 bytes, the next 64 columns of N one atom further.
+__device__ __forceinline__ uint64_t umma_desc_mn(uint32_t smem_addr) {
+  return umma_desc(smem_addr) | ((uint64_t)(ATOM >> 4) << 16);
+}
+// D (+)= P V for 64 keys, with P (16-bit pairs, a row per lane) in TMEM and V stored [K][N]: 16 rows of V per tcgen05.mma
+__device__ __forceinline__ void mma_tile_pv(uint32_t tmem_d, uint32_t tmem_p, uint32_t v_base, uint32_t id, bool accum) {
+#pragma unroll
+  for (int ks = 0; ks < SB / 16; ++ks)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(tmem_d), "r"(tmem_p + (uint32_t)(8 * ks)), "l"(umma_desc_mn(v_base + (uint32_t)ks * 2048u)), "r"(id | (1u << 16)),
+        "r"((accum || ks > 0) ? 1u : 0u)
+        : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t* r) {
@@ -81,6 +85,14 @@ __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t* r) {
         "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
         "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() {
@@ -115,61 +127,293 @@ struct ProbeArgs {
   int bf;
 };
 
-// WANT_O: visual query rows -> rows of Z (O_out [B][n_vis][H * dh]).
-// !WANT_O: probe rows -> probabilities of the visual columns (A_out [B][H][n_rows][n_vis]).
-template <typename T, bool WANT_O>
-__global__ void __launch_bounds__(320, 1) probe_kernel(
+constexpr int Z_TMA = 8, Z_MMA = 9, Z_THREADS = 352;   // (a warp that issues products per query tile)
+constexpr int P_TMA = 4, P_MMA = 5, P_THREADS = 192;
+constexpr float MAX_SLACK = 8.f;
+
+// Visual query rows -> rows of Z (out [B][n_vis][H * dh]).  Two neighbouring query tiles per CTA: one
+// tile's softmax runs while the tensor core works for the other, and both read the same key and value
+// tiles, in steps of 64 keys:
+//   - warp 8 (one lane): TMA, two key and value tiles (128 keys) ahead;
+//   - warps 9 and 10: a query tile each, per step Z += P V and the scores of a later step.  P is read
+//     from TMEM, where it lies over the scores that it came from; the two score buffers of a tile
+//     alternate, so that the next scores are there when a step of the softmax ends;
+//   - warps 0-3 and 4-7: the softmax of a tile, a thread per row, all scores of a step in registers.
+//     Z stays in TMEM.  The maximum that the exponents refer to is moved (and Z and the row sum
+//     rescaled) only when a row's own has grown by more than 2^8 over it: Z = P V / sum is the same
+//     whatever the reference, and float16 holds 2^8 with the same relative precision as 1.
+// TMEM is full with 2 x 2 x 64 columns of scores and 2 x 128 of Z.
+// What bounds it: the chain of a step, 1 070 cycles of softmax (512 of them exponentials at the unit's
+// rate), which the other tile's overlaps, and issuing its products with their waits, 1 400 cycles.
+// Measured, 16 prompts of 675 tokens, 32 heads: 220 us (one tile per CTA, P through shared memory, V
+// transposed beforehand) -> 126.
+template <typename T>
+__global__ void __launch_bounds__(Z_THREADS, 1) probe_z_kernel(
     const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
-    const __grid_constant__ CUtensorMap mapVt, ProbeArgs pa, T* __restrict__ out,
+    const __grid_constant__ CUtensorMap mapV, ProbeArgs pa, T* __restrict__ out,
     int32_t* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
-  // bar_k: key tile landed; bar_kfree: its scores are formed (the tile may be reloaded);
-  // bar_v[2]: V^T tile landed; bar_s[2]: scores ready in accumulator 0 / 1; bar_sfree[2]: the
-  // softmax warps are done with that accumulator; bar_p[2]: tile of P written; bar_pv[2]: its
-  // P V done (O_blk ready, that tile of P free); bar_vfree[2]: the same event for the loader of
-  // the V^T tiles (every waiter has a barrier of its own, so none can fall two completions
-  // behind); bar_ofree[2]: the softmax warps have folded that O_blk into their rows
-  __shared__ __align__(8) uint64_t bar_q, bar_k, bar_kfree, bar_v[2], bar_vfree[2], bar_s[2], bar_sfree[2],
-      bar_p[2], bar_pv[2], bar_ofree[2];
-  constexpr uint32_t TMEM_COLS = WANT_O ? TMEM_COLS_O : TMEM_COLS_A;
+  __shared__ __align__(8) uint64_t bar_q[2], bar_k[2], bar_kfree[2], bar_v[2], bar_vfree[2];   // (the last four by stage)
+  __shared__ __align__(8) uint64_t bar_s[2][2], bar_p[2][2], bar_pv[2];   // by query tile: scores ready; P written (both by buffer); P V done
   __shared__ uint32_t s_tmem;
   __shared__ int s_fail;
-  __shared__ float s_xm[2][2][QT];   // block maxima of the two column halves, double-buffered
-  __shared__ float s_xl[2][QT];      // row sums of the two halves
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int qt = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int bh = b * pa.H + h;
-  const int q0 = pa.row0 + qt * QT;                       // position of this tile's first row
-  const int q_last = min(pa.row0 + pa.n_rows, q0 + QT) - 1;  // ... and of its last row in use
-  const int nkb = q_last / KB + 1;                        // causal: keys up to the last row's position
+  const int h = blockIdx.y, b = blockIdx.z, bh = b * pa.H + h;
+  const int tile0 = 2 * (int)(gridDim.x - 1 - blockIdx.x);           // the longest rows first
+  const int end = pa.row0 + pa.n_rows;                               // past the last query row
+  auto q0_of = [&](int t) { return pa.row0 + (tile0 + t) * QT; };
+  auto last_of = [&](int t) { return min(end, q0_of(t) + QT) - 1; };
+  const int nt = q0_of(1) < end ? 2 : 1;                             // tiles that have rows
+  auto steps_of = [&](int t) { return t < nt ? last_of(t) / SB + 1 : 0; };   // causal
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-  const uint32_t sQ = smem_base, sK = smem_base + TILE_B;
-  auto sP = [&](int i) { return smem_base + (uint32_t)(2 + (i & 1)) * TILE_B; };
-  auto sV = [&](int i) { return smem_base + (uint32_t)(4 + (i & 1)) * TILE_B; };
-  const uint32_t id = idesc(pa.bf);
+  auto sQ = [&](int t) { return smem_base + (uint32_t)t * TILE_B; };
+  auto sK = [&](int s) { return smem_base + (uint32_t)(2 + s) * TILE_B; };
+  auto sV = [&](int s) { return smem_base + (uint32_t)(4 + s) * TILE_B; };
+  const uint32_t id_s = idesc(pa.bf, SB), id_o = idesc(pa.bf);
 
   if (threadIdx.x == 0) {
-    mbar_init(smem_u32(&bar_q), 1);
-    mbar_init(smem_u32(&bar_k), 1);
-    mbar_init(smem_u32(&bar_kfree), 1);
     for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&bar_q[i]), 1);
+      mbar_init(smem_u32(&bar_k[i]), 1);
+      mbar_init(smem_u32(&bar_kfree[i]), (uint32_t)nt);
       mbar_init(smem_u32(&bar_v[i]), 1);
-      mbar_init(smem_u32(&bar_vfree[i]), 1);
-      mbar_init(smem_u32(&bar_s[i]), 1);
-      mbar_init(smem_u32(&bar_sfree[i]), 8);
-      mbar_init(smem_u32(&bar_p[i]), 8);
+      mbar_init(smem_u32(&bar_vfree[i]), (uint32_t)nt);
+      for (int u = 0; u < 2; ++u) {
+        mbar_init(smem_u32(&bar_s[i][u]), 1);
+        mbar_init(smem_u32(&bar_p[i][u]), 4);
+      }
       mbar_init(smem_u32(&bar_pv[i]), 1);
-      mbar_init(smem_u32(&bar_ofree[i]), 8);
     }
     s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 9) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_u32(&s_tmem)),
-                 "r"(TMEM_COLS)
+  if (warp == Z_MMA) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(TMEM_COLS_Z)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  auto tmem_s = [&](int t, int i) { return s_tmem + (uint32_t)t * 128u + ((uint32_t)i & 1u) * 64u; };
+  auto tmem_o = [&](int t) { return s_tmem + 256u + (uint32_t)t * 128u; };
+  auto phase = [](int i) { return (uint32_t)i & 1u; };               // of a barrier without stages
+  auto sphase = [](int i) { return ((uint32_t)i >> 1) & 1u; };       // of one with two
+
+  if (warp == Z_TMA) {
+    if (lane == 0) {
+      bool ok = true;
+      auto load = [&](const CUtensorMap* map, uint32_t dst, int row, uint64_t* bar) {
+        mbar_expect_tx(smem_u32(bar), TILE_B);
+        tma_load_3d(dst, map, 0, row, bh, smem_u32(bar));
+        tma_load_3d(dst + ATOM, map, 64, row, bh, smem_u32(bar));
+      };
+      load(&mapQ, sQ(0), q0_of(0), &bar_q[0]);
+      // (a stage is free when every tile is done with it: both walk all key tiles but the last, which
+      // no other follows in its stage)
+      for (int it = 0; 2 * it < steps_of(nt - 1) && ok; ++it) {
+        const int s = it & 1;
+        if (it >= 2 && !mbar_wait(smem_u32(&bar_kfree[s]), sphase(it - 2))) { ok = false; break; }
+        load(&mapK, sK(s), it * KB, &bar_k[s]);
+        if (it == 0 && nt > 1) load(&mapQ, sQ(1), q0_of(1), &bar_q[1]);
+        if (it >= 2 && !mbar_wait(smem_u32(&bar_vfree[s]), sphase(it - 2))) { ok = false; break; }
+        load(&mapV, sV(s), it * KB, &bar_v[s]);
+      }
+      if (!ok) s_fail = 1;
+    }
+  } else if (warp >= Z_MMA) {
+    // A step's few waits and commits take as long to issue as its products: a warp per tile.
+    const int t = warp - Z_MMA, n = steps_of(t);
+    // scores of step i, over the buffer of step i - 2
+    auto scores = [&](int i) {
+      const int s = (i >> 1) & 1;
+      if (i == 0 && !mbar_wait(smem_u32(&bar_q[t]), 0)) return false;
+      if ((i & 1) == 0 && !mbar_wait(smem_u32(&bar_k[s]), sphase(i >> 1))) return false;
+      if (i >= 2 && !mbar_wait(smem_u32(&bar_pv[t]), phase(i - 2))) return false;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (elect_one()) {
+        mma_tile(tmem_s(t, i), sQ(t), sK(s) + ((uint32_t)i & 1u) * (SB * 128u), id_s);
+        umma_commit(smem_u32(&bar_s[t][i & 1]));
+        if ((i & 1) || i == n - 1) umma_commit(smem_u32(&bar_kfree[s]));
+      }
+      __syncwarp();
+      return true;
+    };
+    auto weigh = [&](int i) {   // Z += P V of step i
+      const int s = (i >> 1) & 1;
+      if ((i & 1) == 0 && !mbar_wait(smem_u32(&bar_v[s]), sphase(i >> 1))) return false;
+      if (!mbar_wait(smem_u32(&bar_p[t][i & 1]), sphase(i))) return false;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (elect_one()) {
+        mma_tile_pv(tmem_o(t), tmem_s(t, i), sV(s) + ((uint32_t)i & 1u) * (SB * 128u), id_o, i > 0);
+        umma_commit(smem_u32(&bar_pv[t]));
+        if ((i & 1) || i == n - 1) umma_commit(smem_u32(&bar_vfree[s]));
+      }
+      __syncwarp();
+      return true;
+    };
+    bool ok = n < 1 || (scores(0) && (n < 2 || scores(1)));
+    for (int i = 0; i < n && ok; ++i) ok = weigh(i) && (i + 2 >= n || scores(i + 2));
+    if (!ok && lane == 0) s_fail = 1;
+  } else {
+    const int t = warp >> 2, row = (warp & 3) * 32 + lane;
+    const int qpos = q0_of(t) + row, q_last = last_of(t), n = steps_of(t);
+    const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16, to = tmem_o(t) + lanes;
+    // (a warp without rows in use only keeps the barriers going)
+    const bool work = q0_of(t) + (warp & 3) * 32 <= q_last;
+    float m = -INFINITY, l = 0.f;
+    bool ok = true;
+    for (int i = 0; i < n; ++i) {
+      if (ok && !mbar_wait(smem_u32(&bar_s[t][i & 1]), sphase(i))) ok = false;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (work) {
+        const uint32_t ts = tmem_s(t, i) + lanes;
+        float x[SB];
+        {
+          uint32_t* r = reinterpret_cast<uint32_t*>(x);
+#pragma unroll
+          for (int c = 0; c < SB / 32; ++c) tmem_ld32_issue(ts + (uint32_t)(c * 32), r + c * 32);
+          tmem_wait_ld();
+        }
+        const int jmax = qpos - i * SB;   // columns 0 .. jmax are visible (a row in use is no later than the last key)
+        if (!__all_sync(0xffffffffu, jmax >= SB - 1)) {   // (only on the diagonal)
+#pragma unroll
+          for (int j = 0; j < SB; ++j) x[j] = j <= jmax ? x[j] : -INFINITY;
+        }
+        float bm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int j = 0; j < SB; j += 8)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) bm[u] = fmaxf(fmaxf(bm[u], x[j + u]), x[j + 4 + u]);
+        const float own = fmaxf(fmaxf(bm[0], bm[1]), fmaxf(bm[2], bm[3])) * pa.scale2;
+        if (__any_sync(0xffffffffu, own > m + MAX_SLACK)) {
+          const float m_new = fmaxf(m, own), alpha = m_new == -INFINITY ? 1.f : ex2(m - m_new);
+          m = m_new;
+          l *= alpha;
+          if (i > 0) {
+            if (ok && !mbar_wait(smem_u32(&bar_pv[t]), phase(i - 1))) ok = false;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+            for (int c = 0; c < DH / 32; ++c) {
+              uint32_t r[32];
+              tmem_ld32_issue(to + (uint32_t)(c * 32), r);
+              tmem_wait_ld();
+#pragma unroll
+              for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) * alpha);
+              tmem_st16(to + (uint32_t)(c * 32), r);
+              tmem_st16(to + (uint32_t)(c * 32 + 16), r + 16);
+            }
+          }
+        }
+        const float mm = m == -INFINITY ? 0.f : m;
+        float ls[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int c = 0; c < SB / 32; ++c) {
+          uint32_t r[16];
+#pragma unroll
+          for (int j = 0; j < 32; j += 2) {
+            const float e0 = ex2(fmaf(x[c * 32 + j], pa.scale2, -mm)), e1 = ex2(fmaf(x[c * 32 + j + 1], pa.scale2, -mm));
+            ls[j & 2] += e0;
+            ls[(j & 2) + 1] += e1;
+            r[j / 2] = pack2<T>(e0, e1);
+          }
+          tmem_st16(ts + (uint32_t)(c * 16), r);
+        }
+        l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_p[t][i & 1])) : "memory");
+    }
+    if (n > 0) {
+      if (ok && !mbar_wait(smem_u32(&bar_pv[t]), phase(n - 1))) ok = false;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (!ok) s_fail = 1;
+      // The rows leave through the tile's query tile (its last scores are formed): a thread owns a row,
+      // so stores from its registers would put each lane of a store into a sector of its own; from
+      // there a warp writes a row per store.  16-byte chunk c of row r lies at c ^ (r & 7).
+      uint8_t* stg = smem_gen + (uint32_t)t * TILE_B + (uint32_t)((warp & 3) * 32) * 256u;
+      if (work) {
+        const float inv_l = l > 0.f ? 1.0f / l : 0.f;
+#pragma unroll
+        for (int c = 0; c < DH / 32; ++c) {
+          uint32_t r[32];
+          tmem_ld32_issue(to + (uint32_t)(c * 32), r);
+          tmem_wait_ld();
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            auto z = [&](int j) { return __uint_as_float(r[q * 8 + j]) * inv_l; };
+            uint4 v;
+            v.x = pack2<T>(z(0), z(1));
+            v.y = pack2<T>(z(2), z(3));
+            v.z = pack2<T>(z(4), z(5));
+            v.w = pack2<T>(z(6), z(7));
+            *reinterpret_cast<uint4*>(stg + (uint32_t)lane * 256u + (((uint32_t)(c * 4 + q) ^ ((uint32_t)lane & 7u)) << 4)) = v;
+          }
+        }
+        __syncwarp();
+        if (s_fail == 0) {   // its own 32 rows
+          const int q0w = q0_of(t) + (warp & 3) * 32, n_out = min(32, q_last + 1 - q0w);
+          // row q0w + i - n_sys of O, columns h * dh ..: 256 bytes, 8 per lane
+          uint2* dst = reinterpret_cast<uint2*>(out + (((size_t)b * pa.n_vis + (q0w - pa.n_sys)) * pa.H + h) * DH) + lane;
+#pragma unroll 8
+          for (int i = 0; i < n_out; ++i)
+            dst[(size_t)i * pa.H * (DH / 4)] = *reinterpret_cast<const uint2*>(
+                stg + (uint32_t)i * 256u + ((((uint32_t)lane >> 1) ^ ((uint32_t)i & 7u)) << 4) + ((uint32_t)lane & 1u) * 8u);
+        }
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x == 0 && s_fail != 0 && status != nullptr) atomicMax(&status[b], (int)TC_ERR_CUDA);
+  if (warp == Z_MMA) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(TMEM_COLS_Z) : "memory");
+  }
+}
+
+// Probe rows -> probabilities of the visual columns (out [B][H][n_rows][n_vis]), 128 rows per CTA, in
+// two passes over the keys: row maxima and sums of all of them, then the normalised probabilities of
+// the blocks with visual columns.  Warp 4 (one lane) loads, two key tiles ahead; warp 5 forms scores, one
+// block ahead; warps 0-3: a thread per row.  Prompts are short, so most tiles hold few rows and what
+// bounds a CTA is the chain of a block (load, product, exponentials): two CTAs share an SM.
+// Measured, 64 rows against 675 keys, 512 heads: 95 us (one CTA per SM, scores read twice) -> 74.
+template <typename T>
+__global__ void __launch_bounds__(P_THREADS, 2) probe_rows_kernel(
+    const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK, ProbeArgs pa,
+    T* __restrict__ out, int32_t* __restrict__ status) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t bar_q, bar_k[2], bar_kfree[2], bar_s[2], bar_sfree[2];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_fail;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int h = blockIdx.y, b = blockIdx.z, bh = b * pa.H + h;
+  const int q0 = pa.row0 + (int)blockIdx.x * QT;             // position of this tile's first row
+  const int q_last = min(pa.row0 + pa.n_rows, q0 + QT) - 1;  // ... and of its last row in use
+  const int nkb = q_last / KB + 1;                           // causal: keys up to the last row's position
+  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
+  const uint32_t sQ = smem_base;
+  auto sK = [&](int i) { return smem_base + (uint32_t)(1 + (i & 1)) * TILE_B; };
+  const uint32_t id = idesc(pa.bf);
+
+  if (threadIdx.x == 0) {
+    mbar_init(smem_u32(&bar_q), 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&bar_k[i]), 1);
+      mbar_init(smem_u32(&bar_kfree[i]), 1);
+      mbar_init(smem_u32(&bar_s[i]), 1);
+      mbar_init(smem_u32(&bar_sfree[i]), 4);
+    }
+    s_fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == P_MMA) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(TMEM_COLS_P)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -177,311 +421,127 @@ __global__ void __launch_bounds__(320, 1) probe_kernel(
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   auto tmem_s = [&](int i) { return s_tmem + (uint32_t)(i & 1) * 128u; };
-  auto tmem_o = [&](int i) { return s_tmem + 256u + (uint32_t)(i & 1) * 128u; };
+  auto phase = [](int i) { return ((uint32_t)i >> 1) & 1u; };
 
-  // key blocks in the order they are walked: all of them once (WANT_O), or all of them for the
-  // row statistics and then those that hold visual columns once more
+  // key blocks in the order they are walked
   const int vb0 = pa.n_sys / KB, vb1 = min(nkb - 1, (pa.n_sys + pa.n_vis - 1) / KB);
-  const int n_second = WANT_O ? 0 : max(0, vb1 - vb0 + 1);
-  const int n_iter = nkb + n_second;
+  const int n_iter = nkb + max(0, vb1 - vb0 + 1);
   auto block_of = [&](int it) { return it < nkb ? it : vb0 + (it - nkb); };
 
-  if (warp == 8) {
-    // ---- TMA producer: the key tile of block it + 1 as soon as the scores of block it are
-    //      formed, the V^T tile of block it + 1 as soon as P V of block it - 1 is done ----
+  if (warp == P_TMA) {
     if (lane == 0) {
       mbar_expect_tx(smem_u32(&bar_q), TILE_B);
       tma_load_3d(sQ, &mapQ, 0, q0, bh, smem_u32(&bar_q));
       tma_load_3d(sQ + ATOM, &mapQ, 64, q0, bh, smem_u32(&bar_q));
-      bool ok = true;
-      for (int it = 0; it < n_iter && ok; ++it) {
-        const int kb = block_of(it);
-        if (it > 0 && !mbar_wait(smem_u32(&bar_kfree), (uint32_t)(it - 1) & 1u)) { ok = false; break; }
-        mbar_expect_tx(smem_u32(&bar_k), TILE_B);
-        tma_load_3d(sK, &mapK, 0, kb * KB, bh, smem_u32(&bar_k));
-        tma_load_3d(sK + ATOM, &mapK, 64, kb * KB, bh, smem_u32(&bar_k));
-        if (WANT_O) {
-          if (it >= 2 && !mbar_wait(smem_u32(&bar_vfree[it & 1]), ((uint32_t)(it - 2) >> 1) & 1u)) { ok = false; break; }
-          mbar_expect_tx(smem_u32(&bar_v[it & 1]), TILE_B);
-          tma_load_3d(sV(it), &mapVt, kb * KB, 0, bh, smem_u32(&bar_v[it & 1]));
-          tma_load_3d(sV(it) + ATOM, &mapVt, kb * KB + 64, 0, bh, smem_u32(&bar_v[it & 1]));
+      for (int it = 0; it < n_iter; ++it) {
+        if (it >= 2 && !mbar_wait(smem_u32(&bar_kfree[it & 1]), phase(it - 2))) {
+          s_fail = 1;
+          break;
         }
+        const uint32_t full = smem_u32(&bar_k[it & 1]);
+        mbar_expect_tx(full, TILE_B);
+        tma_load_3d(sK(it), &mapK, 0, block_of(it) * KB, bh, full);
+        tma_load_3d(sK(it) + ATOM, &mapK, 64, block_of(it) * KB, bh, full);
       }
-      if (!ok) s_fail = 1;
     }
-  } else if (warp == 9) {
-    // ---- MMA issuer: scores one block ahead of the softmax ----
-    if (lane == 0) {
-      bool ok = mbar_wait(smem_u32(&bar_q), 0);
-      auto scores = [&](int it) {   // S[it & 1] = Q K(it)^T
-        if (!mbar_wait(smem_u32(&bar_k), (uint32_t)it & 1u)) return false;
-        if (it >= 2 && !mbar_wait(smem_u32(&bar_sfree[it & 1]), ((uint32_t)(it - 2) >> 1) & 1u)) return false;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        mma_tile(tmem_s(it), sQ, sK, id);
-        umma_commit(smem_u32(&bar_kfree));
+  } else if (warp == P_MMA) {
+    bool ok = mbar_wait(smem_u32(&bar_q), 0);
+    for (int it = 0; it < n_iter && ok; ++it) {
+      ok = mbar_wait(smem_u32(&bar_k[it & 1]), phase(it)) &&
+           (it < 2 || mbar_wait(smem_u32(&bar_sfree[it & 1]), phase(it - 2)));
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (elect_one()) {
+        mma_tile(tmem_s(it), sQ, sK(it), id);
         umma_commit(smem_u32(&bar_s[it & 1]));
-        return true;
-      };
-      if (ok) ok = scores(0);
-      for (int it = 0; it < n_iter && ok; ++it) {
-        if (it + 1 < n_iter) ok = scores(it + 1);
-        if (WANT_O && ok) {
-          const uint32_t par = ((uint32_t)it >> 1) & 1u;
-          if (!mbar_wait(smem_u32(&bar_p[it & 1]), par) || !mbar_wait(smem_u32(&bar_v[it & 1]), par) ||
-              (it >= 2 && !mbar_wait(smem_u32(&bar_ofree[it & 1]), ((uint32_t)(it - 2) >> 1) & 1u))) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          mma_tile(tmem_o(it), sP(it), sV(it), id);     // O_blk = P V
-          umma_commit(smem_u32(&bar_vfree[it & 1]));
-          umma_commit(smem_u32(&bar_pv[it & 1]));
-        }
+        umma_commit(smem_u32(&bar_kfree[it & 1]));
       }
-      if (!ok) s_fail = 1;
-    }
-  } else {
-    // ---- warps 0-7: softmax.  Thread = (query row = TMEM lane, column half) ----
-    constexpr int HC = KB / 2;                      // columns of a block per thread
-    const int row = (warp & 3) * 32 + lane, half = warp >> 2;
-    const int qpos = q0 + row;                       // sequence position of this row
-    const bool live = qpos <= q_last;
-    const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-    const uint32_t col0 = (uint32_t)(half * HC);
-    float m = -INFINITY, l = 0.f;                    // l: this thread's half of the row sum
-    float o[WANT_O ? HC : 1];
-    if (WANT_O) {
-#pragma unroll
-      for (int i = 0; i < HC; ++i) o[i] = 0.f;
-    }
-    auto pair_sync = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
-    bool ok = true;
-    float inv_l = 0.f;
-    float alpha_prev = 1.f;
-    // o = o * alpha_j + (P V of block j); alpha_j = 2^(m_{j-1} - m_j) is the factor block j's new
-    // maximum put on everything before it
-    auto fold = [&](int j, float alpha_j) {
-      if (ok && !mbar_wait(smem_u32(&bar_pv[j & 1]), ((uint32_t)j >> 1) & 1u)) ok = false;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-      for (int c = 0; c < HC / 32; ++c) {
-        uint32_t r[32];
-        tmem_ld32_issue(tmem_o(j) + lane_addr + col0 + (uint32_t)(c * 32), r);
-        tmem_wait_ld();
-#pragma unroll
-        for (int jj = 0; jj < 32; ++jj) o[c * 32 + jj] = fmaf(o[c * 32 + jj], alpha_j, __uint_as_float(r[jj]));
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0)
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_ofree[j & 1])) : "memory");
-    };
+    }
+    if (!ok && lane == 0) s_fail = 1;
+  } else {
+    const int row = warp * 32 + lane, qpos = q0 + row;
+    const bool work = q0 + warp * 32 <= q_last;   // some row of the warp is in use
+    uint8_t* stg = smem_gen + 3 * TILE_B + (uint32_t)warp * (32u * 64u);   // 32 rows x 32 columns
+    float m = -INFINITY, l = 0.f, inv_l = 0.f;
+    bool ok = true;
     for (int it = 0; it < n_iter; ++it) {
-      const int kb = block_of(it);
-      const bool second = it >= nkb;
-      const uint32_t ts = tmem_s(it) + lane_addr + col0;
-      if (!WANT_O && it == nkb) {
-        // between the two passes of the probe rows: the whole row sum
-        s_xl[half][row] = l;
-        pair_sync();
-        const float lt = s_xl[0][row] + s_xl[1][row];
-        inv_l = (lt > 0.f) ? 1.0f / lt : 0.f;
-      }
-      // A wait that runs out must not take this thread out of the loop: its partner would wait
-      // for it at the pair barrier for ever.  It goes on (on whatever the accumulators hold)
-      // without waiting again, and the image is reported at the end.
-      if (ok && !mbar_wait(smem_u32(&bar_s[it & 1]), ((uint32_t)it >> 1) & 1u)) ok = false;
+      if (ok && !mbar_wait(smem_u32(&bar_s[it & 1]), phase(it))) ok = false;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int jmax = min(qpos, pa.L - 1) - kb * KB - (int)col0;   // own columns 0 .. jmax are visible
-      float alpha = 1.f;
-      if (!second) {
-        // pass over the block for its maximum: own half, then the partner's through shared memory
-        float bm = -INFINITY;
+      float x[KB];
+      if (work) {
+        uint32_t* r = reinterpret_cast<uint32_t*>(x);
 #pragma unroll
-        for (int c = 0; c < HC / 32; ++c) {
-          uint32_t r[32];
-          tmem_ld32_issue(ts + (uint32_t)(c * 32), r);
-          tmem_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (c * 32 + j <= jmax) bm = fmaxf(bm, __uint_as_float(r[j]));
-        }
-        s_xm[it & 1][half][row] = bm;
-        pair_sync();
-        bm = fmaxf(bm, s_xm[it & 1][half ^ 1][row]);
-        const float m_new = fmaxf(m, bm * pa.scale2);
-        alpha = (m_new == -INFINITY) ? 1.f : ex2(m - m_new);
-        m = m_new;
-        l *= alpha;
-      }
-      if (WANT_O || !second) {
-        // probabilities of the own columns (unnormalised), their sum, and, with Z, the tile of P
-        float ls = 0.f;
-#pragma unroll
-        for (int c = 0; c < HC / 32; ++c) {
-          uint32_t r[32];
-          tmem_ld32_issue(ts + (uint32_t)(c * 32), r);
-          tmem_wait_ld();
-          float pr[32];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float e = ex2(fmaf(__uint_as_float(r[j]), pa.scale2, -m));
-            pr[j] = (c * 32 + j <= jmax && m != -INFINITY) ? e : 0.f;
-            ls += pr[j];
-          }
-          if (WANT_O) {
-            // The half's 64 columns are one swizzle atom of the P tile; chunk ch (8 columns) of
-            // the row lies at atom * ATOM + row * 128 + ((ch ^ (row & 7)) * 16).  (P V of the
-            // block before, which read this tile, was waited for when its result was folded in.)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const uint32_t ch = (uint32_t)(c * 4 + q);
-              uint4 v;
-              v.x = pack2<T>(pr[q * 8], pr[q * 8 + 1]);
-              v.y = pack2<T>(pr[q * 8 + 2], pr[q * 8 + 3]);
-              v.z = pack2<T>(pr[q * 8 + 4], pr[q * 8 + 5]);
-              v.w = pack2<T>(pr[q * 8 + 6], pr[q * 8 + 7]);
-              *reinterpret_cast<uint4*>(smem_gen + (uint32_t)(2 + (it & 1)) * TILE_B + (uint32_t)half * ATOM + (uint32_t)row * 128u +
-                                        ((ch ^ ((uint32_t)row & 7u)) << 4)) = v;
-            }
-          }
-        }
-        l += ls;
-      } else {
-        // second pass of the probe rows: normalised probabilities of the block's columns into a
-        // staging tile (row-major, 16-bit), from which whole rows leave in runs of 32
-        // neighbouring elements per store (a thread owns a row, so storing from the registers
-        // would put every lane of a store into a sector of its own)
-        uint8_t* stg = smem_gen + 2 * TILE_B;
-        if (it > nkb) pair_sync();   // the rows of the block before have left the tile
-#pragma unroll
-        for (int c = 0; c < HC / 32; ++c) {
-          uint32_t r[32];
-          tmem_ld32_issue(ts + (uint32_t)(c * 32), r);
-          tmem_wait_ld();
-          float pr[32];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float e = ex2(fmaf(__uint_as_float(r[j]), pa.scale2, -m)) * inv_l;
-            pr[j] = (c * 32 + j <= jmax) ? e : 0.f;
-          }
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            uint4 v;
-            v.x = pack2<T>(pr[q * 8], pr[q * 8 + 1]);
-            v.y = pack2<T>(pr[q * 8 + 2], pr[q * 8 + 3]);
-            v.z = pack2<T>(pr[q * 8 + 4], pr[q * 8 + 5]);
-            v.w = pack2<T>(pr[q * 8 + 6], pr[q * 8 + 7]);
-            *reinterpret_cast<uint4*>(stg + (uint32_t)row * STG_ROW + (col0 + (uint32_t)(c * 32 + q * 8)) * 2u) = v;
-          }
-        }
-        pair_sync();
-        {
-          const int x0 = kb * KB - pa.n_sys;   // visual index of the block's first column
-          for (int rr = warp; rr < QT; rr += 8) {
-            const int qp = q0 + rr;
-            if (qp > q_last) break;
-            T* drow = out + (((size_t)bh * pa.n_rows + (qp - pa.row0)) * pa.n_vis);
-            const T* srow = reinterpret_cast<const T*>(stg + (uint32_t)rr * STG_ROW);
-#pragma unroll
-            for (int j = 0; j < KB / 32; ++j) {
-              const int col = lane + 32 * j, x = x0 + col;
-              if (x >= 0 && x < pa.n_vis) drow[x] = srow[col];
-            }
-          }
-        }
+        for (int c = 0; c < KB / 32; ++c)
+          tmem_ld32_issue(tmem_s(it) + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * 32), r + c * 32);
+        tmem_wait_ld();
       }
       // this score accumulator may be overwritten
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0)
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_sfree[it & 1])) : "memory");
-      if (WANT_O) {
-        // hand this block's P to the tensor core, then fold the P V of the block BEFORE into the
-        // own half of the row of Z: that product ran while this block's probabilities were
-        // formed (two tiles of P, two accumulators for P V), so the wait below is short
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (lane == 0)
-          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_p[it & 1])) : "memory");
-        if (it > 0) fold(it - 1, alpha_prev);
-        alpha_prev = alpha;
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_sfree[it & 1])) : "memory");
+      if (!work) continue;
+      const int kb = block_of(it), jmax = qpos - kb * KB;   // columns 0 .. jmax are visible
+      if (!__all_sync(0xffffffffu, jmax >= KB - 1)) {       // (only blocks on the diagonal)
+#pragma unroll
+        for (int j = 0; j < KB; ++j) x[j] = j <= jmax ? x[j] : -INFINITY;
       }
-    }
-    if (WANT_O && n_iter > 0) fold(n_iter - 1, alpha_prev);
-    if (WANT_O) {
-      // the whole row sum (every thread of the team comes here, whatever happened above)
-      s_xl[half][row] = l;
-      pair_sync();
-      const float lt = s_xl[0][row] + s_xl[1][row];
-      inv_l = (lt > 0.f) ? 1.0f / lt : 0.f;
+      if (it < nkb) {
+        float bm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY}, ls[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int j = 0; j < KB; ++j) bm[j & 3] = fmaxf(bm[j & 3], x[j]);
+        const float m_new = fmaxf(m, fmaxf(fmaxf(bm[0], bm[1]), fmaxf(bm[2], bm[3])) * pa.scale2);
+        if (m_new != -INFINITY) {
+          l *= ex2(m - m_new);
+          m = m_new;
+#pragma unroll
+          for (int j = 0; j < KB; ++j) ls[j & 3] += ex2(fmaf(x[j], pa.scale2, -m));
+          l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
+        }
+        if (it == nkb - 1) inv_l = l > 0.f ? 1.0f / l : 0.f;
+        continue;
+      }
+      // Normalised probabilities, 32 columns at a time through a staging tile of the warp's, from which
+      // rows leave in runs of 32 neighbouring elements per store (a thread owns a row, so stores from
+      // its registers would put every lane into a sector of its own).  16-byte chunk q of row r lies
+      // at q ^ (r / 2 & 3).
+      const float mm = m == -INFINITY ? 0.f : m;
+      const int x0 = kb * KB - pa.n_sys;   // visual index of the block's first column
+#pragma unroll
+      for (int c = 0; c < KB / 32; ++c) {
+        if (x0 + c * 32 + 31 < 0 || x0 + c * 32 >= pa.n_vis) continue;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          auto p = [&](int j) { return ex2(fmaf(x[c * 32 + q * 8 + j], pa.scale2, -mm)) * inv_l; };
+          uint4 v;
+          v.x = pack2<T>(p(0), p(1));
+          v.y = pack2<T>(p(2), p(3));
+          v.z = pack2<T>(p(4), p(5));
+          v.w = pack2<T>(p(6), p(7));
+          *reinterpret_cast<uint4*>(stg + (uint32_t)lane * 64u + ((uint32_t)(q ^ ((lane >> 1) & 3)) << 4)) = v;
+        }
+        __syncwarp();
+        const int xv = x0 + c * 32 + lane;
+        const int n_out = min(32, q_last + 1 - q0 - warp * 32);
+        if (xv >= 0 && xv < pa.n_vis) {
+          T* dst = out + ((size_t)bh * pa.n_rows + (q0 - pa.row0) + warp * 32) * pa.n_vis + xv;
+#pragma unroll 8
+          for (int rr = 0; rr < n_out; ++rr) {
+            *dst = *reinterpret_cast<const T*>(stg + (uint32_t)rr * 64u + ((uint32_t)((lane >> 3) ^ ((rr >> 1) & 3)) << 4) +
+                                               ((uint32_t)lane & 7u) * 2u);
+            dst += pa.n_vis;
+          }
+        }
+        __syncwarp();
+      }
     }
     if (!ok) s_fail = 1;
-    if (WANT_O) {
-      // The rows of Z leave through a row-major staging tile in the first tile of P (every P V
-      // has completed): a thread owns half a row, so stores from its registers would put each
-      // lane of a store into a sector of its own; from the tile a warp writes a row per store.
-      uint8_t* stg = smem_gen + 2 * TILE_B;
-#pragma unroll
-      for (int q = 0; q < HC / 8; ++q) {
-        uint4 v;
-        v.x = pack2<T>(o[q * 8] * inv_l, o[q * 8 + 1] * inv_l);
-        v.y = pack2<T>(o[q * 8 + 2] * inv_l, o[q * 8 + 3] * inv_l);
-        v.z = pack2<T>(o[q * 8 + 4] * inv_l, o[q * 8 + 5] * inv_l);
-        v.w = pack2<T>(o[q * 8 + 6] * inv_l, o[q * 8 + 7] * inv_l);
-        *reinterpret_cast<uint4*>(stg + (uint32_t)row * STG_ROW + (uint32_t)(half * HC + q * 8) * 2u) = v;
-      }
-    }
-    pair_sync();
-    if (s_fail == 0) {
-      if (WANT_O) {
-        uint8_t* stg = smem_gen + 2 * TILE_B;
-        for (int rr = warp; rr < QT; rr += 8) {
-          const int qp = q0 + rr;
-          if (qp > q_last) break;
-          // row qp - n_sys of O, columns h * dh ..: 256 bytes, 8 per lane
-          uint2* dst = reinterpret_cast<uint2*>(out + (((size_t)b * pa.n_vis + (qp - pa.n_sys)) * pa.H + h) * DH);
-          dst[lane] = *reinterpret_cast<const uint2*>(stg + (uint32_t)rr * STG_ROW + (uint32_t)lane * 8u);
-        }
-      }
-    } else if (status != nullptr && threadIdx.x == 0) {
-      atomicMax(&status[b], (int)TC_ERR_CUDA);
-    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 9) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem),
-                 "r"(TMEM_COLS)
-                 : "memory");
-  }
-}
-
-// Vt [BH][dh][Lp] = V [BH][L][dh]^T, columns L .. Lp - 1 zero (Lp and dh even).  64 x 64 tiles,
-// two elements per access: a warp reads and writes 128 contiguous bytes.  grid (Lp / 64 rounded
-// up, dh / 64 rounded up, BH), block (32, 8).
-template <typename T>
-__global__ void __launch_bounds__(256) transpose_v_kernel(const T* __restrict__ V, T* __restrict__ Vt,
-                                                         int L, int Lp, int dh) {
-  __shared__ T t[64][66];
-  const size_t bh = blockIdx.z;
-  const int l0 = blockIdx.x * 64, d0 = blockIdx.y * 64;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int l = l0 + ty + 8 * i, d = d0 + 2 * tx;
-    uint32_t v = 0u;
-    if (l < L && d < dh) v = *reinterpret_cast<const uint32_t*>(V + (bh * L + l) * dh + d);
-    *reinterpret_cast<uint32_t*>(&t[ty + 8 * i][2 * tx]) = v;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int dd = ty + 8 * i, d = d0 + dd, l = l0 + 2 * tx;
-    if (d < dh && l < Lp) {
-      T pair[2] = {t[2 * tx][dd], t[2 * tx + 1][dd]};
-      *reinterpret_cast<uint32_t*>(Vt + (bh * dh + d) * Lp + l) = *reinterpret_cast<uint32_t*>(pair);
-    }
+  if (threadIdx.x == 0 && s_fail != 0 && status != nullptr) atomicMax(&status[b], (int)TC_ERR_CUDA);
+  if (warp == P_MMA) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(TMEM_COLS_P) : "memory");
   }
 }
 
@@ -501,16 +561,15 @@ bool encode16(CUtensorMap* map, const void* base, int inner, int rows, int bh, i
 
 template <typename T>
 tc_status run_probe(int B, int H, int L, int n_sys, int n_vis, int probe_start, int n_probe,
-                    const void* Q, const void* K, const void* V, void* O, void* A, void* Vt, int Lp,
+                    const void* Q, const void* K, const void* V, void* O, void* A,
                     int32_t* status, cudaStream_t st, int bf) {
   CUtensorMap mq, mk, mv;
   if (!encode16(&mq, Q, DH, L, B * H, bf) || !encode16(&mk, K, DH, L, B * H, bf)) return TC_ERR_CUDA;
-  if (O != nullptr && !encode16(&mv, Vt, Lp, DH, B * H, bf)) return TC_ERR_CUDA;
-  if (O == nullptr) mv = mk;
-  if (cudaFuncSetAttribute((const void*)probe_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)SMEM_O) != cudaSuccess ||
-      cudaFuncSetAttribute((const void*)probe_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)SMEM_A) != cudaSuccess)
+  if (O != nullptr && !encode16(&mv, V, DH, L, B * H, bf)) return TC_ERR_CUDA;
+  if (cudaFuncSetAttribute((const void*)probe_z_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)SMEM_Z) != cudaSuccess ||
+      cudaFuncSetAttribute((const void*)probe_rows_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)SMEM_P) != cudaSuccess)
     return TC_ERR_CUDA;
   ProbeArgs pa;
   pa.L = L; pa.n_sys = n_sys; pa.n_vis = n_vis; pa.H = H;
@@ -518,21 +577,19 @@ tc_status run_probe(int B, int H, int L, int n_sys, int n_vis, int probe_start, 
   pa.bf = bf;
   if (O != nullptr) {
     Scope scope_(KC_GRAM, st);
-    dim3 tg((Lp + 63) / 64, (DH + 63) / 64, B * H), tb(32, 8);
-    transpose_v_kernel<T><<<tg, tb, 0, st>>>((const T*)V, (T*)Vt, L, Lp, DH);
-    note_launch();
     pa.row0 = n_sys; pa.n_rows = n_vis;
-    dim3 grid((n_vis + QT - 1) / QT, H, B);
-    probe_kernel<T, true><<<grid, 320, SMEM_O, st>>>(mq, mk, mv, pa, (T*)O, status);
+    dim3 grid((n_vis + 2 * QT - 1) / (2 * QT), H, B);
+    probe_z_kernel<T><<<grid, Z_THREADS, SMEM_Z, st>>>(mq, mk, mv, pa, (T*)O, status);
     note_launch();
   }
   if (A != nullptr && n_probe > 0) {
     Scope scope_(KC_ATTN, st);
-    // columns a probe row may not see (keys after it) are never visited: they read as zero
-    if (cudaMemsetAsync(A, 0, (size_t)B * H * n_probe * n_vis * sizeof(T), st) != cudaSuccess) return TC_ERR_CUDA;
+    // columns a probe row may not see (keys after it) are not all visited: they read as zero
+    if (probe_start < n_sys + n_vis - 1 &&
+        cudaMemsetAsync(A, 0, (size_t)B * H * n_probe * n_vis * sizeof(T), st) != cudaSuccess) return TC_ERR_CUDA;
     pa.row0 = probe_start; pa.n_rows = n_probe;
     dim3 grid((n_probe + QT - 1) / QT, H, B);
-    probe_kernel<T, false><<<grid, 320, SMEM_A, st>>>(mq, mk, mv, pa, (T*)A, status);
+    probe_rows_kernel<T><<<grid, P_THREADS, SMEM_P, st>>>(mq, mk, pa, (T*)A, status);
     note_launch();
   }
   return TC_OK;
@@ -541,19 +598,17 @@ tc_status run_probe(int B, int H, int L, int n_sys, int n_vis, int probe_start, 
 }  // namespace
 
 size_t probe_workspace_bytes(int B, int H, int L, int dh) {
-  const size_t Lp = (size_t)(L + 7) / 8 * 8;
-  return align_up((size_t)B * H * dh * Lp * 2, 256);
+  (void)B; (void)H; (void)L; (void)dh;
+  return 256;   // (nothing is kept there)
 }
 
 tc_status launch_probe(int B, int H, int dh, int L, int n_sys, int n_vis, int probe_start, int n_probe,
                        const void* Q, const void* K, const void* V, void* O, void* A, void* ws,
                        int32_t* status, cudaStream_t st, int bf) {
   if (dh != DH) return TC_ERR_UNSUPPORTED;
-  const int Lp = (L + 7) / 8 * 8;
   if (bf)
-    return run_probe<__nv_bfloat16>(B, H, L, n_sys, n_vis, probe_start, n_probe, Q, K, V, O, A, ws, Lp,
-                                    status, st, 1);
-  return run_probe<__half>(B, H, L, n_sys, n_vis, probe_start, n_probe, Q, K, V, O, A, ws, Lp, status, st, 0);
+    return run_probe<__nv_bfloat16>(B, H, L, n_sys, n_vis, probe_start, n_probe, Q, K, V, O, A, status, st, 1);
+  return run_probe<__half>(B, H, L, n_sys, n_vis, probe_start, n_probe, Q, K, V, O, A, status, st, 0);
 }
 
 }  // namespace tc

@@ -102,3 +102,24 @@ def test_probe_rejects_unsupported_shapes():
     with pytest.raises(tcb.TokenCarveError) as e:
         tcb.tc_probe(p, 8, 8, 72, z, z, z)
     assert e.value.status == 2
+
+
+# visual rows that fill one query tile, one more, and a pair; steps of 64 keys with one and two tiles
+@pytest.mark.parametrize("n_sys,N,n_text,T", [(0, 1, 1, 1), (0, 64, 1, 1), (63, 2, 1, 1), (1, 128, 7, 8), (0, 129, 3, 2), (10, 256, 1, 129),
+                                              (70, 257, 130, 128)])
+def test_probe_tile_edges(n_sys, N, n_text, T):
+    L = n_sys + N + n_text
+    _check(B=1, H=2, n_sys=n_sys, N=N, n_text=n_text, probe_start=L - T, T=T, dtype="f16", seed=N)
+
+
+def test_probe_maximum_that_keeps_growing():
+    # scores that rise along the keys: every step moves the maximum by much more than the slack
+    Q, K, V = _qkv(1, 1, 400, 128, "f16", 7)
+    Q[:] = np.float16(0.5)
+    K[:] = (np.arange(400, dtype=np.float32) * 0.02)[None, None, :, None].astype(np.float16)
+    p = tcb.Params(batch=1, n_tokens=396, d_model=128, n_heads=1, head_dim=128, n_query=3, keep=1, dtype="f16")
+    O, A, st = tcb.tc_probe(p, 1, 3, 397, _dev(Q, "f16"), _dev(K, "f16"), _dev(V, "f16"))
+    torch.cuda.synchronize()
+    Or, Ar = orc.layer2_probe_matrix(Q[0], K[0], V[0], 1, 396, range(397, 400))
+    assert np.max(np.abs(_host(O)[0] - Or)) <= 4 * 2.0 ** -11 * np.abs(Or).max() + 1e-4
+    assert np.max(np.abs(_host(A)[0] - Ar) - 2.0 ** -10 * Ar) <= 2e-6
