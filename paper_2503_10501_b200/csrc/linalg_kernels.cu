@@ -11,6 +11,8 @@
 //             subspace is built (sign sketch of O, one multiplication by G, Cholesky-QR
 //             orthonormalisation), G is projected onto it (Rayleigh-Ritz) and only the k x k
 //             projection is decomposed.
+#include <cooperative_groups.h>
+
 #include "tc_internal.cuh"
 
 #include <utility>
@@ -342,7 +344,11 @@ __global__ void sketch_vec_kernel(const T* __restrict__ O, float* __restrict__ Y
 // Pairs follow a round-robin tournament: n/2 disjoint pairs per round, one warp per pair,
 // a block barrier between rounds.  R = elements of a column each lane keeps in registers.
 // ==========================================================================================
-template <int R>
+constexpr int JACOBI_CL_THREADS = 640;
+
+// AHEAD: the columns of J are loaded with those of W, not after the decision to rotate (out of L2 the
+// second wait would double a round).
+template <int R, bool AHEAD>
 __device__ inline int jacobi_pair(float* __restrict__ W, float* __restrict__ J, int n, int p,
                                   int q, int lane, float tol, float floor2,
                                   float count_floor2) {
@@ -350,11 +356,21 @@ __device__ inline int jacobi_pair(float* __restrict__ W, float* __restrict__ J, 
   float a = 0.f, bq = 0.f, g = 0.f;
   float* Wp = W + (size_t)p * n;
   float* Wq = W + (size_t)q * n;
+  float* Jp = J + (size_t)p * n;
+  float* Jq = J + (size_t)q * n;
+  float jpv[AHEAD ? R : 1], jqv[AHEAD ? R : 1];
 #pragma unroll
   for (int i = 0; i < R; ++i) {
     const int r = lane + 32 * i;
     wp[i] = (r < n) ? Wp[r] : 0.f;
     wq[i] = (r < n) ? Wq[r] : 0.f;
+    if constexpr (AHEAD) {
+      jpv[i] = (r < n) ? Jp[r] : 0.f;
+      jqv[i] = (r < n) ? Jq[r] : 0.f;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
     a = fmaf(wp[i], wp[i], a);
     bq = fmaf(wq[i], wq[i], bq);
     g = fmaf(wp[i], wq[i], g);
@@ -379,13 +395,11 @@ __device__ inline int jacobi_pair(float* __restrict__ W, float* __restrict__ J, 
       Wq[r] = fmaf(s, wp[i], c * wq[i]);
     }
   }
-  float* Jp = J + (size_t)p * n;
-  float* Jq = J + (size_t)q * n;
 #pragma unroll
   for (int i = 0; i < R; ++i) {
     const int r = lane + 32 * i;
     if (r < n) {
-      const float jp = Jp[r], jq = Jq[r];
+      const float jp = AHEAD ? jpv[AHEAD ? i : 0] : Jp[r], jq = AHEAD ? jqv[AHEAD ? i : 0] : Jq[r];
       Jp[r] = c * jp - s * jq;
       Jq[r] = fmaf(s, jp, c * jq);
     }
@@ -395,38 +409,53 @@ __device__ inline int jacobi_pair(float* __restrict__ W, float* __restrict__ J, 
   return fmaxf(a, bq) > count_floor2 ? 1 : 0;
 }
 
-template <int R>
-__global__ void __launch_bounds__(512) jacobi_kernel(const float* __restrict__ Hin, int ldh,
+// CL == 1: a block per image with both matrices in shared memory.  Else a cluster of CL blocks, the
+// matrices in L2, the pairs of a round dealt over all its warps: every pair's arithmetic is the same
+// whoever does it.  What bounds it is a round's latency, m rounds to a sweep.
+template <int R, int CL>
+__global__ void __launch_bounds__(CL == 1 ? 1024 : JACOBI_CL_THREADS) jacobi_kernel(const float* __restrict__ Hin, int ldh,
                                                     float* __restrict__ Wg, float* __restrict__ ZTg,
                                                     float* __restrict__ theta, int n,
-                                                    int max_sweeps, float tol, int use_smem,
+                                                    int max_sweeps, float tol,
                                                     int32_t* __restrict__ status, float floor_rel,
                                                     float count_rel) {
   extern __shared__ float sm[];
   __shared__ int s_rot;
-  __shared__ float s_red[16];
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ float s_red[32];
+  const int rank = CL == 1 ? 0 : (int)(blockIdx.x % CL), nt = blockDim.x, warps = nt / 32;
+  const int b = blockIdx.x / CL, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int gwarp = warp * CL + rank, gwarps = warps * CL;   // (neighbouring pairs on different SMs)
+  auto everyone = [] {
+    if constexpr (CL == 1) {
+      __syncthreads();
+    } else {
+      __syncwarp();
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+  };
   const size_t nn = (size_t)n * n;
   const float* Hb = Hin + b * (size_t)n * ldh;
-  float* W = use_smem ? sm : Wg + b * nn;
-  float* J = use_smem ? sm + nn : ZTg + b * nn;
+  float* W = CL == 1 ? sm : Wg + b * nn;
+  float* J = CL == 1 ? sm + nn : ZTg + b * nn;
 
   // W = (H + H^T) / 2 (column-major == row-major for a symmetric matrix), J = I
   float md = 0.f;
-  for (size_t e = tid; e < nn; e += 512) {
+  for (size_t e = (size_t)rank * nt + tid; e < nn; e += (size_t)CL * nt) {
     const int p = (int)(e / n), i = (int)(e % n);
     const float v = 0.5f * (Hb[(size_t)p * ldh + i] + Hb[(size_t)i * ldh + p]);
     W[e] = v;
     J[e] = (p == i) ? 1.f : 0.f;
-    if (p == i) md = fmaxf(md, fabsf(v));
   }
+  for (int i = tid; i < n; i += nt) md = fmaxf(md, fabsf(0.5f * (Hb[(size_t)i * ldh + i] + Hb[(size_t)i * ldh + i])));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) md = fmaxf(md, __shfl_xor_sync(0xffffffffu, md, o));
   if (lane == 0) s_red[warp] = md;
   if (tid == 0) s_rot = 0;
   __syncthreads();
+  everyone();
   md = s_red[0];
-  for (int w = 1; w < 16; ++w) md = fmaxf(md, s_red[w]);
+  for (int w = 1; w < warps; ++w) md = fmaxf(md, s_red[w]);
   // column pairs whose norms (eigenvalue estimates) are BOTH below the floor are left alone:
   // they are rounding noise of the largest eigenvalue, or lie below the rank cut-off, and
   // rotating them against each other only slows convergence
@@ -442,7 +471,7 @@ __global__ void __launch_bounds__(512) jacobi_kernel(const float* __restrict__ H
   for (; sweep < max_sweeps; ++sweep) {
     int rot = 0;
     for (int round = 0; round < m; ++round) {
-      for (int slot = warp; slot < half; slot += 16) {
+      for (int slot = gwarp; slot < half; slot += gwarps) {
         int u, v;
         if (slot == 0) {
           u = round;
@@ -455,25 +484,31 @@ __global__ void __launch_bounds__(512) jacobi_kernel(const float* __restrict__ H
         }
         if (u >= n || v >= n) continue;
         const int p = min(u, v), q = max(u, v);
-        rot += jacobi_pair<R>(W, J, n, p, q, lane, tol, floor2, count_floor2);
+        rot += jacobi_pair<R, CL != 1 && R <= 18>(W, J, n, p, q, lane, tol, floor2, count_floor2);
       }
-      __syncthreads();
+      everyone();
     }
-    if (lane == 0 && rot) atomicAdd(&s_rot, rot);
-    __syncthreads();
+    if (lane == 0 && rot) {
+      if constexpr (CL == 1) {
+        atomicAdd(&s_rot, rot);
+      } else {
+        for (int t = 0; t < CL; ++t) atomicAdd(cooperative_groups::this_cluster().map_shared_rank(&s_rot, t), rot);
+      }
+    }
+    everyone();
     const int total = s_rot;
-    __syncthreads();
-    if (tid == 0) s_rot = 0;
+    everyone();
+    if (tid == 0) s_rot = 0;   // (next added to after a sweep's barriers)
     if (total == 0) {
       converged = true;
       break;
     }
   }
-  __syncthreads();
-  if (tid == 0 && !converged) atomicMax(&status[b], (int)TC_ERR_NOT_CONVERGED);
+  everyone();
+  if (rank == 0 && tid == 0 && !converged) atomicMax(&status[b], (int)TC_ERR_NOT_CONVERGED);
 
   // eigenvalues = column norms of W;  eigenvectors = columns of J, written as ZT[p][i]
-  for (int p = warp; p < n; p += 16) {
+  for (int p = gwarp; p < n; p += gwarps) {
     float a = 0.f;
     for (int r = lane; r < n; r += 32) {
       const float v = W[(size_t)p * n + r];
@@ -483,41 +518,53 @@ __global__ void __launch_bounds__(512) jacobi_kernel(const float* __restrict__ H
     for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     if (lane == 0) theta[(size_t)b * n + p] = sqrtf(a);
   }
-  if (use_smem) {
+  if constexpr (CL == 1) {
     float* out = ZTg + b * nn;
-    for (size_t e = tid; e < nn; e += 512) out[e] = J[e];
+    for (size_t e = tid; e < nn; e += nt) out[e] = J[e];
   }
 }
 
-typedef void (*jacobi_fn)(const float*, int, float*, float*, float*, int, int, float, int, int32_t*, float, float);
+typedef void (*jacobi_fn)(const float*, int, float*, float*, float*, int, int, float, int32_t*, float, float);
 
-static jacobi_fn pick_jacobi(int n) {
+// (two matrices of up to 167 columns fit in shared memory)
+static jacobi_fn pick_jacobi(int n, bool use_smem, int cl) {
   const int r = (n + 31) / 32;
-  if (r <= 1) return jacobi_kernel<1>;
-  if (r <= 2) return jacobi_kernel<2>;
-  if (r <= 3) return jacobi_kernel<3>;
-  if (r <= 4) return jacobi_kernel<4>;
-  if (r <= 5) return jacobi_kernel<5>;
-  if (r <= 6) return jacobi_kernel<6>;
-  if (r <= 8) return jacobi_kernel<8>;
-  if (r <= 10) return jacobi_kernel<10>;
-  if (r <= 14) return jacobi_kernel<14>;
-  if (r <= 18) return jacobi_kernel<18>;
-  if (r <= 24) return jacobi_kernel<24>;
-  if (r <= 32) return jacobi_kernel<32>;
+  if (use_smem) {
+    if (r <= 1) return jacobi_kernel<1, 1>;
+    if (r <= 2) return jacobi_kernel<2, 1>;
+    if (r <= 3) return jacobi_kernel<3, 1>;
+    if (r <= 4) return jacobi_kernel<4, 1>;
+    if (r <= 5) return jacobi_kernel<5, 1>;
+    if (r <= 6) return jacobi_kernel<6, 1>;
+    return nullptr;
+  }
+  if (r <= 6) return cl == 8 ? jacobi_kernel<6, 8> : jacobi_kernel<6, 16>;
+  if (r <= 8) return cl == 8 ? jacobi_kernel<8, 8> : jacobi_kernel<8, 16>;
+  if (r <= 10) return cl == 8 ? jacobi_kernel<10, 8> : jacobi_kernel<10, 16>;
+  if (r <= 14) return jacobi_kernel<14, 16>;
+  if (r <= 18) return jacobi_kernel<18, 16>;
+  if (r <= 24) return jacobi_kernel<24, 16>;
+  if (r <= 32) return jacobi_kernel<32, 16>;
   return nullptr;
 }
 
 constexpr size_t SMEM_LIMIT = 220 * 1024;  // leaves room for the static shared variables
 
-static void launch_jacobi(const float* H, int ldh, float* W, float* ZT, float* theta, int n, int batch,
+static tc_status launch_jacobi(const float* H, int ldh, float* W, float* ZT, float* theta, int n, int batch,
                           int max_sweeps, float rank_tol, int32_t* status, cudaStream_t st) {
   Scope scope_(KC_JACOBI, st);
-  jacobi_fn fn = pick_jacobi(n);
   const size_t need = 2 * (size_t)n * n * sizeof(float);
-  const int use_smem = need <= SMEM_LIMIT;
+  const bool use_smem = need <= SMEM_LIMIT;
   const size_t smem = use_smem ? need : 0;
-  if (use_smem) cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // up to 20 warps a block take a round's n / 2 pairs, one each up to 640 columns
+  const int pairs = (n + 1) / 2, cl = use_smem ? 1 : pairs <= 160 ? 8 : 16;
+  const int warps = use_smem ? 32 : min(JACOBI_CL_THREADS / 32, (pairs + cl - 1) / cl);
+  jacobi_fn fn = pick_jacobi(n, use_smem, cl);
+  if (fn == nullptr) return TC_ERR_UNSUPPORTED;
+  if (use_smem && cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return TC_ERR_CUDA;
+  if (cl > 8 && cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+    return TC_ERR_CUDA;
   // off-diagonal threshold a little above the rounding noise of a length-n float32 dot product
   const float tol = fmaxf(1e-6f, 2.5f * sqrtf((float)n) * 1.1920929e-7f);
   // Eigenvalue floors, relative to the largest diagonal entry.  Column pairs that are both
@@ -526,16 +573,31 @@ static void launch_jacobi(const float* H, int ldh, float* W, float* ZT, float* t
   // towards "this sweep still rotated".
   const float floor_rel = 1e-6f;
   const float count_rel = fmaxf(floor_rel, rank_tol * rank_tol);
-  { fn<<<batch, 512, smem, st>>>(H, ldh, W, ZT, theta, n, max_sweeps, tol, use_smem, status, floor_rel, count_rel); note_launch(); }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(batch * cl));
+  cfg.blockDim = dim3((unsigned)(warps * 32));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)cl;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = cl > 1 ? 1 : 0;
+  if (cudaLaunchKernelEx(&cfg, fn, H, ldh, W, ZT, theta, n, max_sweeps, tol, status, floor_rel, count_rel) != cudaSuccess)
+    return TC_ERR_CUDA;
+  note_launch();
+  return TC_OK;
 }
 
-// Which solver decomposes an n x n matrix.  Inverse iteration does not orthogonalise eigenvectors
-// against each other, which is fine while the wanted eigenvalues (rank_tol^2 theta_max and up) stand
-// clear of the float32 rounding level of the largest, about 1e-6 of it: from rank_tol = 1e-3 on.
-// Below that the full solve, and a subspace wider than 224, take Jacobi sweeps, whose vectors are
-// orthogonal whatever the spectrum, at a hundred times the time.  Eigenvalues alone need no such care.
+// Which solver decomposes an n x n matrix.  The vectors of the full solve come from Jacobi sweeps: they
+// are orthogonal whatever the spectrum, and img_status says of every image whether its sweeps ended.
+// So does a subspace wider than 224 with rank_tol under 1e-3: inverse iteration does not orthogonalise
+// eigenvectors against each other, which is fine while the wanted eigenvalues (rank_tol^2 theta_max and
+// up) stand clear of the float32 rounding level of the largest, about 1e-6 of it.  Eigenvalues alone
+// need no such care.
 static bool use_tridiag(int n, bool full, bool values_only, float rank_tol) {
-  return eig_tridiag_supported(n) && (values_only || rank_tol >= 1e-3f || (!full && n <= 224));
+  return eig_tridiag_supported(n) && (values_only || (!full && (rank_tol >= 1e-3f || n <= 224)));
 }
 
 // ==========================================================================================
@@ -724,11 +786,12 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
 
   if (D.full) {
     if (io.g_ready) cudaStreamWaitEvent(st, io.g_ready, 0);
-    if (use_tridiag(N, true, io.values_only, D.rank_tol)) {
+    if (use_tridiag(N, cap == 0, io.values_only, D.rank_tol)) {   // (a bound that left no subspace is not the full solve)
       tc_status e = launch_eig_tridiag(G, sG, ldn, N, B, D.rank_tol, theta, ZT, sK, N, W, img_status, st);
       if (e != TC_OK) return e;
     } else {
-      launch_jacobi(G, ldn, W, ZT, theta, N, B, D.max_sweeps, D.rank_tol, img_status, st);
+      const tc_status e = launch_jacobi(G, ldn, W, ZT, theta, N, B, D.max_sweeps, D.rank_tol, img_status, st);
+      if (e != TC_OK) return e;
     }
     scores(ZT, N, nullptr);
     return TC_OK;
@@ -847,7 +910,8 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
     tc_status e = launch_eig_tridiag(Hm, sK, k, k, B, D.rank_tol, theta, ZT, sK, k, W, img_status, st);
     if (e != TC_OK) return e;
   } else {
-    launch_jacobi(Hm, k, W, ZT, theta, k, B, D.max_sweeps, D.rank_tol, img_status, st);
+    const tc_status e = launch_jacobi(Hm, k, W, ZT, theta, k, B, D.max_sweeps, D.rank_tol, img_status, st);
+    if (e != TC_OK) return e;
   }
   // 5. eigenvectors of G restricted to the subspace:  PT[p][x] = sum_i ZT[p][i] Q1[x][i]
   gemm<float, float, false, true>(ZT, Y2, Y0, k, N, k, k, k, N, sK, sY, sY, B, st);
