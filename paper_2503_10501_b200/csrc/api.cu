@@ -167,6 +167,7 @@ Plan make_plan(const Dims& D) {
     P.W = take(B * jacobi_work_bytes(D.k));
     P.ZT = take(B * k * k * 4);
   }
+  if (D.full) P.rot = take(B * jacobi_rot_bytes(D.N));
   P.setA = take(B * (size_t)(D.nA > 0 ? D.nA : 1) * 4);
   P.setB = take(B * (size_t)D.nB * 4);
   P.best_val = take(B * (size_t)D.nB * 4);

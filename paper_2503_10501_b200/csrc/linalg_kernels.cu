@@ -524,6 +524,251 @@ __global__ void __launch_bounds__(CL == 1 ? 1024 : JACOBI_CL_THREADS) jacobi_ker
   }
 }
 
+// ------------------------------------------------------------------------------------------
+// The same sweeps for 97 to 660 columns, with W in the shared memory of a cluster, and J apart:
+//   jacobi_sweep_kernel   a sweep over W.  Block `rank` holds the columns of its pairs (slots), a warp
+//                         per slot.  In the tournament the first player of slot s moves to slot s - 1,
+//                         the second to s + 1, so a pair's columns are written to where the next
+//                         round reads them, those at the edges into the neighbouring block, and a
+//                         cluster barrier ends the round.  The rotations of the sweep go to `rot`.
+//   jacobi_replay_kernel  the sweep's rotations on J, whose rows do not depend on one another: eight
+//                         rows per block in shared memory.
+// Every number comes from the same operations in the same order as in jacobi_kernel.
+// What bounds it is a round: 83 KB of W through each SM's shared memory and back, the scalar chain of a
+// rotation, the barrier.  Measured, 2 images of 576, 30 sweeps: 77 ms (both matrices out of L2) ->
+// 47 ms, 3 of them the replays.
+// ------------------------------------------------------------------------------------------
+struct JacobiState {
+  float md;        // largest diagonal entry of the matrix
+  int sweeps;      // sweeps done
+  int converged;
+};
+
+__global__ void __launch_bounds__(1024) jacobi_begin_kernel(const float* __restrict__ Hin, int ldh, float* __restrict__ Wg,
+                                                           float* __restrict__ Jg, int n, JacobiState* __restrict__ state) {
+  __shared__ float s_red[32];
+  const size_t b = blockIdx.y, nn = (size_t)n * n;
+  const float* Hb = Hin + b * (size_t)n * ldh;
+  pdl_wait();
+  for (size_t e = blockIdx.x * 1024 + threadIdx.x; e < nn; e += (size_t)gridDim.x * 1024) {
+    const int p = (int)(e / n), i = (int)(e % n);
+    Wg[b * nn + e] = 0.5f * (Hb[(size_t)p * ldh + i] + Hb[(size_t)i * ldh + p]);
+    Jg[b * nn + e] = (p == i) ? 1.f : 0.f;
+  }
+  if (blockIdx.x != 0) return;
+  float md = 0.f;
+  for (int i = threadIdx.x; i < n; i += 1024) md = fmaxf(md, fabsf(0.5f * (Hb[(size_t)i * ldh + i] + Hb[(size_t)i * ldh + i])));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) md = fmaxf(md, __shfl_xor_sync(0xffffffffu, md, o));
+  if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = md;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 32; ++w) md = fmaxf(md, s_red[w]);
+    state[b].md = md;
+    state[b].sweeps = 0;
+    state[b].converged = 0;
+  }
+}
+
+template <int R, int CL>
+__global__ void __launch_bounds__(672) jacobi_sweep_kernel(float* __restrict__ Wg, float2* __restrict__ rot, int n, float tol,
+                                                         float floor_rel, float count_rel, JacobiState* __restrict__ state) {
+  extern __shared__ float sm[];   // [2 buffers][warps][first, second][32 R]
+  __shared__ int s_rot;
+  constexpr int LEN = 32 * R;
+  const int rank = (int)(blockIdx.x % CL), b = blockIdx.x / CL, warps = blockDim.x / 32;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int half = (n + 1) / 2, m = 2 * half - 1;
+  const int slot = rank * warps + warp;
+  const bool live = slot < half;
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  pdl_wait();
+  const JacobiState st = state[b];
+  if (st.converged) return;   // (all blocks of the cluster alike)
+  float* W = Wg + (size_t)b * n * n;
+  const float floor1 = floor_rel * st.md, floor2 = floor1 * floor1;
+  const float count_floor2 = (count_rel * st.md) * (count_rel * st.md);
+  auto local = [&](int w, int which, int buf) { return sm + (size_t)((buf * warps + w) * 2 + which) * LEN; };
+  // a column to where it plays next, in this block or in a neighbour
+  auto put = [&](const float (&x)[R], int s, int which, int buf) {
+    if (s / warps == rank) {
+      float* d = local(s % warps, which, buf);
+#pragma unroll
+      for (int i = 0; i < R; ++i) d[lane + 32 * i] = x[i];
+    } else {
+      float* d = cl.map_shared_rank(local(s % warps, which, buf), s / warps);
+#pragma unroll
+      for (int i = 0; i < R; ++i) d[lane + 32 * i] = x[i];
+    }
+  };
+  auto players = [&](int round, int& u, int& v) {
+    u = round + slot;
+    if (u >= m) u -= m;
+    v = round - slot;
+    if (v < 0) v += m;
+    if (slot == 0) {
+      u = round;
+      v = m;
+    }
+  };
+  if (threadIdx.x == 0) s_rot = 0;
+  float wu[R], wv[R];
+  if (live) {
+    int u, v;
+    players(0, u, v);
+    float *du = local(warp, 0, 0), *dv = local(warp, 1, 0);
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int r = lane + 32 * i;
+      du[r] = r < n ? W[(size_t)u * n + r] : 0.f;
+      dv[r] = r < n && v < n ? W[(size_t)v * n + r] : 0.f;
+    }
+  }
+  cl.sync();
+  int count = 0;
+  float2* out = rot + (size_t)b * m * half + slot;
+  for (int round = 0; round < m; ++round) {
+    if (live) {
+      int u, v;
+      players(round, u, v);
+      const float *su = local(warp, 0, round & 1), *sv = local(warp, 1, round & 1);
+      float a = 0.f, bq = 0.f, g = 0.f;
+      // p is the column of the lower number
+      const bool swap = u > v;
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        wu[i] = su[lane + 32 * i];
+        wv[i] = sv[lane + 32 * i];
+      }
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        a = fmaf(wu[i], wu[i], a);
+        bq = fmaf(wv[i], wv[i], bq);
+        g = fmaf(wu[i], wv[i], g);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        bq += __shfl_xor_sync(0xffffffffu, bq, o);
+        g += __shfl_xor_sync(0xffffffffu, g, o);
+      }
+      if (swap) {
+        const float t = a;
+        a = bq;
+        bq = t;
+      }
+      const float nn = sqrtf(a) * sqrtf(bq);
+      float2 cs = make_float2(1.f, 0.f);
+      if (v < n && fabsf(g) > tol * nn && fmaxf(a, bq) > floor2) {
+        const float zeta = (bq - a) / (2.0f * g);
+        const float t = copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.0f)));
+        const float c = rsqrtf(fmaf(t, t, 1.0f));
+        const float s = c * t;
+        cs = make_float2(c, s);
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          const float wp = swap ? wv[i] : wu[i], wq = swap ? wu[i] : wv[i];
+          const float np = c * wp - s * wq, nq = fmaf(s, wp, c * wq);
+          wu[i] = swap ? nq : np;
+          wv[i] = swap ? np : nq;
+        }
+        count += fmaxf(a, bq) > count_floor2 ? 1 : 0;
+      }
+      if (lane == 0) out[(size_t)round * half] = cs;
+      // slot 0: the first player turns into the second of slot 1, the second stays; the last slot: the
+      // second player turns into the first
+      const int next = (round + 1) & 1;
+      put(wu, slot == 0 ? 1 : slot - 1, slot == 0 ? 1 : 0, next);
+      put(wv, slot == 0 || slot == half - 1 ? slot : slot + 1, slot == half - 1 ? 0 : 1, next);
+    }
+    cl.sync();
+  }
+  if (lane == 0 && count) atomicAdd(cl.map_shared_rank(&s_rot, 0), count);
+  if (live) {   // after m rounds the players are where they began
+    int u, v;
+    players(0, u, v);
+    const float *su = local(warp, 0, m & 1), *sv = local(warp, 1, m & 1);
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int r = lane + 32 * i;
+      if (r < n) {
+        W[(size_t)u * n + r] = su[r];
+        if (v < n) W[(size_t)v * n + r] = sv[r];
+      }
+    }
+  }
+  cl.sync();
+  if (rank == 0 && threadIdx.x == 0) {
+    state[b].sweeps = st.sweeps + 1;
+    state[b].converged = s_rot == 0;
+  }
+}
+
+constexpr int REPLAY_ROWS = 8;
+// grid (row groups, images), 512 threads: 64 pairs x 8 rows
+__global__ void __launch_bounds__(512) jacobi_replay_kernel(float* __restrict__ Jg, const float2* __restrict__ rot, int n, int sweep,
+                                                           const JacobiState* __restrict__ state) {
+  extern __shared__ float js[];   // [n + 1][8]
+  constexpr int SLOTS = 6;        // of a thread: up to 64 x 6 pairs
+  const int b = blockIdx.y, r0 = blockIdx.x * REPLAY_ROWS, row = threadIdx.x & 7, first = threadIdx.x >> 3;
+  const int half = (n + 1) / 2, m = 2 * half - 1;
+  pdl_wait();
+  if (state[b].sweeps <= sweep) return;   // (the sweeps had ended before)
+  float* J = Jg + (size_t)b * n * n;
+  const bool there = r0 + row < n;
+  for (int c = first; c < n; c += 64) js[c * 8 + row] = there ? J[(size_t)c * n + r0 + row] : 0.f;
+  const float2* list = rot + (size_t)b * m * half;
+  float2 cs[SLOTS];
+#pragma unroll
+  for (int k = 0; k < SLOTS; ++k) cs[k] = first + 64 * k < half ? __ldg(list + first + 64 * k) : make_float2(1.f, 0.f);
+  __syncthreads();
+  for (int round = 0; round < m; ++round) {
+    float2 now[SLOTS];
+#pragma unroll
+    for (int k = 0; k < SLOTS; ++k) {
+      now[k] = cs[k];
+      if (round + 1 < m && first + 64 * k < half) cs[k] = __ldg(list + (size_t)(round + 1) * half + first + 64 * k);
+    }
+#pragma unroll
+    for (int k = 0; k < SLOTS; ++k) {
+      const int slot = first + 64 * k;
+      if (slot >= half || now[k].y == 0.f) continue;
+      int u = round + slot, v = round - slot;
+      if (u >= m) u -= m;
+      if (v < 0) v += m;
+      if (slot == 0) {
+        u = round;
+        v = m;
+      }
+      const int p = min(u, v), q = max(u, v);
+      const float c = now[k].x, s = now[k].y, jp = js[p * 8 + row], jq = js[q * 8 + row];
+      js[p * 8 + row] = c * jp - s * jq;
+      js[q * 8 + row] = fmaf(s, jp, c * jq);
+    }
+    __syncthreads();
+  }
+  if (there)
+    for (int c = first; c < n; c += 64) J[(size_t)c * n + r0 + row] = js[c * 8 + row];
+}
+
+// eigenvalues = column norms of W; a warp per column
+__global__ void __launch_bounds__(256) jacobi_end_kernel(const float* __restrict__ Wg, float* __restrict__ theta, int n,
+                                                        const JacobiState* __restrict__ state, int32_t* __restrict__ status) {
+  const int b = blockIdx.y, p = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0 && !state[b].converged) atomicMax(&status[b], (int)TC_ERR_NOT_CONVERGED);
+  if (p >= n) return;
+  float a = 0.f;
+  for (int r = lane; r < n; r += 32) {
+    const float v = Wg[(size_t)b * n * n + (size_t)p * n + r];
+    a = fmaf(v, v, a);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  if (lane == 0) theta[(size_t)b * n + p] = sqrtf(a);
+}
+
 typedef void (*jacobi_fn)(const float*, int, float*, float*, float*, int, int, float, int32_t*, float, float);
 
 // (two matrices of up to 167 columns fit in shared memory)
@@ -550,21 +795,31 @@ static jacobi_fn pick_jacobi(int n, bool use_smem, int cl) {
 
 constexpr size_t SMEM_LIMIT = 220 * 1024;  // leaves room for the static shared variables
 
+typedef void (*sweep_fn)(float*, float2*, int, float, float, float, JacobiState*);
+struct sweep_pick {
+  sweep_fn fn;
+  int len;   // floats of a column in shared memory
+};
+static sweep_pick pick_sweep(int n) {
+  if (n <= 128) return {jacobi_sweep_kernel<4, 8>, 128};
+  if (n <= 192) return {jacobi_sweep_kernel<6, 8>, 192};
+  if (n <= 256) return {jacobi_sweep_kernel<8, 8>, 256};
+  if (n <= 320) return {jacobi_sweep_kernel<10, 8>, 320};
+  if (n <= 448) return {jacobi_sweep_kernel<14, 16>, 448};
+  if (n <= 576) return {jacobi_sweep_kernel<18, 16>, 576};
+  return {jacobi_sweep_kernel<21, 16>, 672};
+}
+// Bytes per image that the sweeps over a cluster's shared memory want (none: another size's kernel)
+size_t jacobi_rot_bytes(int n) {
+  if (n < 97 || n > 672) return 0;
+  const size_t half = (n + 1) / 2;
+  return ((2 * half - 1) * half * sizeof(float2) + sizeof(JacobiState) + 15) / 16 * 16;
+}
+
 static tc_status launch_jacobi(const float* H, int ldh, float* W, float* ZT, float* theta, int n, int batch,
-                          int max_sweeps, float rank_tol, int32_t* status, cudaStream_t st) {
+                          int max_sweeps, float rank_tol, float2* rot, JacobiState* state, int32_t* status,
+                          cudaStream_t st) {
   Scope scope_(KC_JACOBI, st);
-  const size_t need = 2 * (size_t)n * n * sizeof(float);
-  const bool use_smem = need <= SMEM_LIMIT;
-  const size_t smem = use_smem ? need : 0;
-  // up to 20 warps a block take a round's n / 2 pairs, one each up to 640 columns
-  const int pairs = (n + 1) / 2, cl = use_smem ? 1 : pairs <= 160 ? 8 : 16;
-  const int warps = use_smem ? 32 : min(JACOBI_CL_THREADS / 32, (pairs + cl - 1) / cl);
-  jacobi_fn fn = pick_jacobi(n, use_smem, cl);
-  if (fn == nullptr) return TC_ERR_UNSUPPORTED;
-  if (use_smem && cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return TC_ERR_CUDA;
-  if (cl > 8 && cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-    return TC_ERR_CUDA;
   // off-diagonal threshold a little above the rounding noise of a length-n float32 dot product
   const float tol = fmaxf(1e-6f, 2.5f * sqrtf((float)n) * 1.1920929e-7f);
   // Eigenvalue floors, relative to the largest diagonal entry.  Column pairs that are both
@@ -573,6 +828,43 @@ static tc_status launch_jacobi(const float* H, int ldh, float* W, float* ZT, flo
   // towards "this sweep still rotated".
   const float floor_rel = 1e-6f;
   const float count_rel = fmaxf(floor_rel, rank_tol * rank_tol);
+  const int pairs = (n + 1) / 2;
+  // (a launch or two per sweep, so not for bounds on the sweeps that are none)
+  if (rot != nullptr && max_sweeps <= 100) {
+    const int cl = n <= 320 ? 8 : 16, warps = (pairs + cl - 1) / cl;
+    const sweep_pick pk = pick_sweep(n);
+    const size_t smem = (size_t)4 * warps * pk.len * sizeof(float);
+    if (cudaFuncSetAttribute((const void*)pk.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        (cl > 8 && cudaFuncSetAttribute((const void*)pk.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess))
+      return TC_ERR_CUDA;
+    launch_pdl(jacobi_begin_kernel, dim3(16, batch), dim3(1024), 0, st, 0, H, ldh, W, ZT, n, state);
+    note_launch();
+    for (int sweep = 0; sweep < max_sweeps; ++sweep) {
+      if (launch_pdl(pk.fn, dim3((unsigned)(batch * cl)), dim3((unsigned)(warps * 32)), smem, st, cl, W, rot, n, tol, floor_rel,
+                     count_rel, state) != cudaSuccess)
+        return TC_ERR_CUDA;
+      note_launch();
+      launch_pdl(jacobi_replay_kernel, dim3((unsigned)((n + REPLAY_ROWS - 1) / REPLAY_ROWS), batch), dim3(512),
+                 (size_t)n * REPLAY_ROWS * sizeof(float), st, 0, ZT, (const float2*)rot, n, sweep, (const JacobiState*)state);
+      note_launch();
+    }
+    launch_pdl(jacobi_end_kernel, dim3((n + 7) / 8, batch), dim3(256), 0, st, 0, (const float*)W, theta, n,
+               (const JacobiState*)state, status);
+    note_launch();
+    return TC_OK;
+  }
+  const size_t need = 2 * (size_t)n * n * sizeof(float);
+  const bool use_smem = need <= SMEM_LIMIT;
+  const size_t smem = use_smem ? need : 0;
+  // up to 20 warps a block take a round's n / 2 pairs, one each up to 640 columns
+  const int cl = use_smem ? 1 : pairs <= 160 ? 8 : 16;
+  const int warps = use_smem ? 32 : min(JACOBI_CL_THREADS / 32, (pairs + cl - 1) / cl);
+  jacobi_fn fn = pick_jacobi(n, use_smem, cl);
+  if (fn == nullptr) return TC_ERR_UNSUPPORTED;
+  if (use_smem && cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return TC_ERR_CUDA;
+  if (cl > 8 && cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+    return TC_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(batch * cl));
   cfg.blockDim = dim3((unsigned)(warps * 32));
@@ -790,7 +1082,11 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
       tc_status e = launch_eig_tridiag(G, sG, ldn, N, B, D.rank_tol, theta, ZT, sK, N, W, img_status, st);
       if (e != TC_OK) return e;
     } else {
-      const tc_status e = launch_jacobi(G, ldn, W, ZT, theta, N, B, D.max_sweeps, D.rank_tol, img_status, st);
+      const size_t rb = jacobi_rot_bytes(N), half = (N + 1) / 2;
+      // (the batch's lists, then its states; groups have theirs apart)
+      float2* rot = rb ? (float2*)(ws + P.rot + b0 * rb) : nullptr;
+      JacobiState* jst = rb ? (JacobiState*)(rot + (size_t)B * (2 * half - 1) * half) : nullptr;
+      const tc_status e = launch_jacobi(G, ldn, W, ZT, theta, N, B, D.max_sweeps, D.rank_tol, rot, jst, img_status, st);
       if (e != TC_OK) return e;
     }
     scores(ZT, N, nullptr);
@@ -910,7 +1206,7 @@ tc_status launch_ics(const Dims& D, const Plan& P, char* ws, int b0, const void*
     tc_status e = launch_eig_tridiag(Hm, sK, k, k, B, D.rank_tol, theta, ZT, sK, k, W, img_status, st);
     if (e != TC_OK) return e;
   } else {
-    const tc_status e = launch_jacobi(Hm, k, W, ZT, theta, k, B, D.max_sweeps, D.rank_tol, img_status, st);
+    const tc_status e = launch_jacobi(Hm, k, W, ZT, theta, k, B, D.max_sweeps, D.rank_tol, nullptr, nullptr, img_status, st);
     if (e != TC_OK) return e;
   }
   // 5. eigenvectors of G restricted to the subspace:  PT[p][x] = sum_i ZT[p][i] Q1[x][i]

@@ -51,6 +51,7 @@ struct Plan {
   size_t Y0, Y1, Y2;  // [B, N, k] f32 each (subspace solve only)
   size_t Sm, Rinv, Hm;  // [B, k, k] f32 each (subspace solve only)
   size_t W, ZT;    // [B] work array of the eigen-solver; [B, k, k] f32 eigenvectors
+  size_t rot;      // [B] rotations of a Jacobi sweep (full solve)
   size_t setA, setB, best_val, best_dst, msrc, mdst, kept;  // int32 / f32 lists
   size_t rank;     // [B] int32
   size_t flags;    // [B] int32 device status scratch
@@ -207,6 +208,7 @@ tc_status launch_eig_tridiag(const float* H, size_t sH, int ldh, int n, int batc
                              float* ZT, size_t sZ, int ldz, void* scratch, int32_t* status, cudaStream_t st);
 
 // bytes per image of the work array of either eigen-solver (the Jacobi work matrix is k x k)
+size_t jacobi_rot_bytes(int n);   // rotations of a sweep, per image
 inline size_t jacobi_work_bytes(int k) { return align_up(eig_tridiag_scratch_bytes(k), 256); }
 
 // Eigen-decomposition of G and Eq. 3-6:  C, theta (unsorted), then sorted sigma / rank; on the raw

@@ -51,8 +51,8 @@ def test_eigenvalues_of_every_layout(N):
         assert int(g["rank"][b]) == int((s > 2e-3 * s[0]).sum())
 
 
-# full solves: one block with both matrices in shared memory, clusters of both sizes, byes, the largest
-@pytest.mark.parametrize("N", [3, 4, 33, 96, 97, 130, 167, 168, 193, 320, 321, 449, 640, 661, 700])
+# full solves: one block, W in the shared memory of clusters of either size (every column length, byes), out of L2
+@pytest.mark.parametrize("N", [3, 4, 33, 96, 97, 128, 129, 193, 257, 320, 321, 449, 576, 577, 672, 673, 700])
 def test_full_solve(N):
     _check(N, 832, max(2, min(N // 3, 200)), 0, seed=N)
 
