@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(Z_THREADS, 1) probe_z_kernel(
     int32_t* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bar_q[2], bar_k[2], bar_kfree[2], bar_v[2], bar_vfree[2];   // (the last four by stage)
-  __shared__ __align__(8) uint64_t bar_s[2][2], bar_p[2][2], bar_pv[2];   // by query tile: scores ready; P written (both by buffer); P V done
+  __shared__ __align__(8) uint64_t bar_s[2][2], bar_p[2][2], bar_pv[2][2];   // by query tile and buffer: scores ready; P written; P V done
   __shared__ uint32_t s_tmem;
   __shared__ int s_fail;
 
@@ -183,8 +183,8 @@ __global__ void __launch_bounds__(Z_THREADS, 1) probe_z_kernel(
       for (int u = 0; u < 2; ++u) {
         mbar_init(smem_u32(&bar_s[i][u]), 1);
         mbar_init(smem_u32(&bar_p[i][u]), 4);
+        mbar_init(smem_u32(&bar_pv[i][u]), 1);
       }
-      mbar_init(smem_u32(&bar_pv[i]), 1);
     }
     s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -199,8 +199,7 @@ __global__ void __launch_bounds__(Z_THREADS, 1) probe_z_kernel(
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   auto tmem_s = [&](int t, int i) { return s_tmem + (uint32_t)t * 128u + ((uint32_t)i & 1u) * 64u; };
   auto tmem_o = [&](int t) { return s_tmem + 256u + (uint32_t)t * 128u; };
-  auto phase = [](int i) { return (uint32_t)i & 1u; };               // of a barrier without stages
-  auto sphase = [](int i) { return ((uint32_t)i >> 1) & 1u; };       // of one with two
+  auto sphase = [](int i) { return ((uint32_t)i >> 1) & 1u; };
 
   if (warp == Z_TMA) {
     if (lane == 0) {
@@ -231,7 +230,7 @@ __global__ void __launch_bounds__(Z_THREADS, 1) probe_z_kernel(
       const int s = (i >> 1) & 1;
       if (i == 0 && !mbar_wait(smem_u32(&bar_q[t]), 0)) return false;
       if ((i & 1) == 0 && !mbar_wait(smem_u32(&bar_k[s]), sphase(i >> 1))) return false;
-      if (i >= 2 && !mbar_wait(smem_u32(&bar_pv[t]), phase(i - 2))) return false;
+      if (i >= 2 && !mbar_wait(smem_u32(&bar_pv[t][i & 1]), sphase(i - 2))) return false;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (elect_one()) {
         mma_tile(tmem_s(t, i), sQ(t), sK(s) + ((uint32_t)i & 1u) * (SB * 128u), id_s);
@@ -248,7 +247,7 @@ __global__ void __launch_bounds__(Z_THREADS, 1) probe_z_kernel(
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (elect_one()) {
         mma_tile_pv(tmem_o(t), tmem_s(t, i), sV(s) + ((uint32_t)i & 1u) * (SB * 128u), id_o, i > 0);
-        umma_commit(smem_u32(&bar_pv[t]));
+        umma_commit(smem_u32(&bar_pv[t][i & 1]));
         if ((i & 1) || i == n - 1) umma_commit(smem_u32(&bar_vfree[s]));
       }
       __syncwarp();
@@ -293,7 +292,7 @@ __global__ void __launch_bounds__(Z_THREADS, 1) probe_z_kernel(
           m = m_new;
           l *= alpha;
           if (i > 0) {
-            if (ok && !mbar_wait(smem_u32(&bar_pv[t]), phase(i - 1))) ok = false;
+            if (ok && !mbar_wait(smem_u32(&bar_pv[t][(i - 1) & 1]), sphase(i - 1))) ok = false;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
             for (int c = 0; c < DH / 32; ++c) {
@@ -329,7 +328,8 @@ __global__ void __launch_bounds__(Z_THREADS, 1) probe_z_kernel(
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_p[t][i & 1])) : "memory");
     }
     if (n > 0) {
-      if (ok && !mbar_wait(smem_u32(&bar_pv[t]), phase(n - 1))) ok = false;
+      // (by buffer, since a thread that has the last scores knows of the product three steps back, not two)
+      if (ok && !mbar_wait(smem_u32(&bar_pv[t][(n - 1) & 1]), sphase(n - 1))) ok = false;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (!ok) s_fail = 1;
       // The rows leave through the tile's query tile (its last scores are formed): a thread owns a row,

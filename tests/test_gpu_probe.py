@@ -106,10 +106,11 @@ def test_probe_rejects_unsupported_shapes():
 
 # visual rows that fill one query tile, one more, and a pair; steps of 64 keys with one and two tiles
 @pytest.mark.parametrize("n_sys,N,n_text,T", [(0, 1, 1, 1), (0, 64, 1, 1), (63, 2, 1, 1), (1, 128, 7, 8), (0, 129, 3, 2), (10, 256, 1, 129),
-                                              (70, 257, 130, 128)])
-def test_probe_tile_edges(n_sys, N, n_text, T):
+                                              (70, 257, 130, 128), (16, 194, 105, 52), (0, 448, 9, 9)])
+@pytest.mark.parametrize("H", [2, 24])
+def test_probe_tile_edges(H, n_sys, N, n_text, T):
     L = n_sys + N + n_text
-    _check(B=1, H=2, n_sys=n_sys, N=N, n_text=n_text, probe_start=L - T, T=T, dtype="f16", seed=N)
+    _check(B=1, H=H, n_sys=n_sys, N=N, n_text=n_text, probe_start=L - T, T=T, dtype="f16", seed=N)
 
 
 def test_probe_maximum_that_keeps_growing():
