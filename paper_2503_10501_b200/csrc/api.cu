@@ -196,6 +196,14 @@ tc_status launch_gram(const Dims& D, const void* O, float* G, int ldg, int32_t* 
   return launch_gemm_f32x3(op, op, D.N, ldg, D.d, D.B, D.call_B, R, status, st, KC_GRAM);
 }
 
+// The Gram matrix of the scores.  The full solve and the widest subspaces report in img_status what hangs
+// on the last bits of it (sweeps that go on over rounding noise, pivots at the rounding level): their
+// float32 products keep the plain order of multiply-adds, less than a hundredth of those solves.
+static tc_status score_gram(const Dims& D, const void* O, float* G, int ldg, int32_t* status, cudaStream_t st) {
+  if (!D.tcp && !D.f16 && !D.bf16) return launch_gram_simt(D, O, G, ldg, st);
+  return launch_gram(D, O, G, ldg, status, st);
+}
+
 // Eq. 3-10 on the rows of F [B, N, f]: all products of two tokens on the tensor cores, of which the
 // matching reads its own.  (A warp per pair of tokens, on the plain ALUs, took four times as long at
 // 8 images of 576 tokens and d = 4096: 245 us, 64 for both launches here.)
@@ -333,11 +341,11 @@ static tc_status enqueue_score(const Ctx& c, const void* O, const void* A, float
     if (!D.full) {
       cudaStreamWaitEvent(gs->s2[g], gs->fork, 0);
       if (late) cudaStreamWaitEvent(gs->s2[g], gs->gram_done[g - per_wave], 0);
-      err = launch_gram(Dg, Og, Gg, D.ldn, img_status + b0, gs->s2[g]);
+      err = score_gram(Dg, Og, Gg, D.ldn, img_status + b0, gs->s2[g]);
       cudaEventRecord(gs->gram_done[g], gs->s2[g]);
       io.g_ready = gs->gram_done[g];
     } else {
-      err = launch_gram(Dg, Og, Gg, D.ldn, img_status + b0, st);
+      err = score_gram(Dg, Og, Gg, D.ldn, img_status + b0, st);
     }
     if (err == TC_OK)
       err = launch_ics(Dg, c.P, c.ws, b0, Og, io, st);
