@@ -335,8 +335,8 @@ tc_status tc_rope_tables(const int32_t* pos, int64_t n_rows, int32_t head_dim, f
                          float* cos_out, float* sin_out, void* stream);
 
 /*
- * Number of image groups tc_score / tc_carve run side by side (1..16, default 4; the paper has
- * no counterpart).  The batch is cut into that many contiguous groups whose chains (Gram ->
+ * Number of image groups tc_score / tc_carve run side by side (1..16; the paper has no
+ * counterpart).  Until it is called, the batch decides: one under 32 images, two under 64, else four.  The batch is cut into that many contiguous groups whose chains (Gram ->
  * eigen-solve -> scores, and in tc_carve the selection and gather as well) are enqueued on
  * internal streams forked from `stream` and joined back into it, so that the
  * one-block-per-image solver kernels of one group overlap the products of another.  With four
