@@ -346,8 +346,8 @@ tc_status tc_rope_tables(const int32_t* pos, int64_t n_rows, int32_t head_dim, f
  * Results do not depend on the setting.  The setting is process-wide state (one value for all
  * threads and devices), and calls that use groups are serialised on a lock while they enqueue.
  * Each group costs the host a few dozen launches per call: more than four groups pay only when
- * the call is replayed from a CUDA graph, where sixteen is the measured optimum at B = 64
- * (1.29 ms per carve against 1.31 ms with eight and 1.35 ms with eight in one wave).
+ * the call is replayed from a CUDA graph, where eight is the measured optimum at B = 64
+ * (0.995 ms per carve; 1.01 with sixteen, 1.03 with four).
  */
 tc_status tc_set_groups(int32_t groups);
 
